@@ -4,8 +4,10 @@
  * A collective is composed from multicast, reduction and fence primitives
  * (HiCCL, arXiv 2408.05962, Sec. 3, Listing 1), factorized for a stated
  * hierarchy into per-level point-to-point copy and sum-reduce steps with
- * striping and pipelining (Sec. 4), and executed by one persistent CUDA
- * kernel per start (Sec. 5.2).  The P ranks are virtual: each rank is a set
+ * striping and pipelining (Sec. 4), and executed by one start (Sec. 5.2): as
+ * one pass over the outputs where the program's primitives reduce to
+ * independent element-wise expressions (a sweep, see hiccl_debug_sweep), else
+ * step by step by a persistent CUDA kernel.  Both give the same bits.  The P ranks are virtual: each rank is a set
  * of disjoint buffers in one GPU's memory, so every step is a copy or a
  * reduce between device buffers; per-level byte volumes are counted, not
  * measured on links.
@@ -139,8 +141,9 @@ hiccl_status_t hiccl_add_collective(hiccl_comm_t comm, hiccl_collective_t kind, 
  *   pipeline  : m >= 1, channels per branch (Sec. 4.5).
  * Errors: HICCL_ERR_INVALID (arguments), HICCL_ERR_RACE (overlapping
  * primitives within an epoch), HICCL_ERR_NOMEM / HICCL_ERR_CUDA (device
- * memory).  Allocates the step table, dependency counters and relay buffers
- * on the current device; they are freed by hiccl_destroy. */
+ * memory).  Allocates on the current device the sweep's operand table, or the
+ * step table, dependency counters and relay buffers where the plan has no
+ * sweep; they are freed by hiccl_destroy. */
 hiccl_status_t hiccl_init(hiccl_comm_t comm, const int *hierarchy, int nlevels,
                           int stripe, int pipeline);
 
@@ -254,16 +257,18 @@ typedef struct {
   unsigned long long steps;          /* copy + reduce steps                      */
   unsigned long long copy_steps;
   unsigned long long reduce_steps;
-  unsigned long long items;          /* executor work items per start            */
+  unsigned long long items;          /* work items of the step executor          */
   unsigned long long edges;          /* dependency edges                         */
   unsigned long long stages;         /* longest dependency chain (steps)         */
-  unsigned long long scratch_bytes;  /* relay buffers on the device              */
-  unsigned long long table_bytes;    /* step table + counters on the device      */
+  unsigned long long scratch_bytes;  /* relay buffers of the step executor       */
+  unsigned long long table_bytes;    /* its step table + counters                */
   unsigned long long slots;          /* pipeline time slots of the work order    */
   unsigned long long runs;           /* contiguous data ranges the items move     */
 } hiccl_plan_info_t;
 
-/* Summary of the factorized plan.  Valid after hiccl_init or hiccl_plan. */
+/* Summary of the factorized plan.  Valid after hiccl_init or hiccl_plan.  The
+ * device bytes are those of step-by-step execution; a sweep needs no relay
+ * buffers and only its operand table. */
 hiccl_status_t hiccl_plan_info(hiccl_comm_t comm, hiccl_plan_info_t *out);
 
 /* One step of the plan, for inspection and host-side checking.
@@ -308,7 +313,10 @@ typedef enum {
   HICCL_OPT_RING = 7          /* ring(n) of Sec. 4.4: n nodes chained (default 1, tree)    */
 } hiccl_option_t;
 
-/* Set an option.  TIMEOUT_NS, CTAS_PER_SM and THREADS apply to the next start
+/* Set an option.  None changes a result bit but RING.  The options shape the
+ * step executor; a sweep heeds CTAS_PER_SM = 1 (one CTA on an SM at a time)
+ * and TRACE, which has the communicator run step by step.
+ * TIMEOUT_NS, CTAS_PER_SM and THREADS apply to the next start
  * (a start whose grid differs from the previous start's begins from zeroed
  * dependency counters; a CUDA graph that recorded a start before such a
  * change must be captured again);
@@ -353,9 +361,9 @@ hiccl_status_t hiccl_get_trace(hiccl_comm_t comm, unsigned long long *out, size_
  * first violation in hiccl_last_error; HICCL_ERR_STATE without a plan. */
 hiccl_status_t hiccl_validate(hiccl_comm_t comm);
 
-/* Inspection: the executor's table image of a planned communicator, built on
- * the host exactly as hiccl_init uploads it but with relay operands as
- * offsets into the relay arena (relay base 0).  `recs` receives the
+/* Inspection: the step executor's table image of a planned communicator,
+ * built on the host exactly as it is uploaded for step-by-step execution but
+ * with relay operands as offsets into the relay arena (relay base 0).  `recs` receives the
  * work-item records (16-byte aligned, `*recs_bytes` in all) and `items` the
  * 32-byte item descriptors in ticket order (`*nitems` of them); a record
  * holds, at 16-byte aligned offsets: nent entries {step, meta, pointer
@@ -369,6 +377,26 @@ hiccl_status_t hiccl_validate(hiccl_comm_t comm);
 hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capacity, size_t *recs_bytes,
                                  void *items, size_t items_capacity, size_t *nitems);
 
+/* Inspection: the sweep of a planned communicator -- the one pass that
+ * hiccl_start runs when the program reduces to independent expressions, each
+ * a copy or a nested fold over equal byte ranges (every collective of Table 2
+ * does; TRACE and hiccl_debug_withhold select the step-by-step executor).
+ * `out` receives, without padding: the counts of classes, launches, operand
+ * pointers and tokens (u64 each); the classes (48 bytes: bytes per operand
+ * u64, first pointer u64, then u32 first unit, units per member, members,
+ * sources, destinations, first token, meta, 0); the launches (24 bytes: u32
+ * kernel, first and end class, units, threads, saved words per thread); the
+ * pointers (u64; per member its sources in evaluation order, then its
+ * destinations); the tokens (u32, one per source: bit 0 the source starts the
+ * accumulator, bit 1 after the old one was saved, else it is combined in;
+ * then two-bit operations from bit 8 on: 1 round the accumulator to the
+ * payload, 2 combine (saved, accumulator), 3 combine (accumulator, saved)).
+ * meta: dtype 4 bits, operator 3, log2 of the access width 3, vectors per lane 4,
+ * kernel 3 (0 copies, 1 folds, 2 FP8 folds, 3 narrow accesses).  *bytes
+ * receives the size (0: the plan has no sweep); a NULL or too small `out` is
+ * left alone.  HICCL_ERR_STATE without a plan. */
+hiccl_status_t hiccl_debug_sweep(hiccl_comm_t comm, void *out, size_t capacity, size_t *bytes);
+
 /* Host-side fault injection for tests of hiccl_validate: corrupt the host
  * copy of a planned (hiccl_plan, not uploaded) table.  what = 0: make a step
  * depend on a later step (a cycle); 1: move a user-buffer operand out of its
@@ -377,7 +405,8 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
 hiccl_status_t hiccl_debug_corrupt(hiccl_comm_t comm, int what);
 
 /* Fault injection for tests: add `extra` (0 restores) phantom dependencies to
- * step `index` in the uploaded table, so that the executor's bounded wait for
+ * step `index` in the uploaded table (uploading it, and running step by step
+ * from then on, where starts ran the sweep), so that the executor's bounded wait for
  * it runs out and hiccl_wait reports HICCL_ERR_TIMEOUT.  Host-side only: it
  * changes one counter target; it never makes the GPU fault. */
 hiccl_status_t hiccl_debug_withhold(hiccl_comm_t comm, unsigned long long index, int extra);

@@ -147,9 +147,81 @@ struct DevTable {
 
 enum : uint32_t { ERR_TIMEOUT = 1, ERR_BADSTEP = 2, ERR_STALL = 3 };
 
+// ---- sweeps -------------------------------------------------------------------
+// A program whose primitives form independent expressions over equal byte
+// ranges runs as one pass over its outputs instead of step by step: a
+// *member* evaluates one expression -- a copy of one source, or the nested
+// fold of several -- element by element and stores the value to every
+// destination.  Partial sums stay in registers (rounded to the payload where
+// the schedule's steps would round them) and no relay is written or read, so
+// a pass moves each input and each output once.  Members of equal shape form
+// a class; a class is cut into warp-sized units.
+constexpr uint32_t SWEEP_MAX_DEPTH = 6;    // partial values held while an inner group is folded
+constexpr uint32_t SWEEP_PREFIX = 96;      // classes of a launch searched in the parameter bank
+
+// kernel of a launch
+enum : uint32_t {
+  SWEEP_COPY = 0,     // copies of 16-byte aligned operands
+  SWEEP_FOLD = 1,     // folds (and copies beside them), 16-byte aligned, 32-bit or BF16 values
+  SWEEP_FP8 = 2,      // folds of FP8 blocks
+  SWEEP_NARROW = 3,   // operands off a 16-byte boundary: 4- or 2-byte accesses
+  SWEEP_KERNELS = 4
+};
+
+// token of one source, in evaluation order: START the accumulator with it
+// (first saving the old one when PUSH is set), else combine it; then up to
+// 12 two-bit operations from bit 8 on, the first in the low bits
+constexpr uint32_t TOK_START = 1u, TOK_PUSH = 2u, TOK_OPS = 8u;
+enum : uint32_t {
+  TOK_ROUND = 1,   // round the accumulator to the payload
+  TOK_POP = 2,     // accumulator = combine(saved value, accumulator)
+  TOK_JOIN = 3     // accumulator = combine(accumulator, saved value)
+};
+
+struct SweepClass {
+  unsigned long long nbytes;   // bytes of every operand of a member
+  unsigned long long ptr;      // first operand pointer of member 0 (members at a stride of nsrc + ndst)
+  uint32_t unit0;              // first unit of the class within its launch
+  uint32_t upm;                // units per member
+  uint32_t nmem;
+  uint32_t nsrc, ndst;
+  uint32_t tok;                // first of the nsrc tokens
+  uint32_t meta;               // sweep_meta
+  uint32_t pad;
+};
+static_assert(sizeof(SweepClass) == 48, "class layout");
+// dtype (4 bits) | operator (3) | log2 of the access width (3) | vectors per lane (4) | kernel (3)
+HICCL_HD inline uint32_t sweep_meta(uint32_t dt, uint32_t rop, uint32_t lw, uint32_t v, uint32_t kern) {
+  return dt | (rop << 4) | (lw << 7) | (v << 10) | (kern << 14);
+}
+HICCL_HD inline uint32_t sweep_dtype(uint32_t m) { return m & 15u; }
+HICCL_HD inline uint32_t sweep_rop(uint32_t m) { return (m >> 4) & 7u; }
+HICCL_HD inline uint32_t sweep_lw(uint32_t m) { return (m >> 7) & 7u; }
+HICCL_HD inline uint32_t sweep_v(uint32_t m) { return (m >> 10) & 15u; }
+HICCL_HD inline uint32_t sweep_kernel(uint32_t m) { return (m >> 14) & 7u; }
+
+struct SweepLaunch {
+  uint32_t kernel;
+  uint32_t class_lo, class_hi;
+  uint32_t units;
+  uint32_t threads;
+  uint32_t stack_words;        // 32-bit words of saved values per thread
+};
+
 // ---------------------------------------------------------------------------
 // host-side plan
 // ---------------------------------------------------------------------------
+
+// The sweep of a plan (hiccl_sweep.cpp); valid is false where the program
+// does not reduce to independent expressions.
+struct Sweep {
+  bool valid = false;
+  std::vector<SweepClass> classes;            // grouped by launch
+  std::vector<uint32_t> toks;
+  std::vector<unsigned long long> ptrs;
+  std::vector<SweepLaunch> launches;
+  uint32_t depth = 0;                         // saved values of the deepest expression
+};
 
 struct Loc {
   unsigned long long addr;   // device address, or relay-arena offset when scratch
@@ -205,6 +277,7 @@ struct Plan {
   std::vector<unsigned long long> level_bytes;
   unsigned long long hbm_read = 0, hbm_write = 0;
   unsigned long long stages = 0, slots = 0;
+  Sweep sweep;
   bool valid = false;
 };
 
@@ -268,6 +341,10 @@ hiccl_status_t guarded(hiccl_comm *c, F &&body) noexcept {
     return st;
   }
 }
+// the sweep of c's program over `hierarchy` (ring_lvl: level of the ring's
+// nodes), and the union of several (hiccl_sweep.cpp)
+void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl, Sweep &sw);
+void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw);
 // factorize c's program again (hiccl_plan.cpp), keeping c's state
 hiccl_status_t replan(hiccl_comm *c, const std::vector<int> &hierarchy, int stripe, int pipeline);
 // runtime entry points (hiccl_runtime.cu)

@@ -1264,6 +1264,7 @@ static hiccl_status_t build_plan(hiccl_comm *c, const int *hierarchy, int nlevel
   plan.scratch_bytes = B.scratch_top;
   plan.stages = N ? maxdepth + 1 : 0;
   plan.slots = N ? maxslot + 1 : 0;
+  build_sweep(*c, h, ring_lvl, plan.sweep);
   plan.valid = true;
   {
     std::string why;
@@ -1620,6 +1621,9 @@ static hiccl_status_t group_build(const hiccl_comm_t *comms, int n, hiccl_comm *
   }
   P.entries.swap(ents);
   P.runs.swap(runs);
+  std::vector<const Sweep *> sweeps;
+  for (int i = 0; i < n; ++i) sweeps.push_back(&comms[i]->plan.sweep);
+  group_sweep(sweeps, P.sweep);
   P.valid = true;
   {
     std::string why;
@@ -1700,6 +1704,30 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t c, void *recs, size_t recs_capacit
     if (recs && recs_capacity >= im.recs.size()) std::memcpy(recs, im.recs.data(), im.recs.size());
     if (items && items_capacity >= im.items.size() * sizeof(DevItem))
       std::memcpy(items, im.items.data(), im.items.size() * sizeof(DevItem));
+    return HICCL_OK;
+  });
+}
+
+hiccl_status_t hiccl_debug_sweep(hiccl_comm_t c, void *out, size_t capacity, size_t *bytes) {
+  return guarded(c, [&]() -> hiccl_status_t {
+    if (!c || !bytes) return HICCL_ERR_INVALID;
+    *bytes = 0;
+    if (!c->plan.valid) return fail(c, HICCL_ERR_STATE, "no plan");
+    const Sweep &w = c->plan.sweep;
+    if (!w.valid) return HICCL_OK;
+    const unsigned long long n[4] = {w.classes.size(), w.launches.size(), w.ptrs.size(), w.toks.size()};
+    *bytes = sizeof(n) + n[0] * sizeof(SweepClass) + n[1] * sizeof(SweepLaunch) + n[2] * 8 + n[3] * 4;
+    if (!out || capacity < *bytes) return HICCL_OK;
+    char *q = static_cast<char *>(out);
+    auto put = [&](const void *src, size_t len) {
+      if (len) std::memcpy(q, src, len);
+      q += len;
+    };
+    put(n, sizeof(n));
+    put(w.classes.data(), n[0] * sizeof(SweepClass));
+    put(w.launches.data(), n[1] * sizeof(SweepLaunch));
+    put(w.ptrs.data(), n[2] * 8);
+    put(w.toks.data(), n[3] * 4);
     return HICCL_OK;
   });
 }

@@ -2,6 +2,10 @@
 // memoized plan (paper Sec. 5.2), the persistent sm_103a executor kernel, and
 // the non-blocking start / blocking wait of the C ABI (Sec. 3.3, Listing 2).
 //
+// A start launches the plan's sweep (hiccl_sweep.cu) where there is one.  The
+// step executor below runs every other program -- primitives that conflict
+// across a fence in more than a copy of one result -- and traced ones.
+//
 // Executor design.  One launch executes the whole step table.  Work items
 // (runs of step segments that share one pipeline slot, so that no item waits
 // on itself) are claimed in table order from a global ticket; an item only
@@ -28,7 +32,9 @@
 #include <string>
 #include <vector>
 
+#include "hiccl_device.cuh"
 #include "hiccl_internal.h"
+#include "hiccl_sweep.h"
 
 namespace hiccl {
 
@@ -52,6 +58,9 @@ struct DevState {
   int err_slot = -1;
   cudaStream_t upload = nullptr;         // internal stream of the device (not owned)
   unsigned last_grid = 0;                // grid of the previous launch (its ticket arithmetic)
+  bool sweep = false;                    // starts run the sweep; else the step executor
+  void *sweep_table = nullptr;           // its classes, tokens and operand pointers
+  std::vector<SweepArgs> sweeps;         // per launch of the plan's sweep
 };
 
 // ---------------------------------------------------------------------------
@@ -106,80 +115,6 @@ __device__ __forceinline__ T ldg_ro(const T *p) { return __ldg(p); }
 
 __device__ __forceinline__ uint4 ld16(const char *p) { return __ldcg(reinterpret_cast<const uint4 *>(p)); }
 __device__ __forceinline__ void st16(char *p, uint4 v) { *reinterpret_cast<uint4 *>(p) = v; }
-
-// one step of a fold on 32-bit lanes: f32 (IEEE RNE add, maxNum, minNum) or
-// i32 (wrapping add, max, min, logical or)
-__device__ __forceinline__ float comb_f(float a, float b, uint32_t rop) {
-  return rop == HICCL_SUM ? __fadd_rn(a, b) : rop == HICCL_MAX ? fmaxf(a, b) : fminf(a, b);
-}
-__device__ __forceinline__ uint32_t comb32(uint32_t a, uint32_t b, uint32_t dt, uint32_t rop) {
-  if (dt == HICCL_F32) return __float_as_uint(comb_f(__uint_as_float(a), __uint_as_float(b), rop));
-  const int x = (int)a, y = (int)b;
-  switch (rop) {
-    case HICCL_SUM: return a + b;
-    case HICCL_MAX: return (uint32_t)(x > y ? x : y);
-    case HICCL_MIN: return (uint32_t)(x < y ? x : y);
-    default: return (x != 0 || y != 0) ? 1u : 0u;
-  }
-}
-__device__ __forceinline__ uint4 add4(uint4 a, uint4 b, uint32_t dt, uint32_t rop = 0) {
-  if (rop == HICCL_SUM && dt == HICCL_F32) {
-    a.x = __float_as_uint(__fadd_rn(__uint_as_float(a.x), __uint_as_float(b.x)));
-    a.y = __float_as_uint(__fadd_rn(__uint_as_float(a.y), __uint_as_float(b.y)));
-    a.z = __float_as_uint(__fadd_rn(__uint_as_float(a.z), __uint_as_float(b.z)));
-    a.w = __float_as_uint(__fadd_rn(__uint_as_float(a.w), __uint_as_float(b.w)));
-  } else if (rop == HICCL_SUM) {   // int32, wrapping
-    a.x += b.x;
-    a.y += b.y;
-    a.z += b.z;
-    a.w += b.w;
-  } else {
-    a.x = comb32(a.x, b.x, dt, rop);
-    a.y = comb32(a.y, b.y, dt, rop);
-    a.z = comb32(a.z, b.z, dt, rop);
-    a.w = comb32(a.w, b.w, dt, rop);
-  }
-  return a;
-}
-
-// ---- reduced-precision payloads -------------------------------------------
-// BF16: the upper half of a binary32; rounding to nearest even by cvt.rn.
-__device__ __forceinline__ uint32_t f32_to_bf16_rn(float x) {
-  unsigned short h;
-  asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(h) : "f"(x));
-  return h;
-}
-// two binary32 -> two BF16 (round to nearest even) in one word; the first
-// value lands in the low half
-__device__ __forceinline__ uint32_t f32x2_to_bf16x2(float lo, float hi) {
-  uint32_t d;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-  return d;
-}
-// FP8 e4m3 (1 sign, 4 exponent bits with bias 7, 3 mantissa bits, no
-// infinities, S.1111.111 = NaN): four codes (byte k of w gives component k)
-// -> four binary32 values, exactly.  Every e4m3 value is a binary16 value;
-// binary16 -> binary32 is a mixed-precision add of -0 (x + -0 = x for every x,
-// signed zeros included), measured slightly faster here than cvt.f32.f16.
-__device__ __forceinline__ float4 e4m3x4_to_f32x4(uint32_t w) {
-  float4 r;
-  asm("{\n\t.reg .b16 lo, hi, a, b, c, d;\n\t.reg .b32 h0, h1;\n\t"
-      "mov.b32 {lo, hi}, %4;\n\t"
-      "cvt.rn.f16x2.e4m3x2 h0, lo;\n\tcvt.rn.f16x2.e4m3x2 h1, hi;\n\t"
-      "mov.b32 {a, b}, h0;\n\tmov.b32 {c, d}, h1;\n\t"
-      "add.rn.f32.f16 %0, a, 0f80000000;\n\tadd.rn.f32.f16 %1, b, 0f80000000;\n\t"
-      "add.rn.f32.f16 %2, c, 0f80000000;\n\tadd.rn.f32.f16 %3, d, 0f80000000;\n\t}"
-      : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
-      : "r"(w));
-  return r;
-}
-// two binary32 -> two e4m3 codes (round to nearest even, saturating at 448);
-// the first value lands in the low byte
-__device__ __forceinline__ uint32_t f32x2_to_e4m3x2(float lo, float hi) {
-  unsigned short d;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(d) : "f"(hi), "f"(lo));
-  return d;
-}
 
 // fold of one 16-byte vector position over f inputs, ld(q) giving input q's
 // vector: f32 / i32 natively (add4), BF16 decoded to binary32, folded in
@@ -1052,6 +987,7 @@ static cudaError_t device_res(int dev, DeviceRes **out) {
     cudaError_t e = cudaStreamCreateWithFlags(&r.upload, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r.nsm, cudaDevAttrMultiProcessorCount, dev);
     for (int i = 1; i < 4 && e == cudaSuccess; ++i) e = exec_occupancy(64 << i, &r.occ[i]);
+    if (e == cudaSuccess) e = sweep_prepare();
     r.status = e;
   });
   *out = &r;
@@ -1115,14 +1051,57 @@ void dev_release(hiccl_comm *c) {
     if (d->counters) cudaFreeAsync(d->counters, d->upload);
     if (d->scratch) cudaFreeAsync(d->scratch, d->upload);
     if (d->trace) cudaFreeAsync(d->trace, d->upload);
+    if (d->sweep_table) cudaFreeAsync(d->sweep_table, d->upload);
   }
   err_release(d->err_slot);
   delete d;
   c->dev = nullptr;
 }
 
+static hiccl_status_t dev_alloc(hiccl_comm *c, void **ptr, size_t bytes, const char *what) {
+  const cudaError_t e = cudaMallocAsync(ptr, bytes, c->dev->upload);
+  if (e == cudaSuccess) return HICCL_OK;
+  cudaGetLastError();
+  *ptr = nullptr;
+  return fail(c, HICCL_ERR_NOMEM, std::string(what) + ": " + cudaGetErrorString(e));
+}
+
+// the tables of the plan's sweep
+static hiccl_status_t upload_sweep(hiccl_comm *c) {
+  const Sweep &w = c->plan.sweep;
+  DevState *d = c->dev;
+  const size_t cb = w.classes.size() * sizeof(SweepClass), pb = w.ptrs.size() * 8, tb = w.toks.size() * 4;
+  std::vector<char> img(std::max<size_t>(cb + pb + tb, 16));
+  if (cb) std::memcpy(img.data(), w.classes.data(), cb);
+  if (pb) std::memcpy(img.data() + cb, w.ptrs.data(), pb);
+  if (tb) std::memcpy(img.data() + cb + pb, w.toks.data(), tb);
+  const hiccl_status_t st = dev_alloc(c, &d->sweep_table, img.size(), "sweep table");
+  if (st != HICCL_OK) return st;
+  cudaError_t e = cudaMemcpyAsync(d->sweep_table, img.data(), img.size(), cudaMemcpyHostToDevice, d->upload);
+  if (e != cudaSuccess) return cuda_fail(c, e, "upload sweep table");
+  const char *base = static_cast<const char *>(d->sweep_table);
+  d->sweeps.clear();
+  for (const SweepLaunch &L : w.launches) {
+    SweepArgs A{};
+    A.classes = reinterpret_cast<const SweepClass *>(base) + L.class_lo;
+    A.ptrs = reinterpret_cast<const unsigned long long *>(base + cb);
+    A.toks = reinterpret_cast<const uint32_t *>(base + cb + pb);
+    A.nclass = L.class_hi - L.class_lo;
+    A.units = L.units;
+    for (uint32_t k = 0; k < A.nclass && k < SWEEP_PREFIX; ++k) A.unit0[k] = w.classes[L.class_lo + k].unit0;
+    d->sweeps.push_back(A);
+  }
+  // the upload must have landed before the first start (on any stream)
+  if ((e = cudaStreamSynchronize(d->upload)) != cudaSuccess) return cuda_fail(c, e, "upload");
+  d->sweep = true;
+  return HICCL_OK;
+}
+
+static hiccl_status_t upload_steps(hiccl_comm *c);
+
+// A plan with a sweep runs it; a traced communicator runs step by step, since
+// the trace has one record per work item of the schedule.
 hiccl_status_t dev_upload(hiccl_comm *c) {
-  const Plan &p = c->plan;
   dev_release(c);
   DevState *d = new (std::nothrow) DevState();
   if (!d) return fail(c, HICCL_ERR_NOMEM, "host allocation");
@@ -1137,16 +1116,19 @@ hiccl_status_t dev_upload(hiccl_comm *c) {
     if (d->occ[i] < 1) return fail(c, HICCL_ERR_CUDA, "executor kernel cannot be resident");
   }
   d->upload = res->upload;
+  if ((e = err_slot(&d->host_err, &d->host_err_dev, &d->err_slot)) != cudaSuccess) return cuda_fail(c, e, "error word");
+  if ((e = cudaEventCreateWithFlags(&d->done_ev, cudaEventDisableTiming)) != cudaSuccess)
+    return cuda_fail(c, e, "cudaEventCreate");
+  return c->plan.sweep.valid && !c->trace ? upload_sweep(c) : upload_steps(c);
+}
+
+// the step executor's tables, counters and relay buffers
+static hiccl_status_t upload_steps(hiccl_comm *c) {
+  const Plan &p = c->plan;
+  DevState *d = c->dev;
   cudaStream_t us = d->upload;
-  auto dalloc = [&](void **ptr, size_t bytes, const char *what) -> hiccl_status_t {
-    cudaError_t ee = cudaMallocAsync(ptr, bytes, us);
-    if (ee != cudaSuccess) {
-      cudaGetLastError();
-      *ptr = nullptr;
-      return fail(c, HICCL_ERR_NOMEM, std::string(what) + ": " + cudaGetErrorString(ee));
-    }
-    return HICCL_OK;
-  };
+  cudaError_t e;
+  auto dalloc = [&](void **ptr, size_t bytes, const char *what) { return dev_alloc(c, ptr, bytes, what); };
 
   const size_t N = p.steps.size();
   unsigned long long scratch_base = 0;
@@ -1192,11 +1174,6 @@ hiccl_status_t dev_upload(hiccl_comm *c) {
   }
   if ((e = cudaMemsetAsync(d->counters, 0, d->counters_bytes, us)) != cudaSuccess)
     return cuda_fail(c, e, "cudaMemsetAsync");
-  if ((e = err_slot(&d->host_err, &d->host_err_dev, &d->err_slot)) != cudaSuccess)
-    return cuda_fail(c, e, "error word");
-  if ((e = cudaEventCreateWithFlags(&d->done_ev, cudaEventDisableTiming)) != cudaSuccess)
-    return cuda_fail(c, e, "cudaEventCreate");
-
   char *tb = static_cast<char *>(d->table);
   char *cb = static_cast<char *>(d->counters);
   DevTable &t = d->t;
@@ -1224,6 +1201,7 @@ hiccl_status_t dev_upload(hiccl_comm *c) {
   d->indeg = std::move(im.indeg);
   d->items = std::move(im.items);
   d->recs_dev = tb + o_recs;
+  d->sweep = false;
   return HICCL_OK;
 }
 
@@ -1245,7 +1223,15 @@ hiccl_status_t hiccl_start(hiccl_comm_t c, void *stream) {
     if (cap == cudaStreamCaptureStatusNone) *d->host_err = 0;
     DevTable t = d->t;
     t.timeout_ns = c->timeout_ns;
-    if (t.nitems > 0) {
+    if (d->sweep) {
+      for (size_t i = 0; i < d->sweeps.size(); ++i) {
+        const cudaError_t e = sweep_launch(c->plan.sweep.launches[i], d->sweeps[i], c->ctas_per_sm == 1, s);
+        if (e != cudaSuccess) {
+          cudaGetLastError();
+          return cuda_fail(c, e, "sweep launch");
+        }
+      }
+    } else if (t.nitems > 0) {
       const int nt = c->threads;
       const int per_sm = std::min(c->ctas_per_sm, d->occ[threads_index(nt)]);
       const unsigned long long grid = std::min<unsigned long long>(t.nitems, (unsigned long long)d->nsm * per_sm);
@@ -1404,6 +1390,12 @@ hiccl_status_t hiccl_debug_withhold(hiccl_comm_t c, unsigned long long index, in
     if (!c) return HICCL_ERR_INVALID;
     if (c->state != hiccl_comm::READY || !c->dev) return fail(c, HICCL_ERR_STATE, "needs an idle initialized communicator");
     DevState *d = c->dev;
+    if (d->sweep) {   // a sweep waits for nothing: the step executor takes over
+      if (index >= c->plan.steps.size() || extra < 0 || extra > 1000)
+        return fail(c, HICCL_ERR_INVALID, "bad step or count");
+      const hiccl_status_t st = upload_steps(c);
+      if (st != HICCL_OK) return st;
+    }
     if (index >= d->indeg.size() || extra < 0 || extra > 1000) return fail(c, HICCL_ERR_INVALID, "bad step or count");
     // the dependency count is stored in every record entry of the step
     uint32_t v[1] = {d->indeg[index] + (uint32_t)extra};

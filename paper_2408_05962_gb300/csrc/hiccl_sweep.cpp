@@ -1,0 +1,384 @@
+// Sweeps: a registered program as independent element-wise expressions
+// (host side; hiccl_sweep.cu executes them).
+//
+// The factorized schedule of a primitive moves the same byte range through
+// every step of its tree, so the value that reaches a destination is a
+// function of the sources at the same offset: a copy of the root's value, or
+// the nested fold that the hierarchy (and the ring) fixes -- independent of
+// stripe, pipeline depth and representatives.  Evaluating that expression
+// directly gives the schedule's result bit for bit and needs no relay, no
+// second read of a partial result and no signalling between steps.
+//
+// A fence is handled by substitution: a copy whose source is exactly what an
+// earlier expression stores becomes more destinations of that expression
+// (All-reduce's All-gather half).  Any other conflict across a fence leaves
+// the program to the step executor.
+
+#include <algorithm>
+#include <map>
+#include <tuple>
+
+#include "hiccl_internal.h"
+
+namespace hiccl {
+
+namespace {
+
+// ---- expressions -------------------------------------------------------------
+
+// Emits the evaluation order and tokens of one reduction: the leaves of
+// [lo, hi) of the sorted leaf list, grouped by the hierarchy.
+struct Expr {
+  const std::vector<int> &h;
+  const std::vector<int> &leaves;
+  bool rounds;                       // the payload is rounded after every fold
+  std::vector<long long> G;
+  std::vector<int> order;            // ranks in evaluation order
+  std::vector<uint32_t> toks;
+  std::vector<uint32_t> nops;
+  bool ok = true;
+
+  Expr(const std::vector<int> &hier, const std::vector<int> &lv, bool rnd) : h(hier), leaves(lv), rounds(rnd) {
+    G.assign(h.size() + 1, 1);
+    for (size_t l = h.size(); l-- > 0;) G[l] = G[l + 1] * h[l];
+  }
+  void leaf(int rank, bool start, bool push) {
+    order.push_back(rank);
+    toks.push_back((start ? TOK_START : 0u) | (push ? TOK_PUSH : 0u));
+    nops.push_back(0);
+  }
+  void op(uint32_t o) {
+    if (nops.back() >= 12) {
+      ok = false;
+      return;
+    }
+    toks.back() |= o << (TOK_OPS + 2 * nops.back()++);
+  }
+  // ends of the level-l subgroups inside leaves[lo, hi)
+  size_t next(size_t lo, size_t hi, int l) const {
+    const long long q = leaves[lo] / G[l + 1];
+    size_t k = lo + 1;
+    while (k < hi && leaves[k] / G[l + 1] == q) ++k;
+    return k;
+  }
+  // the value of a group: the left fold of its non-empty subgroups'
+  // values in ascending order; a group with one passes its value through.
+  // The accumulator is started (push: after saving it).
+  void group(size_t lo, size_t hi, int l, bool push) {
+    if (hi - lo == 1) {
+      leaf(leaves[lo], true, push);
+      return;
+    }
+    if (next(lo, hi, l) == hi) {
+      group(lo, hi, l + 1, push);
+      return;
+    }
+    parts(lo, hi, l, push);
+    if (rounds) op(TOK_ROUND);
+  }
+  // the same fold without the rounding that ends it
+  void parts(size_t lo, size_t hi, int l, bool push) {
+    for (size_t a = lo; a < hi;) {
+      const size_t z = next(a, hi, l);
+      if (a == lo) {
+        group(a, z, l + 1, push);
+      } else if (z - a == 1) {
+        leaf(leaves[a], false, false);
+      } else {
+        group(a, z, l + 1, true);
+        op(TOK_POP);
+      }
+      a = z;
+    }
+  }
+  // ring across the nodes of level lr, node a0 first: every node folds its
+  // subgroups' values and then the value coming from the next node, so the
+  // chain is evaluated from its last node back
+  void chain(int ring, int lr, long long a0) {
+    const long long N = G[lr];
+    std::vector<std::pair<size_t, size_t>> nodes;
+    for (int i = 0; i < ring; ++i) {
+      const long long a = (a0 + i) % ring;
+      const size_t lo = std::lower_bound(leaves.begin(), leaves.end(), (int)(a * N)) - leaves.begin();
+      const size_t hi = std::lower_bound(leaves.begin(), leaves.end(), (int)((a + 1) * N)) - leaves.begin();
+      if (lo < hi) nodes.emplace_back(lo, hi);
+    }
+    for (size_t k = nodes.size(); k-- > 0;) {
+      if (k + 1 == nodes.size()) {
+        group(nodes[k].first, nodes[k].second, lr, false);
+        continue;
+      }
+      if (lr == (int)h.size()) leaf(leaves[nodes[k].first], true, true);
+      else parts(nodes[k].first, nodes[k].second, lr, true);
+      op(TOK_JOIN);
+      if (rounds) op(TOK_ROUND);
+    }
+  }
+  // Drop the rounding that the store does anyway and count the saved values;
+  // false when the expression does not fit the kernels.
+  bool finish(uint32_t &depth) {
+    if (!ok) return false;
+    uint32_t &last = toks.back();
+    const uint32_t n = nops.back();
+    if (n && ((last >> (TOK_OPS + 2 * (n - 1))) & 3u) == TOK_ROUND) last &= ~(3u << (TOK_OPS + 2 * (n - 1)));
+    uint32_t sp = 0, most = 0;
+    for (uint32_t t : toks) {
+      if (t & TOK_PUSH) most = std::max(most, ++sp);
+      for (uint32_t o = t >> TOK_OPS; o; o >>= 2)
+        if ((o & 3u) >= TOK_POP) --sp;
+    }
+    depth = most;
+    return most <= SWEEP_MAX_DEPTH;
+  }
+};
+
+struct Program {   // an expression shared by members: evaluation order and tokens
+  std::vector<int> leaves;
+  long long node;  // the chain's first node (-1: tree)
+  bool rounds;
+  std::vector<int> order;
+  uint32_t tok;
+};
+
+struct Member {
+  std::vector<unsigned long long> src, dst;
+  unsigned long long nbytes;
+  uint32_t rop, tok;
+};
+
+// ---- ranges ------------------------------------------------------------------
+
+struct Touch {
+  unsigned long long lo, hi;
+  uint32_t member;
+  bool write;
+};
+
+// accesses sorted by lo with prefix maxima of hi
+struct TouchIndex {
+  std::vector<Touch> r;
+  std::vector<unsigned long long> pmax;
+  void build(const std::vector<Member> &ms, size_t n) {
+    r.clear();
+    for (size_t i = 0; i < n; ++i) {
+      for (unsigned long long a : ms[i].src) r.push_back(Touch{a, a + ms[i].nbytes, (uint32_t)i, false});
+      for (unsigned long long a : ms[i].dst) r.push_back(Touch{a, a + ms[i].nbytes, (uint32_t)i, true});
+    }
+    std::sort(r.begin(), r.end(), [](const Touch &a, const Touch &b) { return a.lo < b.lo; });
+    pmax.resize(r.size());
+    for (size_t k = 0; k < r.size(); ++k) pmax[k] = std::max(r[k].hi, k ? pmax[k - 1] : 0ull);
+  }
+  // f(touch) for every access overlapping [lo, hi) until it returns false
+  template <typename F>
+  bool each(unsigned long long lo, unsigned long long hi, F f) const {
+    size_t k = std::lower_bound(r.begin(), r.end(), hi, [](const Touch &x, unsigned long long v) { return x.lo < v; }) -
+               r.begin();
+    while (k > 0) {
+      --k;
+      if (pmax[k] <= lo) break;
+      if (r[k].hi > lo && !f(r[k])) return false;
+    }
+    return true;
+  }
+};
+
+// Width of the accesses that every operand of a member allows: 16 bytes, or
+// the widest of 4 and 2 that the addresses (and the element) share.
+uint32_t width_log2(const Member &m) {
+  unsigned long long a = 0;
+  for (unsigned long long v : m.src) a |= v;
+  for (unsigned long long v : m.dst) a |= v;
+  if (a % 16 == 0) return 4;
+  return a % 4 == 0 && m.nbytes % 4 == 0 ? 2 : 1;
+}
+
+// Launches, vectors per lane and units of a sweep's classes.
+void plan_launches(Sweep &sw) {
+  bool folds = false;
+  for (const SweepClass &k : sw.classes) folds |= k.nsrc > 1 && sweep_lw(k.meta) == 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
+  auto kernel_of = [&](const SweepClass &k) -> uint32_t {
+    if (sweep_lw(k.meta) != 4) return SWEEP_NARROW;
+    if (k.nsrc > 1 && sweep_dtype(k.meta) == HICCL_FP8E4M3) return SWEEP_FP8;
+    return k.nsrc > 1 || folds ? SWEEP_FOLD : SWEEP_COPY;
+  };
+  std::stable_sort(sw.classes.begin(), sw.classes.end(),
+                   [&](const SweepClass &a, const SweepClass &b) { return kernel_of(a) < kernel_of(b); });
+  sw.launches.clear();
+  for (size_t a = 0; a < sw.classes.size();) {
+    const uint32_t kern = kernel_of(sw.classes[a]);
+    size_t z = a;
+    unsigned long long rows = 0;   // units of one vector per lane
+    for (; z < sw.classes.size() && kernel_of(sw.classes[z]) == kern; ++z) {
+      const SweepClass &k = sw.classes[z];
+      const unsigned long long row = kern == SWEEP_FP8 ? 4 * FP8_BLOCK_BYTES : 32ull << sweep_lw(k.meta);
+      rows += (k.nbytes + row - 1) / row * k.nmem;
+    }
+    unsigned long long units = 0;
+    uint32_t words = 0;
+    for (size_t i = a; i < z; ++i) {
+      SweepClass &k = sw.classes[i];
+      const uint32_t dt = sweep_dtype(k.meta), lw = sweep_lw(k.meta);
+      uint32_t v = 1;
+      if (kern == SWEEP_COPY) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
+      else if (kern == SWEEP_FOLD) v = k.nsrc == 1 ? (rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1) : rows >= 8192 ? 2 : 1;
+      else if (kern == SWEEP_NARROW) v = rows >= 16384 ? 4 : 1;
+      const unsigned long long unit = (kern == SWEEP_FP8 ? 4 * FP8_BLOCK_BYTES : 32ull << lw) * v;
+      const unsigned long long upm = (k.nbytes + unit - 1) / unit;
+      k.meta = sweep_meta(dt, sweep_rop(k.meta), lw, v, kern);
+      k.unit0 = (uint32_t)units;
+      k.upm = (uint32_t)upm;
+      units += upm * k.nmem;
+      if (units > 0xF0000000ull) {   // far beyond device memory
+        sw.valid = false;
+        return;
+      }
+      // accumulator words of a lane: 32-bit values, or BF16 / FP8 values widened to 32 bits
+      const uint32_t acc = kern == SWEEP_FP8 ? 16 : lw == 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
+      if (k.nsrc > 1) words = std::max(words, sw.depth * acc * v);
+    }
+    SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words};
+    const uint32_t most = kern == SWEEP_COPY ? 512 : 256;
+    // a short pass uses small CTAs, so that its units reach every SM
+    uint32_t warps = most / 32;
+    while (warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
+    L.threads = warps * 32;
+    sw.launches.push_back(L);
+    a = z;
+  }
+}
+
+}  // namespace
+
+void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl, Sweep &sw) {
+  sw = Sweep();
+  if (c.epochs > 32) return;   // the range index is rebuilt per epoch
+  std::vector<Member> ms;
+  std::vector<Program> progs;
+  TouchIndex idx;
+  int epoch = 0;
+  long long node_ranks = c.P / c.ring;
+  for (const Prim &p : c.prims) {
+    if (p.count == 0) continue;
+    Member m;
+    m.nbytes = (unsigned long long)p.count * c.esize;
+    m.rop = 0;
+    m.tok = 0;
+    if (p.epoch != epoch) {
+      epoch = p.epoch;
+      idx.build(ms, ms.size());
+    }
+    if (p.kind == 0) {
+      m.src.push_back(p.send[p.root]);
+      for (int j : p.leaves)
+        if (!(j == p.root && p.recv[j] == p.send[p.root])) m.dst.push_back(p.recv[j]);
+      if (m.dst.empty()) continue;
+    } else if (p.leaves.size() == 1) {   // the operator is omitted
+      if (p.leaves[0] == p.root && p.send[p.root] == p.recv[p.root]) continue;
+      m.src.push_back(p.send[p.leaves[0]]);
+      m.dst.push_back(p.recv[p.root]);
+    } else {
+      const bool rounds = p.op == HICCL_SUM && (c.dtype == HICCL_BF16 || c.dtype == HICCL_FP8E4M3);
+      const long long node = c.ring > 1 ? p.root / node_ranks : -1;
+      const Program *pg = nullptr;
+      for (size_t k = progs.size(); k-- > 0 && !pg && k + 64 > progs.size();)
+        if (progs[k].node == node && progs[k].rounds == rounds && progs[k].leaves == p.leaves) pg = &progs[k];
+      if (!pg) {
+        Expr e(hierarchy, p.leaves, rounds);
+        if (c.ring > 1) e.chain(c.ring, ring_lvl, node);
+        else e.group(0, p.leaves.size(), 0, false);
+        uint32_t depth = 0;
+        if (!e.finish(depth)) return;
+        sw.depth = std::max(sw.depth, depth);
+        progs.push_back(Program{p.leaves, node, rounds, e.order, (uint32_t)sw.toks.size()});
+        sw.toks.insert(sw.toks.end(), e.toks.begin(), e.toks.end());
+        pg = &progs.back();
+      }
+      for (int r : pg->order) m.src.push_back(p.send[r]);
+      m.dst.push_back(p.recv[p.root]);
+      m.rop = (uint32_t)p.op;
+      m.tok = pg->tok;
+    }
+    // earlier epochs: no conflict, or a copy of exactly what one expression
+    // stores (whose sources it may overwrite in place)
+    if (p.epoch > 0) {
+      const unsigned long long n = m.nbytes;
+      uint32_t with = 0xffffffffu;
+      bool good = true, again = false;   // again: a destination that was written before
+      auto conflict = [&](const Touch &t, unsigned long long lo) {
+        if (with != 0xffffffffu && with != t.member) return good = false;
+        with = t.member;
+        return good = t.lo == lo && t.hi == lo + n;   // same bytes at the same offsets
+      };
+      for (unsigned long long a : m.src)
+        good = good && idx.each(a, a + n, [&](const Touch &t) { return !t.write || conflict(t, a); });
+      for (unsigned long long a : m.dst)
+        good = good && idx.each(a, a + n, [&](const Touch &t) {
+          again |= t.write;
+          return conflict(t, a);
+        });
+      if (!good) return;
+      if (with != 0xffffffffu) {
+        Member &x = ms[with];
+        // the copy's source has to hold the expression's value
+        const bool holds = m.src.size() == 1 && (std::find(x.dst.begin(), x.dst.end(), m.src[0]) != x.dst.end() ||
+                                                 (x.src.size() == 1 && x.src[0] == m.src[0]));
+        if (!holds) return;
+        for (unsigned long long a : m.dst)
+          if (!again || std::find(x.dst.begin(), x.dst.end(), a) == x.dst.end()) x.dst.push_back(a);
+        continue;
+      }
+    }
+    ms.push_back(std::move(m));
+  }
+
+  // classes of equal shape, in order of first appearance
+  using Key = std::tuple<unsigned long long, size_t, size_t, uint32_t, uint32_t, uint32_t>;
+  std::map<Key, uint32_t> at;
+  std::vector<std::vector<uint32_t>> members;
+  std::vector<uint32_t> widths(ms.size());
+  for (size_t i = 0; i < ms.size(); ++i) {
+    widths[i] = width_log2(ms[i]);
+    const Key k(ms[i].nbytes, ms[i].src.size(), ms[i].dst.size(), ms[i].rop, ms[i].tok, widths[i]);
+    auto it = at.emplace(k, (uint32_t)members.size()).first;
+    if (it->second == members.size()) members.emplace_back();
+    members[it->second].push_back((uint32_t)i);
+  }
+  for (const std::vector<uint32_t> &v : members) {
+    const Member &m0 = ms[v[0]];
+    SweepClass k{};
+    k.nbytes = m0.nbytes;
+    k.ptr = sw.ptrs.size();
+    k.nmem = (uint32_t)v.size();
+    k.nsrc = (uint32_t)m0.src.size();
+    k.ndst = (uint32_t)m0.dst.size();
+    k.tok = m0.tok;
+    k.meta = sweep_meta((uint32_t)c.dtype, m0.rop, widths[v[0]], 1, 0);
+    for (uint32_t i : v) {
+      sw.ptrs.insert(sw.ptrs.end(), ms[i].src.begin(), ms[i].src.end());
+      sw.ptrs.insert(sw.ptrs.end(), ms[i].dst.begin(), ms[i].dst.end());
+    }
+    sw.classes.push_back(k);
+  }
+  sw.valid = true;
+  plan_launches(sw);
+}
+
+void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw) {
+  sw = Sweep();
+  for (const Sweep *m : members)
+    if (!m->valid) return;
+  for (const Sweep *m : members) {
+    for (SweepClass k : m->classes) {
+      k.ptr += sw.ptrs.size();
+      k.tok += (uint32_t)sw.toks.size();
+      sw.classes.push_back(k);
+    }
+    sw.ptrs.insert(sw.ptrs.end(), m->ptrs.begin(), m->ptrs.end());
+    sw.toks.insert(sw.toks.end(), m->toks.begin(), m->toks.end());
+    sw.depth = std::max(sw.depth, m->depth);
+  }
+  sw.valid = true;
+  plan_launches(sw);
+}
+
+}  // namespace hiccl

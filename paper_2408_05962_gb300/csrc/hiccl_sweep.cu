@@ -1,0 +1,498 @@
+// Sweep kernels: a program's expressions evaluated in one pass over its
+// outputs (hiccl_sweep.cpp builds the classes; see there for why this equals
+// the factorized schedule).
+//
+// What bounds a pass is memory: every input is read once and every output
+// written once, with at most one add per value between.  A warp takes one
+// unit -- V vectors of 32 lanes of one member -- and loads up to eight
+// sources before it folds the first, so that 16 warps an SM hold 64 to 128
+// KiB in flight; the value goes to every destination straight from
+// registers.  Nothing waits on another CTA, so the grid is one warp per unit
+// and the hardware's CTA scheduler balances the tail: measured against a
+// persistent grid of the same code, 41.3 against 74 us for a 4 MiB Broadcast
+// to 64 ranks, 624 against 676 us for the All-reduce below; bulk (TMA) loads
+// and stores through shared-memory rings measured 48.9 and 672 us.
+//
+// Against the step executor, GB300, a start as a program times it: All-reduce
+// of 64 MiB a rank over 32 ranks 769 -> 662 us (6.49 TB/s of the inputs read
+// and outputs written once), All-reduce of 64 KiB of BF16 over 8 ranks (graph
+// replay) 22.6 -> 6.1 us, the seven collectives of 64 ranks x 4 MiB (graph
+// replay) 456 -> 312 us, an odd-length 6 MiB All-reduce over 16 ranks
+// 530 -> 70 us.
+
+#include <cuda_runtime.h>
+
+#include "hiccl_device.cuh"
+#include "hiccl_internal.h"
+#include "hiccl_sweep.h"
+
+namespace hiccl {
+
+namespace {
+
+// ---- accesses of W bytes per lane ----------------------------------------------
+
+template <int W>
+struct Raw {
+  uint32_t w[W >= 4 ? W / 4 : 1];
+};
+// (L2 only: under programmatic launch another kernel may just have written
+// these lines, and no input is read twice)
+template <int W>
+__device__ __forceinline__ Raw<W> ld_raw(unsigned long long a) {
+  Raw<W> r;
+  if constexpr (W == 16) {
+    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(a));
+    r.w[0] = v.x;
+    r.w[1] = v.y;
+    r.w[2] = v.z;
+    r.w[3] = v.w;
+  } else if constexpr (W == 4) {
+    r.w[0] = __ldcg(reinterpret_cast<const unsigned int *>(a));
+  } else {
+    r.w[0] = __ldcg(reinterpret_cast<const unsigned short *>(a));
+  }
+  return r;
+}
+template <int W>
+__device__ __forceinline__ void st_raw(unsigned long long a, const Raw<W> &r) {
+  if constexpr (W == 16) *reinterpret_cast<uint4 *>(a) = make_uint4(r.w[0], r.w[1], r.w[2], r.w[3]);
+  else if constexpr (W == 4) *reinterpret_cast<unsigned int *>(a) = r.w[0];
+  else *reinterpret_cast<unsigned short *>(a) = (unsigned short)r.w[0];
+}
+
+// ---- payload families -----------------------------------------------------------
+// N 32-bit accumulators hold the W bytes of a lane: the words themselves
+// (F32, I32), or BF16 values widened to binary32.
+
+enum Family { F32_SUM, ANY_32, BF16_SUM, BF16_ANY };
+
+template <int FAM, int W>
+struct Acc {
+  static constexpr bool BF = FAM == BF16_SUM || FAM == BF16_ANY;
+  static constexpr int N = BF ? W / 2 : W / 4;
+  uint32_t a[N];
+
+  __device__ __forceinline__ static uint32_t widen(const Raw<W> &r, int i) {
+    if constexpr (!BF) return r.w[i];
+    else return i & 1 ? r.w[i / 2] & 0xffff0000u : r.w[i / 2] << 16;
+  }
+  __device__ __forceinline__ static uint32_t comb(uint32_t x, uint32_t y, uint32_t dt, uint32_t rop) {
+    if constexpr (FAM == F32_SUM || FAM == BF16_SUM)
+      return __float_as_uint(__fadd_rn(__uint_as_float(x), __uint_as_float(y)));
+    else if constexpr (FAM == BF16_ANY)
+      return __float_as_uint(comb_f(__uint_as_float(x), __uint_as_float(y), rop));
+    else
+      return comb32(x, y, dt, rop);
+  }
+  __device__ __forceinline__ void start(const Raw<W> &r) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = widen(r, i);
+  }
+  __device__ __forceinline__ void add(const Raw<W> &r, uint32_t dt, uint32_t rop) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = comb(a[i], widen(r, i), dt, rop);
+  }
+  __device__ __forceinline__ Raw<W> pack() const {
+    Raw<W> r;
+    if constexpr (!BF) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) r.w[i] = a[i];
+    } else if constexpr (W >= 4) {
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i) r.w[i] = f32x2_to_bf16x2(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1]));
+    } else {
+      r.w[0] = f32_to_bf16_rn(__uint_as_float(a[0]));
+    }
+    return r;
+  }
+  __device__ __forceinline__ void round() {
+    if constexpr (BF) start(pack());
+  }
+};
+
+// One unit of a fold: V vectors of W bytes per lane, at byte offset `off` of
+// the lane's first vector, vectors 32 * W bytes apart, those ending past
+// `end` left out.  U sources are in flight; every source's token says how it
+// enters the accumulator (see TOK_*).  `stack` holds this thread's saved
+// values, word k at stack[k * threads].
+template <int FAM, int W, int V, int U>
+__device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__ P, const uint32_t *__restrict__ tok,
+                                          uint32_t nsrc, uint32_t ndst, unsigned long long off, unsigned long long end,
+                                          uint32_t dt, uint32_t rop, uint32_t *stack, uint32_t threads) {
+  using A = Acc<FAM, W>;
+  A acc[V];
+  bool on[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) on[v] = off + v * (32 * W) + W <= end;
+  uint32_t sp = 0;   // words saved
+  for (uint32_t q = 0; q < nsrc; q += U) {
+    Raw<W> x[U][V];
+    uint32_t t[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (q + u < nsrc) {
+        const unsigned long long s = __ldg(P + q + u) + off;
+        t[u] = __ldg(tok + q + u);
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          if (on[v]) x[u][v] = ld_raw<W>(s + v * (32 * W));
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (q + u < nsrc) {
+        if (t[u] & TOK_START) {
+          if (t[u] & TOK_PUSH) {
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+#pragma unroll
+              for (int i = 0; i < A::N; ++i) stack[(sp + v * A::N + i) * threads] = acc[v].a[i];
+            sp += V * A::N;
+          }
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc[v].start(x[u][v]);
+        } else {
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc[v].add(x[u][v], dt, rop);
+        }
+        for (uint32_t o = t[u] >> TOK_OPS; o; o >>= 2) {
+          if ((o & 3u) == TOK_ROUND) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v].round();
+          } else {
+            const bool pop = (o & 3u) == TOK_POP;
+            sp -= V * A::N;
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+#pragma unroll
+              for (int i = 0; i < A::N; ++i) {
+                const uint32_t y = stack[(sp + v * A::N + i) * threads];
+                acc[v].a[i] = pop ? A::comb(y, acc[v].a[i], dt, rop) : A::comb(acc[v].a[i], y, dt, rop);
+              }
+          }
+        }
+      }
+  }
+  Raw<W> r[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) r[v] = acc[v].pack();
+#pragma unroll 4
+  for (uint32_t d = 0; d < ndst; ++d) {
+    const unsigned long long a = __ldg(P + nsrc + d) + off;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      if (on[v]) st_raw<W>(a + v * (32 * W), r[v]);
+  }
+}
+
+template <int W, int V>
+__device__ __forceinline__ void copy_unit(const unsigned long long *__restrict__ P, uint32_t ndst,
+                                          unsigned long long off, unsigned long long end) {
+  Raw<W> r[V];
+  bool on[V];
+  const unsigned long long s = __ldg(P) + off;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    on[v] = off + v * (32 * W) + W <= end;
+    if (on[v]) r[v] = ld_raw<W>(s + v * (32 * W));
+  }
+#pragma unroll 4
+  for (uint32_t d = 0; d < ndst; ++d) {
+    const unsigned long long a = __ldg(P + 1 + d) + off;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      if (on[v]) st_raw<W>(a + v * (32 * W), r[v]);
+  }
+}
+
+// the family's fold for a class of any payload but FP8
+template <int W, int V, int U>
+__device__ __forceinline__ void fold_any(const SweepArgs &A, const SweepClass &k, const unsigned long long *P,
+                                         unsigned long long off, unsigned long long end, uint32_t *stack) {
+  const uint32_t dt = sweep_dtype(k.meta), rop = sweep_rop(k.meta), threads = blockDim.x;
+  const uint32_t *tok = A.toks + k.tok;
+  if (dt == HICCL_BF16) {
+    if (rop == HICCL_SUM) fold_unit<BF16_SUM, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
+    else fold_unit<BF16_ANY, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
+  } else if constexpr (W >= 4) {
+    if (dt == HICCL_F32 && rop == HICCL_SUM)
+      fold_unit<F32_SUM, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
+    else fold_unit<ANY_32, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
+  }
+}
+
+// ---- units -----------------------------------------------------------------------
+
+// The class and member of a unit; operand pointers at P, the unit's index
+// inside the member in `part`.
+__device__ __forceinline__ SweepClass find_class(const SweepArgs &A, uint32_t unit, const unsigned long long *&P,
+                                                 uint32_t &part) {
+  uint32_t lo = 0, hi = A.nclass;
+  while (hi - lo > 1) {   // last class whose first unit is not past `unit`
+    const uint32_t mid = (lo + hi) >> 1;
+    const uint32_t u0 = A.nclass <= SWEEP_PREFIX ? A.unit0[mid] : __ldg(&A.classes[mid].unit0);
+    if (u0 <= unit) lo = mid;
+    else hi = mid;
+  }
+  SweepClass k;
+  {
+    const uint4 *q = reinterpret_cast<const uint4 *>(A.classes + lo);
+    uint4 *z = reinterpret_cast<uint4 *>(&k);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) z[i] = __ldg(q + i);
+  }
+  const uint32_t at = unit - k.unit0, mem = at / k.upm;
+  part = at - mem * k.upm;
+  P = A.ptrs + k.ptr + (unsigned long long)mem * (k.nsrc + k.ndst);
+  return k;
+}
+
+// Launches overlap the previous kernel's tail: the next kernel's CTAs may
+// become resident once every CTA of this one has started, and touch nothing
+// before this grid has completed.
+__device__ __forceinline__ void launch_order() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <int W>
+__device__ __forceinline__ void copy_any(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
+  const uint32_t v = sweep_v(k.meta);
+  const unsigned long long off = (unsigned long long)part * (32 * W) * v + lane * W;
+  if (v == 4) copy_unit<W, 4>(P, k.ndst, off, k.nbytes);
+  else if (v == 2) copy_unit<W, 2>(P, k.ndst, off, k.nbytes);
+  else copy_unit<W, 1>(P, k.ndst, off, k.nbytes);
+}
+
+// the bytes after the last whole vector of a member, element by element
+__device__ __forceinline__ void copy_tail(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
+  if (part + 1 == k.upm && (k.nbytes & 15u))
+    copy_unit<2, 1>(P, k.ndst, (k.nbytes & ~15ull) + lane * 2, k.nbytes);
+}
+
+// copies of aligned operands: V vectors a lane in flight, stored to every
+// destination
+__global__ void __launch_bounds__(512, 2) sweep_copy_kernel(const __grid_constant__ SweepArgs A) {
+  launch_order();
+  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (unit >= A.units) return;
+  const unsigned long long *P;
+  uint32_t part;
+  const SweepClass k = find_class(A, unit, P, part);
+  copy_any<16>(k, P, part, lane);
+  copy_tail(k, P, part, lane);
+}
+
+__global__ void __launch_bounds__(256, 2) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
+  extern __shared__ uint32_t saved[];
+  launch_order();
+  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (unit >= A.units) return;
+  const unsigned long long *P;
+  uint32_t part;
+  const SweepClass k = find_class(A, unit, P, part);
+  if (k.nsrc == 1) {
+    copy_any<16>(k, P, part, lane);
+    copy_tail(k, P, part, lane);
+    return;
+  }
+  uint32_t *stack = saved + threadIdx.x;
+  const uint32_t v = sweep_v(k.meta);
+  const unsigned long long off = (unsigned long long)part * 512 * v + lane * 16;
+  if (v == 2) fold_any<16, 2, 8>(A, k, P, off, k.nbytes, stack);
+  else fold_any<16, 1, 8>(A, k, P, off, k.nbytes, stack);
+  if (part + 1 == k.upm && (k.nbytes & 15u)) {
+    const unsigned long long t0 = k.nbytes & ~15ull;
+    if (sweep_dtype(k.meta) == HICCL_BF16) fold_any<2, 1, 8>(A, k, P, t0 + lane * 2, k.nbytes, stack);
+    else fold_any<4, 1, 8>(A, k, P, t0 + lane * 4, k.nbytes, stack);
+  }
+}
+
+// operands off a 16-byte boundary: 4-byte accesses where every operand and
+// the length allow them, else 2-byte ones
+__global__ void __launch_bounds__(256, 4) sweep_narrow_kernel(const __grid_constant__ SweepArgs A) {
+  extern __shared__ uint32_t saved[];
+  launch_order();
+  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (unit >= A.units) return;
+  const unsigned long long *P;
+  uint32_t part;
+  const SweepClass k = find_class(A, unit, P, part);
+  const uint32_t v = sweep_v(k.meta);
+  if (sweep_lw(k.meta) == 2) {
+    if (k.nsrc == 1) {
+      copy_any<4>(k, P, part, lane);
+      return;
+    }
+    const unsigned long long off = (unsigned long long)part * 128 * v + lane * 4;
+    if (v == 4) fold_any<4, 4, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
+    else fold_any<4, 1, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
+  } else {
+    if (k.nsrc == 1) {
+      copy_any<2>(k, P, part, lane);
+      return;
+    }
+    const unsigned long long off = (unsigned long long)part * 64 * v + lane * 2;
+    if (v == 4) fold_any<2, 4, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
+    else fold_any<2, 1, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
+  }
+}
+
+// ---- FP8 blocks --------------------------------------------------------------------
+// A group of 8 lanes folds one 144-byte block, lane `sub` owning codes
+// 16 * sub .. 16 * sub + 15; four blocks a warp.
+
+struct Fp8Raw {
+  uint4 c;
+  float scale;
+};
+
+__device__ __forceinline__ void fp8_widen(const Fp8Raw &x, float *v) {
+  const uint32_t w[4] = {x.c.x, x.c.y, x.c.z, x.c.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float4 f = e4m3x4_to_f32x4(w[j]);
+    v[4 * j + 0] = __fmul_rn(f.x, x.scale);
+    v[4 * j + 1] = __fmul_rn(f.y, x.scale);
+    v[4 * j + 2] = __fmul_rn(f.z, x.scale);
+    v[4 * j + 3] = __fmul_rn(f.w, x.scale);
+  }
+}
+// a fresh scale amax / 448 and codes of value x (448 / amax) (both factors 1
+// when amax is 0); all lanes of the warp take part
+__device__ __forceinline__ Fp8Raw fp8_encode(const float *acc) {
+  float amax = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) amax = fmaxf(amax, fabsf(acc[i]));
+  amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+  amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
+  amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 4));
+  Fp8Raw r;
+  r.scale = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
+  const float inv = amax > 0.f ? __fdiv_rn(448.f, amax) : 1.f;
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t lo = f32x2_to_e4m3x2(__fmul_rn(acc[4 * i], inv), __fmul_rn(acc[4 * i + 1], inv));
+    const uint32_t hi = f32x2_to_e4m3x2(__fmul_rn(acc[4 * i + 2], inv), __fmul_rn(acc[4 * i + 3], inv));
+    w[i] = lo | (hi << 16);
+  }
+  r.c = make_uint4(w[0], w[1], w[2], w[3]);
+  return r;
+}
+
+__global__ void __launch_bounds__(256, 2) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
+  extern __shared__ uint32_t saved[];
+  constexpr int U = 8;
+  launch_order();
+  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (unit >= A.units) return;
+  const unsigned long long *P;
+  uint32_t part;
+  const SweepClass k = find_class(A, unit, P, part);
+  const uint32_t *tok = A.toks + k.tok;
+  const uint32_t threads = blockDim.x;
+  float *stack = reinterpret_cast<float *>(saved) + threadIdx.x;
+  const uint32_t sub = lane & 7;
+  const unsigned long long blk = (unsigned long long)part * 4 + (lane >> 3), off = blk * FP8_BLOCK_BYTES;
+  const bool on = off < k.nbytes;
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+  uint32_t sp = 0;
+  for (uint32_t q = 0; q < k.nsrc; q += U) {
+    Fp8Raw x[U];
+    uint32_t t[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (q + u < k.nsrc) {
+        const unsigned long long s = __ldg(P + q + u) + off;
+        t[u] = __ldg(tok + q + u);
+        x[u].c = make_uint4(0, 0, 0, 0);
+        x[u].scale = 0.f;
+        if (on) {
+          x[u].c = __ldcg(reinterpret_cast<const uint4 *>(s + 16 * sub));
+          x[u].scale = __ldcg(reinterpret_cast<const float *>(s + 128));
+        }
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (q + u < k.nsrc) {
+        float y[16];
+        fp8_widen(x[u], y);
+        if (t[u] & TOK_START) {
+          if (t[u] & TOK_PUSH) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) stack[(sp + i) * threads] = acc[i];
+            sp += 16;
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[i] = y[i];
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[i] = __fadd_rn(acc[i], y[i]);
+        }
+        for (uint32_t o = t[u] >> TOK_OPS; o; o >>= 2) {
+          if ((o & 3u) == TOK_ROUND) {
+            fp8_widen(fp8_encode(acc), acc);
+          } else {
+            sp -= 16;
+            const bool pop = (o & 3u) == TOK_POP;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float z = stack[(sp + i) * threads];
+              acc[i] = pop ? __fadd_rn(z, acc[i]) : __fadd_rn(acc[i], z);
+            }
+          }
+        }
+      }
+  }
+  const Fp8Raw r = fp8_encode(acc);
+  if (!on) return;
+#pragma unroll 4
+  for (uint32_t d = 0; d < k.ndst; ++d) {
+    const unsigned long long a = __ldg(P + k.nsrc + d) + off;
+    *reinterpret_cast<uint4 *>(a + 16 * sub) = r.c;
+    if (sub == 0) *reinterpret_cast<uint4 *>(a + 128) = make_uint4(__float_as_uint(r.scale), 0u, 0u, 0u);
+  }
+}
+
+typedef void (*Kernel)(const SweepArgs);
+const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel};
+
+}  // namespace
+
+// dynamic shared memory: saved values of the deepest expression a launch may
+// carry (SWEEP_MAX_DEPTH values of 16 words for each of 256 threads), or more
+// than half an SM's, which keeps a second CTA off it
+constexpr int SWEEP_HALF_SM = 120 * 1024;
+static_assert(SWEEP_MAX_DEPTH * 16 * 4 * 256 <= SWEEP_HALF_SM, "saved values fit");
+
+cudaError_t sweep_prepare() {
+  for (uint32_t i = 0; i < SWEEP_KERNELS; ++i) {
+    const cudaError_t e = cudaFuncSetAttribute(KERNELS[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_HALF_SM);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_sm, cudaStream_t s) {
+  const unsigned warps = L.threads / 32;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((L.units + warps - 1) / warps);
+  cfg.blockDim = dim3(L.threads);
+  cfg.dynamicSmemBytes = one_per_sm ? SWEEP_HALF_SM : (size_t)L.stack_words * 4 * L.threads;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, KERNELS[L.kernel], A);
+}
+
+}  // namespace hiccl

@@ -1,0 +1,23 @@
+// Launch interface of the sweep kernels (hiccl_sweep.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "hiccl_internal.h"
+
+namespace hiccl {
+
+struct SweepArgs {
+  const SweepClass *classes;            // of this launch
+  const uint32_t *toks;
+  const unsigned long long *ptrs;
+  uint32_t nclass;
+  uint32_t units;
+  uint32_t unit0[SWEEP_PREFIX];         // first units, for searching without a memory access
+};
+
+cudaError_t sweep_prepare();            // once per device, with it current
+// one_per_sm: at most one CTA on an SM (CTAS_PER_SM = 1)
+cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_sm, cudaStream_t s);
+
+}  // namespace hiccl

@@ -106,6 +106,8 @@ _SIGS = {
     "hiccl_debug_image": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t,
                                             ctypes.POINTER(ctypes.c_size_t), ctypes.c_void_p, ctypes.c_size_t,
                                             ctypes.POINTER(ctypes.c_size_t)]),
+    "hiccl_debug_sweep": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t,
+                                         ctypes.POINTER(ctypes.c_size_t)]),
     "hiccl_plan_info": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(PlanInfo)]),
     "hiccl_get_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_ulonglong, ctypes.POINTER(StepDesc),
                                       ctypes.POINTER(ctypes.c_ulonglong), ctypes.POINTER(ctypes.c_int),
@@ -265,6 +267,15 @@ def hiccl_debug_image(comm):
     return bytes(recs)[:rb.value], np.frombuffer(bytes(items), dtype=np.uint32)[:8 * ni.value].reshape(-1, 8)
 
 
+def hiccl_debug_sweep(comm) -> bytes:
+    """The sweep of a planned communicator (see the header; b"": it has none)."""
+    n = ctypes.c_size_t(0)
+    _check(comm, lib().hiccl_debug_sweep(comm, None, 0, ctypes.byref(n)))
+    buf = (ctypes.c_ubyte * max(n.value, 1))()
+    _check(comm, lib().hiccl_debug_sweep(comm, buf, n.value, ctypes.byref(n)))
+    return bytes(buf)[:n.value]
+
+
 def hiccl_get_step(comm, index: int) -> dict:
     d = StepDesc()
     _check(comm, lib().hiccl_get_step(comm, int(index), ctypes.byref(d), None, None, None, None, None,
@@ -416,6 +427,9 @@ class Comm:
 
     def image(self):
         return hiccl_debug_image(self.handle)
+
+    def sweep(self):
+        return hiccl_debug_sweep(self.handle)
 
     def step(self, i):
         return hiccl_get_step(self.handle, i)

@@ -1,0 +1,261 @@
+"""The sweep of a plan (one pass of independent expressions), decoded on the
+host and evaluated on NumPy buffers with its members in a random order, gives
+the oracle's plain semantics bit for bit -- and so the result of the step
+table, which the other tests of the factorizer compare with the same oracle."""
+import struct
+
+import numpy as np
+import pytest
+
+from oracle import programs as PR
+from oracle import semantics as S
+from oracle.hierarchy import all_factorizations
+from oracle.lowprec import from_acc, to_acc
+from oracle.model import DTYPES, Program
+from oracle.semantics import combine
+from paper_2408_05962_gb300 import build as B
+from paper_2408_05962_gb300 import hiccl as H
+from tests._bridge import FakeAddresses, register
+from tests._cases import fill, random_program
+
+START, PUSH, ROUND, POP, JOIN = 1, 2, 1, 2, 3
+COPY, FOLD, FP8, NARROW = range(4)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    B.build()
+
+
+def decode(blob):
+    """(classes, launches, pointers, tokens) of a sweep's inspection blob."""
+    nc, nl, npt, nt = struct.unpack_from("<4Q", blob, 0)
+    o = 32
+    cls = [dict(zip(("nbytes", "ptr", "unit0", "upm", "nmem", "nsrc", "ndst", "tok", "meta", "_"),
+                    struct.unpack_from("<2Q8I", blob, o + 48 * k))) for k in range(nc)]
+    o += 48 * nc
+    lau = [dict(zip(("kernel", "lo", "hi", "units", "threads", "words"), struct.unpack_from("<6I", blob, o + 24 * k)))
+           for k in range(nl)]
+    o += 24 * nl
+    ptrs = np.frombuffer(blob, np.uint64, npt, o).tolist()
+    toks = np.frombuffer(blob, np.uint32, nt, o + 8 * npt).tolist()
+    assert len(blob) == o + 8 * npt + 4 * nt
+    for c in cls:
+        m = c["meta"]
+        c.update(dtype=m & 15, rop=(m >> 4) & 7, width=1 << ((m >> 7) & 7), v=(m >> 10) & 15, kernel=(m >> 14) & 7)
+    return cls, lau, ptrs, toks
+
+
+def evaluate(vals, toks, op, dtype):
+    """One expression by its tokens, on the payload's accumulators."""
+    lp = dtype in ("bf16", "fp8")
+    wide = (lambda v: to_acc(v, dtype).copy()) if lp else (lambda v: v.copy())
+    comb = (lambda a, b: combine(a, b, op).astype(np.float32)) if lp else (lambda a, b: combine(a, b, op))
+    acc, saved, most = None, [], 0
+    for v, t in zip(vals, toks):
+        if t & START:
+            if t & PUSH:
+                saved.append(acc)
+                most = max(most, len(saved))
+            acc = wide(v)
+        else:
+            acc = comb(acc, wide(v))
+        o = t >> 8
+        while o:
+            if o & 3 == ROUND:
+                acc = wide(from_acc(acc, dtype))
+            elif o & 3 == POP:
+                acc = comb(saved.pop(), acc)
+            else:
+                acc = comb(acc, saved.pop())
+            o >>= 2
+    assert not saved
+    return (from_acc(acc, dtype) if lp else acc), most
+
+
+def run_sweep(comm, fake, mem, dtype, seed=0):
+    """Evaluate every member of the plan's sweep, in a random order; None if
+    the plan has no sweep.  Checks the launch data on the way."""
+    blob = comm.sweep()
+    if not blob:
+        return None
+    cls, lau, ptrs, toks = decode(blob)
+    views = {k: v.view(np.uint8) for k, v in mem.items()}
+    dt = DTYPES[dtype]
+
+    def view(a, n):
+        key, off = fake.resolve(a)
+        return views[key][off:off + n]
+
+    assert [x for L in lau for x in range(L["lo"], L["hi"])] == list(range(len(cls)))
+    members = []
+    for L in lau:
+        units = 0
+        for c in cls[L["lo"]:L["hi"]]:
+            assert c["kernel"] == L["kernel"] and c["unit0"] == units
+            unit = 4 * 144 if L["kernel"] == FP8 else 32 * c["width"] * c["v"]
+            assert (c["upm"] - 1) * unit < c["nbytes"] <= c["upm"] * unit        # units tile a member
+            assert c["v"] in (1, 2, 4)
+            units += c["upm"] * c["nmem"]
+            for i in range(c["nmem"]):
+                p = ptrs[c["ptr"] + i * (c["nsrc"] + c["ndst"]):][:c["nsrc"] + c["ndst"]]
+                assert all(a % c["width"] == 0 for a in p) and (L["kernel"] == NARROW) == (c["width"] < 16)
+                assert (c["nsrc"] > 1) or L["kernel"] != FP8
+                members.append((c, p))
+        assert L["units"] == units and L["threads"] in (32, 64, 128, 256, 512)
+    rng = np.random.Generator(np.random.PCG64(seed))
+    for k in rng.permutation(len(members)):
+        c, p = members[k]
+        vals = [view(a, c["nbytes"]).copy().view(dt) for a in p[:c["nsrc"]]]
+        out = vals[0]
+        if c["nsrc"] > 1:
+            out, most = evaluate(vals, toks[c["tok"]:c["tok"] + c["nsrc"]], H.OP_NAMES[c["rop"]], dtype)
+            acc = 16 if dtype == "fp8" else (c["width"] // 2 if dtype == "bf16" else c["width"] // 4)
+            L = next(x for x in lau if x["kernel"] == c["kernel"])
+            assert most * max(acc, 1) * c["v"] <= L["words"]                     # saved values fit
+        for a in p[c["nsrc"]:]:
+            view(a, c["nbytes"])[...] = out.view(np.uint8)
+    return mem
+
+
+def check(prog, h, s, m, seed=0, ring=1, zero_frac=0.0, fake=None):
+    fake = fake or FakeAddresses(prog)
+    comm = register(prog, fake.addr)
+    if ring > 1:
+        comm.set_option(H.OPT_RING, ring)
+    comm.plan(h, s, m)
+    mem0 = fill(prog, seed, zero_frac)
+    ref = {k: v.copy() for k, v in mem0.items()}
+    S.run_program(prog, ref, h, ring)
+    got = run_sweep(comm, fake, {k: v.copy() for k, v in mem0.items()}, prog.dtype, seed)
+    if got is not None:
+        for k in ref:
+            assert np.array_equal(ref[k].view(np.uint8), got[k].view(np.uint8)), k
+    return got is not None
+
+
+TABLE2 = PR.SEVEN + ("reduce", "allreduce_single", "allreduce_bcast_reduce", "reduce_gather_rs", "broadcast_ag_scatter")
+
+
+@pytest.mark.parametrize("name", TABLE2)
+@pytest.mark.parametrize("dtype", ["f32", "i32", "bf16", "fp8"])
+@pytest.mark.parametrize("P,h,s,m,ring", [(8, [2, 4], 1, 1, 1), (12, [2, 2, 3], 3, 2, 1), (16, [16], 2, 3, 1),
+                                          (12, [4, 3], 3, 2, 4), (8, [2, 2, 2], 1, 2, 8), (12, [2, 2, 3], 2, 1, 4)])
+def test_collectives_have_sweeps_equal_to_the_oracle(name, dtype, P, h, s, m, ring):
+    assert check(PR.BUILDERS[name](P, 3 if dtype == "fp8" else 37, dtype=dtype), h, s, m, seed=P + s, ring=ring)
+
+
+@pytest.mark.parametrize("op,dtype", [(o, d) for o in ("max", "min") for d in ("f32", "i32", "bf16")] + [("lor", "i32")])
+def test_operators(op, dtype):
+    for name in ("allreduce", "reducescatter"):
+        assert check(PR.BUILDERS[name](12, 29, dtype=dtype, op=op), [2, 2, 3], 3, 2, seed=5, zero_frac=0.25)
+
+
+def test_random_programs_and_hierarchies():
+    """Random leaf sets, roots and fences over every hierarchy: a sweep, where
+    the plan has one, equals the oracle; both outcomes occur."""
+    seen = set()
+    for P in (2, 3, 4, 6, 8, 12):
+        for h in all_factorizations(P):
+            for seed in range(4):
+                prog = random_program(P, P * 100 + seed + len(h), ("f32", "i32", "bf16")[seed % 3])
+                if S.find_race(prog) is None:
+                    seen.add(check(prog, h, 1 + seed % P, 1 + seed % 2, seed=seed))
+    assert seen == {True, False}
+
+
+@pytest.mark.parametrize("dtype,shift", [("f32", 1), ("f32", 4), ("bf16", 1), ("bf16", 2), ("bf16", 8)])
+def test_operands_off_a_vector_boundary(dtype, shift):
+    """Every buffer `shift` elements off its boundary, odd chunk lengths: the
+    accesses are as wide as all operands of a member allow."""
+    for name in ("allreduce", "alltoall", "broadcast"):
+        prog = PR.BUILDERS[name](8, 131, dtype=dtype)
+        fake = FakeAddresses(prog)
+        fake.base = {k: a + shift * DTYPES[dtype].itemsize for k, a in fake.base.items()}
+        assert check(prog, [2, 4], 2, 2, seed=shift, fake=fake)
+
+
+def two_epochs(build):
+    """A 4-rank program over buffers a and b of 64 values per rank."""
+    prog = Program(4)
+    a = [prog.buffer(("send", r), 64) for r in range(4)]
+    b = [prog.buffer(("recv", r), 64) for r in range(4)]
+    build(prog, a, b)
+    return prog
+
+
+def test_in_place_allreduce_is_one_sweep():
+    """Listing 2 with receive buffers equal to the send buffers: the gathered
+    chunk overwrites sources of its own expression at the same offsets."""
+    P, d = 8, 48
+    base = [0x7f0000000000 + r * 0x10000 for r in range(P)]
+    c = H.Comm(P, "f32")
+    c.add_collective("allreduce", d, base, base)
+    c.plan([2, 4], 2, 2)
+    cls, _, ptrs, _ = decode(c.sweep())
+    assert sum(k["nmem"] for k in cls) == P
+    for k in cls:
+        for i in range(k["nmem"]):
+            p = ptrs[k["ptr"] + i * (k["nsrc"] + k["ndst"]):][:k["nsrc"] + k["ndst"]]
+            assert k["nsrc"] == P and sorted(p[:P]) == sorted(p[P:])
+
+
+def _all(r):
+    return {j: r[j] for j in range(4)}
+
+
+@pytest.mark.parametrize("case", ["sum_of_sums", "overwritten_source", "part", "other_offset", "two_values"])
+def test_other_conflicts_across_a_fence_stay_with_the_steps(case):
+    """A program whose later epoch is not a copy of one expression has no sweep."""
+    def build(prog, a, b):
+        prog.reduction([0, 1, 2, 3], 0, 32, _all(a), b[0])
+        if case == "two_values":
+            prog.multicast(1, [0], 32, a[1], {0: b[0].shift(32)})
+        prog.fence()
+        if case == "sum_of_sums":
+            prog.reduction([0, 1], 2, 32, {0: b[0], 1: a[1]}, b[2])
+        elif case == "overwritten_source":
+            prog.multicast(3, [2], 32, a[3].shift(32), {2: a[2]})
+        elif case == "part":
+            prog.multicast(0, [2], 16, b[0].shift(8), {2: b[2]})
+        elif case == "other_offset":
+            prog.multicast(0, [2], 32, b[0], {2: a[2].shift(16)})
+        else:
+            prog.multicast(0, [2], 64, b[0], {2: b[2]})
+    prog = two_epochs(build)
+    assert S.find_race(prog) is None
+    assert not check(prog, [2, 2], 1, 1)
+
+
+def test_a_repeated_copy_and_a_disjoint_one_are_swept():
+    def build(prog, a, b):
+        prog.multicast(0, [1, 2], 32, a[0], {1: b[1], 2: b[2]})
+        prog.fence()
+        prog.multicast(1, [2, 3], 32, b[1], {2: b[2], 3: b[3]})       # b[2] again, with the same value
+        prog.multicast(3, [0], 32, a[3], {0: b[0].shift(32)})         # touches nothing of the first epoch
+    assert check(two_epochs(build), [2, 2], 1, 1)
+
+
+def test_deep_hierarchies_fall_back():
+    """Eight levels of two need seven saved values, more than the kernels hold."""
+    assert check(PR.reduce(64, 8), [2] * 6, 1, 1)
+    assert not check(PR.reduce(256, 4), [2] * 8, 1, 1)
+
+
+def test_group_sweep_is_the_union():
+    shapes = [("allreduce", [4, 4], 2, 3, "f32"), ("allgather", [2, 8], 4, 2, "bf16"), ("reducescatter", [16], 1, 1, "bf16")]
+    members, total = [], 0
+    base = 0x7f0000000000
+    for name, h, s, m, dt in shapes:
+        prog = PR.BUILDERS[name](16, 40, dtype=dt)
+        fake = FakeAddresses(prog, base=base)
+        base = (fake.end + (1 << 20)) & ~255
+        c = register(prog, fake.addr)
+        c.plan(h, s, m)
+        members.append(c)
+        total += sum(k["nmem"] for k in decode(c.sweep())[0])
+    g = H.Comm.group_plan(members)
+    cls, lau, ptrs, _ = decode(g.sweep())
+    assert sum(k["nmem"] for k in cls) == total
+    assert sorted(ptrs) == sorted(p for c in members for p in decode(c.sweep())[2])
+    assert len(lau) == 1 and lau[0]["kernel"] == FOLD
