@@ -237,7 +237,7 @@ void plan_launches(Sweep &sw) {
       if (k.nsrc > 1) words = std::max(words, sw.depth * acc * v);
     }
     SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words};
-    const uint32_t most = kern == SWEEP_COPY ? 512 : 256;
+    const uint32_t most = kern == SWEEP_COPY ? 512 : kern == SWEEP_FP8 ? 128 : 256;
     // a short pass uses small CTAs, so that its units reach every SM
     uint32_t warps = most / 32;
     while (warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;

@@ -350,20 +350,46 @@ struct Fp8Raw {
   float scale;
 };
 
-__device__ __forceinline__ void fp8_widen(const Fp8Raw &x, float *v) {
+// two binary32 values in one 64-bit register pair
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpack2(unsigned long long d, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(d));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// rounded products: fma with -0, which a kernel argument supplies so that the
+// product is not contracted into the add that follows it
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b,
+                                                   unsigned long long minus0) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(minus0));
+  return d;
+}
+
+// the 16 values of a lane, code x scale
+__device__ __forceinline__ void fp8_widen(const Fp8Raw &x, unsigned long long minus0, unsigned long long *v) {
   const uint32_t w[4] = {x.c.x, x.c.y, x.c.z, x.c.w};
+  const unsigned long long s = pack2(x.scale, x.scale);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float4 f = e4m3x4_to_f32x4(w[j]);
-    v[4 * j + 0] = __fmul_rn(f.x, x.scale);
-    v[4 * j + 1] = __fmul_rn(f.y, x.scale);
-    v[4 * j + 2] = __fmul_rn(f.z, x.scale);
-    v[4 * j + 3] = __fmul_rn(f.w, x.scale);
+    v[2 * j] = mul2(pack2(f.x, f.y), s, minus0);
+    v[2 * j + 1] = mul2(pack2(f.z, f.w), s, minus0);
   }
 }
 // a fresh scale amax / 448 and codes of value x (448 / amax) (both factors 1
 // when amax is 0); all lanes of the warp take part
-__device__ __forceinline__ Fp8Raw fp8_encode(const float *acc) {
+__device__ __forceinline__ Fp8Raw fp8_encode(const unsigned long long *v) {
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) unpack2(v[i], acc[2 * i], acc[2 * i + 1]);
   float amax = 0.f;
 #pragma unroll
   for (int i = 0; i < 16; ++i) amax = fmaxf(amax, fabsf(acc[i]));
@@ -384,9 +410,32 @@ __device__ __forceinline__ Fp8Raw fp8_encode(const float *acc) {
   return r;
 }
 
-__global__ void __launch_bounds__(256, 2) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
-  extern __shared__ uint32_t saved[];
-  constexpr int U = 8;
+constexpr int FP8_SLOTS = 8;                                    // sources a warp keeps in flight
+constexpr uint32_t FP8_STEP = 4 * FP8_BLOCK_BYTES;              // bytes of a source in one slot
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, unsigned long long src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// A unit is four blocks, 576 bytes of every operand.  A source takes about 100
+// instructions, so a warp is busy while its loads should fly; they
+// pass through a ring of slots in shared memory, one asynchronous copy group
+// a source, which keeps FP8_SLOTS - 1 in flight through folds, encodings and
+// stores without holding registers (72 a thread, 24 warps an SM).  Copies and
+// stores move the unit as one range of whole sectors, and only the fold reads
+// it by blocks.  All-reduce of 2 Mi values a rank over 32 ranks ({4, 8}),
+// 1.21 GB in and out: 265 us with the next sources loaded into registers (16
+// warps an SM; 403 us when refilled one by one), 223 us through the ring by
+// blocks, 199 us by the unit's range, 6.1 TB/s; two or four units a warp
+// lose 5 and 10 %, neighbouring warps on neighbouring units read longer
+// stretches of each source at a time.
+__global__ void __launch_bounds__(128, 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
+  extern __shared__ __align__(16) uint32_t saved[];
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -395,69 +444,94 @@ __global__ void __launch_bounds__(256, 2) sweep_fp8_kernel(const __grid_constant
   uint32_t part;
   const SweepClass k = find_class(A, unit, P, part);
   const uint32_t *tok = A.toks + k.tok;
-  const uint32_t threads = blockDim.x;
-  float *stack = reinterpret_cast<float *>(saved) + threadIdx.x;
-  const uint32_t sub = lane & 7;
-  const unsigned long long blk = (unsigned long long)part * 4 + (lane >> 3), off = blk * FP8_BLOCK_BYTES;
-  const bool on = off < k.nbytes;
-  float acc[16];
+  const uint32_t threads = blockDim.x, sub = lane & 7;
+  const unsigned long long minus0 = A.minus0;
+  char *ring = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (FP8_SLOTS * FP8_STEP);
+  char *mine = ring + (lane >> 3) * FP8_BLOCK_BYTES;   // this group's block in slot 0
+  const uint32_t ring_at = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + 16 * lane;
+  float *stack = reinterpret_cast<float *>(saved) + (threads >> 5) * (FP8_SLOTS * FP8_STEP / 4) + threadIdx.x;
+
+  // this lane's 16 bytes of the unit, and (lanes 0 .. 3) 16 of its last 64
+  const unsigned long long off = (unsigned long long)part * FP8_STEP + 16 * lane;
+  const bool on = off < k.nbytes, on2 = lane < 4 && off + 512 < k.nbytes;
+  unsigned long long lptr = __ldg(P);   // of source lq
+  uint32_t lq = 0;
+  auto load = [&](int slot) {
+    if (lq < k.nsrc) {
+      const unsigned long long s = lptr + off;
+      if (on) cp_async16(ring_at + slot * FP8_STEP, s);
+      if (on2) cp_async16(ring_at + slot * FP8_STEP + 512, s + 512);
+      if (++lq < k.nsrc) lptr = __ldg(P + lq);
+    }
+    cp_commit();
+  };
 #pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-  uint32_t sp = 0;
-  for (uint32_t q = 0; q < k.nsrc; q += U) {
-    Fp8Raw x[U];
-    uint32_t t[U];
+  for (int u = 0; u < FP8_SLOTS - 1; ++u) load(u);
+  unsigned long long acc[8];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (q + u < k.nsrc) {
-        const unsigned long long s = __ldg(P + q + u) + off;
-        t[u] = __ldg(tok + q + u);
-        x[u].c = make_uint4(0, 0, 0, 0);
-        x[u].scale = 0.f;
-        if (on) {
-          x[u].c = __ldcg(reinterpret_cast<const uint4 *>(s + 16 * sub));
-          x[u].scale = __ldcg(reinterpret_cast<const float *>(s + 128));
+  for (int i = 0; i < 8; ++i) acc[i] = 0ull;
+  uint32_t sp = 0, nz = 0;   // words saved; which of 32 tokens do more than combine
+  uint32_t slot = 0;
+  for (uint32_t q = 0; q < k.nsrc; ++q) {
+    if ((q & 31u) == 0) nz = __ballot_sync(0xffffffffu, q + lane < k.nsrc && __ldg(tok + q + lane) != 0u);
+    cp_wait<FP8_SLOTS - 2>();
+    __syncwarp();              // every lane's copies have landed, and the slot read last is free
+    load((slot + FP8_SLOTS - 1) % FP8_SLOTS);
+    Fp8Raw x;
+    x.c = *reinterpret_cast<const uint4 *>(mine + slot * FP8_STEP + 16 * sub);
+    x.scale = *reinterpret_cast<const float *>(mine + slot * FP8_STEP + 128);
+    slot = (slot + 1) % FP8_SLOTS;
+    unsigned long long y[8];
+    fp8_widen(x, minus0, y);
+    if (!((nz >> (q & 31u)) & 1u)) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] = add2(acc[i], y[i]);
+      continue;
+    }
+    const uint32_t tk = __ldg(tok + q);
+    if (tk & TOK_START) {
+      if (tk & TOK_PUSH) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float lo, hi;
+          unpack2(acc[i], lo, hi);
+          stack[(sp + 2 * i) * threads] = lo;
+          stack[(sp + 2 * i + 1) * threads] = hi;
         }
+        sp += 16;
       }
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (q + u < k.nsrc) {
-        float y[16];
-        fp8_widen(x[u], y);
-        if (t[u] & TOK_START) {
-          if (t[u] & TOK_PUSH) {
+      for (int i = 0; i < 8; ++i) acc[i] = y[i];
+    } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) stack[(sp + i) * threads] = acc[i];
-            sp += 16;
-          }
+      for (int i = 0; i < 8; ++i) acc[i] = add2(acc[i], y[i]);
+    }
+    for (uint32_t o = tk >> TOK_OPS; o; o >>= 2) {
+      if ((o & 3u) == TOK_ROUND) {
+        fp8_widen(fp8_encode(acc), minus0, acc);
+      } else {
+        sp -= 16;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) acc[i] = y[i];
-        } else {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) acc[i] = __fadd_rn(acc[i], y[i]);
-        }
-        for (uint32_t o = t[u] >> TOK_OPS; o; o >>= 2) {
-          if ((o & 3u) == TOK_ROUND) {
-            fp8_widen(fp8_encode(acc), acc);
-          } else {
-            sp -= 16;
-            const bool pop = (o & 3u) == TOK_POP;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float z = stack[(sp + i) * threads];
-              acc[i] = pop ? __fadd_rn(z, acc[i]) : __fadd_rn(acc[i], z);
-            }
-          }
+        for (int i = 0; i < 8; ++i) {   // (a sum of two is the same in both orders)
+          const float lo = stack[(sp + 2 * i) * threads], hi = stack[(sp + 2 * i + 1) * threads];
+          acc[i] = add2(pack2(lo, hi), acc[i]);
         }
       }
+    }
   }
   const Fp8Raw r = fp8_encode(acc);
-  if (!on) return;
+  cp_wait<0>();
+  __syncwarp();   // the ring is free: the result takes slot 0
+  *reinterpret_cast<uint4 *>(mine + 16 * sub) = r.c;
+  if (sub == 0) *reinterpret_cast<uint4 *>(mine + 128) = make_uint4(__float_as_uint(r.scale), 0u, 0u, 0u);
+  __syncwarp();
+  const uint4 v = *reinterpret_cast<const uint4 *>(ring + 16 * lane);
+  const uint4 v2 = *reinterpret_cast<const uint4 *>(ring + 512 + 16 * (lane & 3));
 #pragma unroll 4
   for (uint32_t d = 0; d < k.ndst; ++d) {
     const unsigned long long a = __ldg(P + k.nsrc + d) + off;
-    *reinterpret_cast<uint4 *>(a + 16 * sub) = r.c;
-    if (sub == 0) *reinterpret_cast<uint4 *>(a + 128) = make_uint4(__float_as_uint(r.scale), 0u, 0u, 0u);
+    if (on) *reinterpret_cast<uint4 *>(a) = v;
+    if (on2) *reinterpret_cast<uint4 *>(a + 512) = v2;
   }
 }
 
@@ -466,15 +540,14 @@ const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, swe
 
 }  // namespace
 
-// dynamic shared memory: saved values of the deepest expression a launch may
-// carry (SWEEP_MAX_DEPTH values of 16 words for each of 256 threads), or more
-// than half an SM's, which keeps a second CTA off it
-constexpr int SWEEP_HALF_SM = 120 * 1024;
-static_assert(SWEEP_MAX_DEPTH * 16 * 4 * 256 <= SWEEP_HALF_SM, "saved values fit");
+// dynamic shared memory: at most SWEEP_MAX_DEPTH values of 16 words for each
+// of 128 threads and four rings, or of 16 words for 256; more than half an SM's keeps a second CTA
+// off it
+constexpr size_t SWEEP_MAX_SMEM = SWEEP_MAX_DEPTH * 16 * 4 * 256 + 8 * FP8_SLOTS * FP8_STEP, SWEEP_HALF_SM = 120 * 1024;
 
 cudaError_t sweep_prepare() {
   for (uint32_t i = 0; i < SWEEP_KERNELS; ++i) {
-    const cudaError_t e = cudaFuncSetAttribute(KERNELS[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_HALF_SM);
+    const cudaError_t e = cudaFuncSetAttribute(KERNELS[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_MAX_SMEM);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -485,7 +558,9 @@ cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((L.units + warps - 1) / warps);
   cfg.blockDim = dim3(L.threads);
-  cfg.dynamicSmemBytes = one_per_sm ? SWEEP_HALF_SM : (size_t)L.stack_words * 4 * L.threads;
+  cfg.dynamicSmemBytes = (size_t)L.stack_words * 4 * L.threads;
+  if (L.kernel == SWEEP_FP8) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;
+  if (one_per_sm && cfg.dynamicSmemBytes < SWEEP_HALF_SM) cfg.dynamicSmemBytes = SWEEP_HALF_SM;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

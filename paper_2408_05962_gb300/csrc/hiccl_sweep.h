@@ -13,6 +13,7 @@ struct SweepArgs {
   const unsigned long long *ptrs;
   uint32_t nclass;
   uint32_t units;
+  unsigned long long minus0 = 0x8000000080000000ull;   // two binary32 -0 (see mul2)
   uint32_t unit0[SWEEP_PREFIX];         // first units, for searching without a memory access
 };
 

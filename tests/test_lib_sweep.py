@@ -93,7 +93,7 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         units = 0
         for c in cls[L["lo"]:L["hi"]]:
             assert c["kernel"] == L["kernel"] and c["unit0"] == units
-            unit = 4 * 144 if L["kernel"] == FP8 else 32 * c["width"] * c["v"]
+            unit = (4 * 144 if L["kernel"] == FP8 else 32 * c["width"]) * c["v"]
             assert (c["upm"] - 1) * unit < c["nbytes"] <= c["upm"] * unit        # units tile a member
             assert c["v"] in (1, 2, 4)
             units += c["upm"] * c["nmem"]
@@ -112,7 +112,7 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
             out, most = evaluate(vals, toks[c["tok"]:c["tok"] + c["nsrc"]], H.OP_NAMES[c["rop"]], dtype)
             acc = 16 if dtype == "fp8" else (c["width"] // 2 if dtype == "bf16" else c["width"] // 4)
             L = next(x for x in lau if x["kernel"] == c["kernel"])
-            assert most * max(acc, 1) * c["v"] <= L["words"]                     # saved values fit
+            assert most * max(acc, 1) * c["v"] <= L["words"]   # saved values fit
         for a in p[c["nsrc"]:]:
             view(a, c["nbytes"])[...] = out.view(np.uint8)
     return mem
