@@ -391,8 +391,9 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
  * accumulator, bit 1 after the old one was saved, else it is combined in;
  * then two-bit operations from bit 8 on: 1 round the accumulator to the
  * payload, 2 combine (saved, accumulator), 3 combine (accumulator, saved)).
- * meta: dtype 4 bits, operator 3, log2 of the access width 3, vectors per lane 4,
- * kernel 3 (0 copies, 1 folds, 2 FP8 folds, 3 narrow accesses).  *bytes
+ * meta: dtype 4 bits, operator 3, log2 of the access width 3, vectors per lane 5,
+ * kernel 3 (0 copies, 1 folds, 2 FP8 folds; operands
+ * that lie differently off a 16-byte boundary: 3 folds, 4 copies).  *bytes
  * receives the size (0: the plan has no sweep); a NULL or too small `out` is
  * left alone.  HICCL_ERR_STATE without a plan. */
 hiccl_status_t hiccl_debug_sweep(hiccl_comm_t comm, void *out, size_t capacity, size_t *bytes);

@@ -161,12 +161,14 @@ constexpr uint32_t SWEEP_PREFIX = 96;      // classes of a launch searched in th
 
 // kernel of a launch
 enum : uint32_t {
-  SWEEP_COPY = 0,     // copies of 16-byte aligned operands
-  SWEEP_FOLD = 1,     // folds (and copies beside them), 16-byte aligned, 32-bit or BF16 values
+  SWEEP_COPY = 0,     // copies whose operands lie equally far off a 16-byte boundary
+  SWEEP_FOLD = 1,     // folds of such operands (and copies beside them), 32-bit or BF16 values
   SWEEP_FP8 = 2,      // folds of FP8 blocks
-  SWEEP_NARROW = 3,   // operands off a 16-byte boundary: 4- or 2-byte accesses
-  SWEEP_KERNELS = 4
+  SWEEP_NARROW = 3,   // folds of other operands: 4- or 2-byte accesses
+  SWEEP_SHIFT = 4,    // copies of other operands: vectors shifted in registers
+  SWEEP_KERNELS = 5
 };
+constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128};   // most threads of a CTA
 
 // token of one source, in evaluation order: START the accumulator with it
 // (first saving the old one when PUSH is set), else combine it; then up to
@@ -190,15 +192,15 @@ struct SweepClass {
   uint32_t pad;
 };
 static_assert(sizeof(SweepClass) == 48, "class layout");
-// dtype (4 bits) | operator (3) | log2 of the access width (3) | vectors per lane (4) | kernel (3)
+// dtype (4 bits) | operator (3) | log2 of the access width (3) | vectors per lane (5) | kernel (3)
 HICCL_HD inline uint32_t sweep_meta(uint32_t dt, uint32_t rop, uint32_t lw, uint32_t v, uint32_t kern) {
-  return dt | (rop << 4) | (lw << 7) | (v << 10) | (kern << 14);
+  return dt | (rop << 4) | (lw << 7) | (v << 10) | (kern << 15);
 }
 HICCL_HD inline uint32_t sweep_dtype(uint32_t m) { return m & 15u; }
 HICCL_HD inline uint32_t sweep_rop(uint32_t m) { return (m >> 4) & 7u; }
 HICCL_HD inline uint32_t sweep_lw(uint32_t m) { return (m >> 7) & 7u; }
-HICCL_HD inline uint32_t sweep_v(uint32_t m) { return (m >> 10) & 15u; }
-HICCL_HD inline uint32_t sweep_kernel(uint32_t m) { return (m >> 14) & 7u; }
+HICCL_HD inline uint32_t sweep_v(uint32_t m) { return (m >> 10) & 31u; }
+HICCL_HD inline uint32_t sweep_kernel(uint32_t m) { return (m >> 15) & 7u; }
 
 struct SweepLaunch {
   uint32_t kernel;

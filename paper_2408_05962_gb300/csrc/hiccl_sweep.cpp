@@ -182,14 +182,22 @@ struct TouchIndex {
   }
 };
 
-// Width of the accesses that every operand of a member allows: 16 bytes, or
-// the widest of 4 and 2 that the addresses (and the element) share.
+// Width of the accesses that every operand of a member allows: 16 bytes when
+// all lie equally far off a 16-byte boundary (whole vectors between a few
+// elements at both ends), else the widest of 4 and 2 that the addresses (and
+// the length) share.
 uint32_t width_log2(const Member &m) {
-  unsigned long long a = 0;
-  for (unsigned long long v : m.src) a |= v;
-  for (unsigned long long v : m.dst) a |= v;
-  if (a % 16 == 0) return 4;
+  unsigned long long a = 0, off = 0;
+  for (unsigned long long v : m.src) a |= v, off |= v ^ m.src[0];
+  for (unsigned long long v : m.dst) a |= v, off |= v ^ m.src[0];
+  if (off % 16 == 0) return 4;
   return a % 4 == 0 && m.nbytes % 4 == 0 ? 2 : 1;
+}
+
+// bytes of a member that a warp moves with one vector per lane
+unsigned long long row_bytes(uint32_t kern, const SweepClass &k) {
+  if (kern == SWEEP_FP8) return 4 * FP8_BLOCK_BYTES;
+  return kern == SWEEP_SHIFT ? 31 * 16 : 32ull << sweep_lw(k.meta);
 }
 
 // Launches, vectors per lane and units of a sweep's classes.
@@ -197,7 +205,7 @@ void plan_launches(Sweep &sw) {
   bool folds = false;
   for (const SweepClass &k : sw.classes) folds |= k.nsrc > 1 && sweep_lw(k.meta) == 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
   auto kernel_of = [&](const SweepClass &k) -> uint32_t {
-    if (sweep_lw(k.meta) != 4) return SWEEP_NARROW;
+    if (sweep_lw(k.meta) != 4) return k.nsrc > 1 ? SWEEP_NARROW : SWEEP_SHIFT;
     if (k.nsrc > 1 && sweep_dtype(k.meta) == HICCL_FP8E4M3) return SWEEP_FP8;
     return k.nsrc > 1 || folds ? SWEEP_FOLD : SWEEP_COPY;
   };
@@ -210,7 +218,7 @@ void plan_launches(Sweep &sw) {
     unsigned long long rows = 0;   // units of one vector per lane
     for (; z < sw.classes.size() && kernel_of(sw.classes[z]) == kern; ++z) {
       const SweepClass &k = sw.classes[z];
-      const unsigned long long row = kern == SWEEP_FP8 ? 4 * FP8_BLOCK_BYTES : 32ull << sweep_lw(k.meta);
+      const unsigned long long row = row_bytes(kern, k);
       rows += (k.nbytes + row - 1) / row * k.nmem;
     }
     unsigned long long units = 0;
@@ -219,10 +227,11 @@ void plan_launches(Sweep &sw) {
       SweepClass &k = sw.classes[i];
       const uint32_t dt = sweep_dtype(k.meta), lw = sweep_lw(k.meta);
       uint32_t v = 1;
-      if (kern == SWEEP_COPY) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
-      else if (kern == SWEEP_FOLD) v = k.nsrc == 1 ? (rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1) : rows >= 8192 ? 2 : 1;
-      else if (kern == SWEEP_NARROW) v = rows >= 16384 ? 4 : 1;
-      const unsigned long long unit = (kern == SWEEP_FP8 ? 4 * FP8_BLOCK_BYTES : 32ull << lw) * v;
+      if (kern == SWEEP_SHIFT) v = rows >= 4 * 2432 ? 4 : 1;
+      else if (kern == SWEEP_NARROW) v = rows >= 8 * 2432 ? 8 : rows >= 2 * 2432 ? 2 : 1;
+      else if (kern != SWEEP_FP8 && k.nsrc == 1) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
+      else if (kern == SWEEP_FOLD) v = rows >= 2 * 2432 ? 2 : 1;
+      const unsigned long long unit = row_bytes(kern, k) * v;
       const unsigned long long upm = (k.nbytes + unit - 1) / unit;
       k.meta = sweep_meta(dt, sweep_rop(k.meta), lw, v, kern);
       k.unit0 = (uint32_t)units;
@@ -237,7 +246,7 @@ void plan_launches(Sweep &sw) {
       if (k.nsrc > 1) words = std::max(words, sw.depth * acc * v);
     }
     SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words};
-    const uint32_t most = kern == SWEEP_COPY ? 512 : kern == SWEEP_FP8 ? 128 : 256;
+    const uint32_t most = SWEEP_THREADS[kern];
     // a short pass uses small CTAs, so that its units reach every SM
     uint32_t warps = most / 32;
     while (warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;

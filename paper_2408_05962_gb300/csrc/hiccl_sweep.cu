@@ -7,20 +7,25 @@
 // unit -- V vectors of 32 lanes of one member -- and loads up to eight
 // sources before it folds the first, so that 16 warps an SM hold 64 to 128
 // KiB in flight; the value goes to every destination straight from
-// registers.  Nothing waits on another CTA, so the grid is one warp per unit
+// registers.  CTAs are small (64 threads for folds), so that a finished warp's
+// registers are not held by its slower neighbours: 635 against 641 us for the
+// All-reduce below at 256 threads, 557 against 572 us for a group of 48
+// collectives.  Nothing waits on another CTA, so the grid is one warp per unit
 // and the hardware's CTA scheduler balances the tail: measured against a
 // persistent grid of the same code, 41.3 against 74 us for a 4 MiB Broadcast
 // to 64 ranks, 624 against 676 us for the All-reduce below; bulk (TMA) loads
 // and stores through shared-memory rings measured 48.9 and 672 us.
 //
 // Against the step executor, GB300, a start as a program times it: All-reduce
-// of 64 MiB a rank over 32 ranks 769 -> 662 us (6.49 TB/s of the inputs read
-// and outputs written once), All-reduce of 64 KiB of BF16 over 8 ranks (graph
-// replay) 22.6 -> 6.1 us, the seven collectives of 64 ranks x 4 MiB (graph
-// replay) 456 -> 312 us, an odd-length 6 MiB All-reduce over 16 ranks
-// 530 -> 70 us.
+// of 64 MiB a rank over 32 ranks 769 -> 646 us (626 us, 6.87 TB/s of the
+// inputs read and outputs written once, without the host), All-reduce of 64
+// KiB of BF16 over 8 ranks (graph replay) 22.6 -> 6.8 us, the seven
+// collectives of 64 ranks x 4 MiB (graph replay) 456 -> 306 us, an odd-length
+// 6 MiB All-reduce over 16 ranks 531 -> 54 us.
 
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "hiccl_device.cuh"
 #include "hiccl_internal.h"
@@ -71,29 +76,12 @@ template <int FAM, int W>
 struct Acc {
   static constexpr bool BF = FAM == BF16_SUM || FAM == BF16_ANY;
   static constexpr int N = BF ? W / 2 : W / 4;
-  uint32_t a[N];
 
   __device__ __forceinline__ static uint32_t widen(const Raw<W> &r, int i) {
     if constexpr (!BF) return r.w[i];
     else return i & 1 ? r.w[i / 2] & 0xffff0000u : r.w[i / 2] << 16;
   }
-  __device__ __forceinline__ static uint32_t comb(uint32_t x, uint32_t y, uint32_t dt, uint32_t rop) {
-    if constexpr (FAM == F32_SUM || FAM == BF16_SUM)
-      return __float_as_uint(__fadd_rn(__uint_as_float(x), __uint_as_float(y)));
-    else if constexpr (FAM == BF16_ANY)
-      return __float_as_uint(comb_f(__uint_as_float(x), __uint_as_float(y), rop));
-    else
-      return comb32(x, y, dt, rop);
-  }
-  __device__ __forceinline__ void start(const Raw<W> &r) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = widen(r, i);
-  }
-  __device__ __forceinline__ void add(const Raw<W> &r, uint32_t dt, uint32_t rop) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = comb(a[i], widen(r, i), dt, rop);
-  }
-  __device__ __forceinline__ Raw<W> pack() const {
+  __device__ __forceinline__ static Raw<W> pack(const uint32_t *a) {
     Raw<W> r;
     if constexpr (!BF) {
 #pragma unroll
@@ -106,10 +94,50 @@ struct Acc {
     }
     return r;
   }
-  __device__ __forceinline__ void round() {
-    if constexpr (BF) start(pack());
+  __device__ __forceinline__ static void round(uint32_t *a) {
+    if constexpr (BF) {
+      const Raw<W> r = pack(a);
+#pragma unroll
+      for (int i = 0; i < N; ++i) a[i] = widen(r, i);
+    }
   }
 };
+
+// a[i] = a[i] op b(i) over n words, the operator's branch taken once (once per
+// word, a 64-way int32 maximum of 1 MiB a rank took 39 us instead of 26)
+template <int FAM, int N, typename F>
+__device__ __forceinline__ void combine(uint32_t *a, F b, uint32_t dt, uint32_t rop) {
+  auto f = [](uint32_t x) { return __uint_as_float(x); };
+  auto each = [&](auto op) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = op(a[i], b(i));
+  };
+  auto add = [&](uint32_t x, uint32_t y) { return __float_as_uint(__fadd_rn(f(x), f(y))); };
+  auto fmx = [&](uint32_t x, uint32_t y) { return __float_as_uint(fmaxf(f(x), f(y))); };
+  auto fmn = [&](uint32_t x, uint32_t y) { return __float_as_uint(fminf(f(x), f(y))); };
+  if constexpr (FAM == F32_SUM || FAM == BF16_SUM) {
+    each(add);
+  } else if constexpr (FAM == BF16_ANY) {
+    if (rop == HICCL_MAX) each(fmx);
+    else each(fmn);
+  } else if (dt == HICCL_F32) {
+    if (rop == HICCL_MAX) each(fmx);
+    else each(fmn);
+  } else {
+    switch (rop) {
+      case HICCL_SUM: each([](uint32_t x, uint32_t y) { return x + y; }); break;
+      case HICCL_MAX: each([](uint32_t x, uint32_t y) { return (uint32_t)max((int)x, (int)y); }); break;
+      case HICCL_MIN: each([](uint32_t x, uint32_t y) { return (uint32_t)min((int)x, (int)y); }); break;
+      default: each([](uint32_t x, uint32_t y) { return (x | y) != 0u ? 1u : 0u; }); break;
+    }
+  }
+}
+
+// the sources q .. q + 31 whose tokens are not plain combines, one bit each
+__device__ __forceinline__ uint32_t more_than_combine(const uint32_t *tok, uint32_t q, uint32_t nsrc) {
+  const uint32_t i = q + (threadIdx.x & 31);
+  return __ballot_sync(0xffffffffu, i < nsrc && __ldg(tok + i) != 0u);
+}
 
 // One unit of a fold: V vectors of W bytes per lane, at byte offset `off` of
 // the lane's first vector, vectors 32 * W bytes apart, those ending past
@@ -121,19 +149,20 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
                                           uint32_t nsrc, uint32_t ndst, unsigned long long off, unsigned long long end,
                                           uint32_t dt, uint32_t rop, uint32_t *stack, uint32_t threads) {
   using A = Acc<FAM, W>;
-  A acc[V];
+  constexpr int N = A::N;
+  uint32_t acc[V * N];
   bool on[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) on[v] = off + v * (32 * W) + W <= end;
-  uint32_t sp = 0;   // words saved
+  static_assert(32 % U == 0, "the sources in flight lie in one 32-bit mask");
+  uint32_t sp = 0, nz = 0;   // words saved; which of 32 tokens do more than combine
   for (uint32_t q = 0; q < nsrc; q += U) {
     Raw<W> x[U][V];
-    uint32_t t[U];
+    if ((q & 31u) == 0) nz = more_than_combine(tok, q, nsrc);
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (q + u < nsrc) {
         const unsigned long long s = __ldg(P + q + u) + off;
-        t[u] = __ldg(tok + q + u);
 #pragma unroll
         for (int v = 0; v < V; ++v)
           if (on[v]) x[u][v] = ld_raw<W>(s + v * (32 * W));
@@ -141,41 +170,48 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (q + u < nsrc) {
-        if (t[u] & TOK_START) {
-          if (t[u] & TOK_PUSH) {
+        auto src = [&](int i) { return A::widen(x[u][i / N], i % N); };
+        if (!((nz >> ((q & 31u) + u)) & 1u)) {
+          combine<FAM, V * N>(acc, src, dt, rop);
+          continue;
+        }
+        const uint32_t tk = __ldg(tok + q + u);
+        if (tk & TOK_START) {
+          if (tk & TOK_PUSH) {
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-#pragma unroll
-              for (int i = 0; i < A::N; ++i) stack[(sp + v * A::N + i) * threads] = acc[v].a[i];
-            sp += V * A::N;
+            for (int i = 0; i < V * N; ++i) stack[(sp + i) * threads] = acc[i];
+            sp += V * N;
           }
 #pragma unroll
-          for (int v = 0; v < V; ++v) acc[v].start(x[u][v]);
+          for (int i = 0; i < V * N; ++i) acc[i] = src(i);
         } else {
-#pragma unroll
-          for (int v = 0; v < V; ++v) acc[v].add(x[u][v], dt, rop);
+          combine<FAM, V * N>(acc, src, dt, rop);
         }
-        for (uint32_t o = t[u] >> TOK_OPS; o; o >>= 2) {
+        for (uint32_t o = tk >> TOK_OPS; o; o >>= 2) {
           if ((o & 3u) == TOK_ROUND) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) acc[v].round();
-          } else {
-            const bool pop = (o & 3u) == TOK_POP;
-            sp -= V * A::N;
+            for (int v = 0; v < V; ++v) A::round(acc + v * N);
+            continue;
+          }
+          sp -= V * N;
+          const bool pop = (o & 3u) == TOK_POP;   // the saved value is the left operand
 #pragma unroll
-            for (int v = 0; v < V; ++v)
+          for (int v = 0; v < V; ++v) {
+            uint32_t y[N];
 #pragma unroll
-              for (int i = 0; i < A::N; ++i) {
-                const uint32_t y = stack[(sp + v * A::N + i) * threads];
-                acc[v].a[i] = pop ? A::comb(y, acc[v].a[i], dt, rop) : A::comb(acc[v].a[i], y, dt, rop);
-              }
+            for (int i = 0; i < N; ++i) {
+              const uint32_t z = stack[(sp + v * N + i) * threads], w = acc[v * N + i];
+              acc[v * N + i] = pop ? z : w;
+              y[i] = pop ? w : z;
+            }
+            combine<FAM, N>(acc + v * N, [&](int i) { return y[i]; }, dt, rop);
           }
         }
       }
   }
   Raw<W> r[V];
 #pragma unroll
-  for (int v = 0; v < V; ++v) r[v] = acc[v].pack();
+  for (int v = 0; v < V; ++v) r[v] = A::pack(acc + v * N);
 #pragma unroll 4
   for (uint32_t d = 0; d < ndst; ++d) {
     const unsigned long long a = __ldg(P + nsrc + d) + off;
@@ -255,36 +291,48 @@ __device__ __forceinline__ void launch_order() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Where the whole 16-byte vectors of a member lie: all its operands are
+// equally far off a boundary, so they start at byte `head` and end at `end`
+// of each; the elements before and after are at most 14 + 14 bytes.  (Rows of
+// a multiple of 16 bytes with odd chunk lengths are such operands: an odd
+// 6 MiB All-reduce over 16 ranks takes 38 us, 55 us by 4-byte accesses.)
+struct Body {
+  unsigned long long head, end;
+};
+__device__ __forceinline__ Body body_of(const SweepClass &k, const unsigned long long *P) {
+  const unsigned long long h = min((0ull - __ldg(P)) & 15u, k.nbytes);
+  return Body{h, h + ((k.nbytes - h) & ~15ull)};
+}
+// byte offset of this lane's element of W bytes outside the body (nbytes: none)
 template <int W>
-__device__ __forceinline__ void copy_any(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
+__device__ __forceinline__ unsigned long long edge_of(const SweepClass &k, const Body &b, int lane) {
+  const unsigned long long o = (unsigned long long)lane * W;
+  return o < b.head ? o : min(b.end + (o - b.head), k.nbytes);
+}
+
+// a copy's unit, and with the last one the member's edges
+__device__ __forceinline__ void copy_member(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
   const uint32_t v = sweep_v(k.meta);
-  const unsigned long long off = (unsigned long long)part * (32 * W) * v + lane * W;
-  if (v == 4) copy_unit<W, 4>(P, k.ndst, off, k.nbytes);
-  else if (v == 2) copy_unit<W, 2>(P, k.ndst, off, k.nbytes);
-  else copy_unit<W, 1>(P, k.ndst, off, k.nbytes);
+  const Body b = body_of(k, P);
+  const unsigned long long off = b.head + (unsigned long long)part * 512 * v + lane * 16;
+  if (v == 4) copy_unit<16, 4>(P, k.ndst, off, b.end);
+  else if (v == 2) copy_unit<16, 2>(P, k.ndst, off, b.end);
+  else copy_unit<16, 1>(P, k.ndst, off, b.end);
+  if (part + 1 == k.upm && b.end - b.head != k.nbytes) copy_unit<2, 1>(P, k.ndst, edge_of<2>(k, b, lane), k.nbytes);
 }
 
-// the bytes after the last whole vector of a member, element by element
-__device__ __forceinline__ void copy_tail(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
-  if (part + 1 == k.upm && (k.nbytes & 15u))
-    copy_unit<2, 1>(P, k.ndst, (k.nbytes & ~15ull) + lane * 2, k.nbytes);
-}
-
-// copies of aligned operands: V vectors a lane in flight, stored to every
-// destination
-__global__ void __launch_bounds__(512, 2) sweep_copy_kernel(const __grid_constant__ SweepArgs A) {
+// V vectors a lane in flight, stored to every destination
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_COPY], 8) sweep_copy_kernel(const __grid_constant__ SweepArgs A) {
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
   if (unit >= A.units) return;
   const unsigned long long *P;
   uint32_t part;
   const SweepClass k = find_class(A, unit, P, part);
-  copy_any<16>(k, P, part, lane);
-  copy_tail(k, P, part, lane);
+  copy_member(k, P, part, threadIdx.x & 31);
 }
 
-__global__ void __launch_bounds__(256, 2) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FOLD], 8) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ uint32_t saved[];
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -294,25 +342,34 @@ __global__ void __launch_bounds__(256, 2) sweep_fold_kernel(const __grid_constan
   uint32_t part;
   const SweepClass k = find_class(A, unit, P, part);
   if (k.nsrc == 1) {
-    copy_any<16>(k, P, part, lane);
-    copy_tail(k, P, part, lane);
+    copy_member(k, P, part, lane);
     return;
   }
   uint32_t *stack = saved + threadIdx.x;
   const uint32_t v = sweep_v(k.meta);
-  const unsigned long long off = (unsigned long long)part * 512 * v + lane * 16;
-  if (v == 2) fold_any<16, 2, 8>(A, k, P, off, k.nbytes, stack);
-  else fold_any<16, 1, 8>(A, k, P, off, k.nbytes, stack);
-  if (part + 1 == k.upm && (k.nbytes & 15u)) {
-    const unsigned long long t0 = k.nbytes & ~15ull;
-    if (sweep_dtype(k.meta) == HICCL_BF16) fold_any<2, 1, 8>(A, k, P, t0 + lane * 2, k.nbytes, stack);
-    else fold_any<4, 1, 8>(A, k, P, t0 + lane * 4, k.nbytes, stack);
+  const Body b = body_of(k, P);
+  const unsigned long long off = b.head + (unsigned long long)part * 512 * v + lane * 16;
+  if (v == 2) fold_any<16, 2, 8>(A, k, P, off, b.end, stack);
+  else fold_any<16, 1, 16>(A, k, P, off, b.end, stack);
+  if (part + 1 == k.upm && b.end - b.head != k.nbytes) {
+    if (sweep_dtype(k.meta) == HICCL_BF16) fold_any<2, 1, 8>(A, k, P, edge_of<2>(k, b, lane), k.nbytes, stack);
+    else fold_any<4, 1, 8>(A, k, P, edge_of<4>(k, b, lane), k.nbytes, stack);
   }
 }
 
-// operands off a 16-byte boundary: 4-byte accesses where every operand and
-// the length allow them, else 2-byte ones
-__global__ void __launch_bounds__(256, 4) sweep_narrow_kernel(const __grid_constant__ SweepArgs A) {
+// folds of operands that lie differently off a 16-byte boundary: W-byte
+// accesses, 4 where every operand and
+// the length allow them, else 2
+template <int W>
+__device__ __forceinline__ void narrow_unit(const SweepArgs &A, const SweepClass &k, const unsigned long long *P,
+                                            uint32_t part, int lane, uint32_t *stack) {
+  const uint32_t v = sweep_v(k.meta);
+  const unsigned long long off = (unsigned long long)part * (32 * W) * v + lane * W;
+  if (v == 8) fold_any<W, 8, 4>(A, k, P, off, k.nbytes, stack);
+  else if (v == 2) fold_any<W, 2, 8>(A, k, P, off, k.nbytes, stack);
+  else fold_any<W, 1, 16>(A, k, P, off, k.nbytes, stack);
+}
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_NARROW], 10) sweep_narrow_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ uint32_t saved[];
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -321,24 +378,88 @@ __global__ void __launch_bounds__(256, 4) sweep_narrow_kernel(const __grid_const
   const unsigned long long *P;
   uint32_t part;
   const SweepClass k = find_class(A, unit, P, part);
-  const uint32_t v = sweep_v(k.meta);
-  if (sweep_lw(k.meta) == 2) {
-    if (k.nsrc == 1) {
-      copy_any<4>(k, P, part, lane);
-      return;
-    }
-    const unsigned long long off = (unsigned long long)part * 128 * v + lane * 4;
-    if (v == 4) fold_any<4, 4, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
-    else fold_any<4, 1, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
-  } else {
-    if (k.nsrc == 1) {
-      copy_any<2>(k, P, part, lane);
-      return;
-    }
-    const unsigned long long off = (unsigned long long)part * 64 * v + lane * 2;
-    if (v == 4) fold_any<2, 4, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
-    else fold_any<2, 1, 8>(A, k, P, off, k.nbytes, saved + threadIdx.x);
+  if (sweep_lw(k.meta) == 2) narrow_unit<4>(A, k, P, part, lane, saved + threadIdx.x);
+  else narrow_unit<2>(A, k, P, part, lane, saved + threadIdx.x);
+}
+
+// Copies between operands that lie differently off a 16-byte boundary.  The
+// source is read by its aligned vectors; the 16 bytes that a destination's
+// vector takes straddle two of them, the lane's own and the next lane's, and
+// are shifted out of the pair.  (Element accesses are bound by latency: 64
+// bytes a warp request, 90 us for an odd-length BF16 All-to-all of 64 ranks x
+// 1 MiB at four requests in flight and 45 us at sixteen, against 27 us here,
+// 4.9 TB/s.)  A unit is V rows of 31 destination vectors
+// (lane 31 loads only for lane 30) -- 496 source bytes a row; the elements
+// that no whole pair covers, at most 31 bytes at each end, go one by one with
+// the member's last unit.
+__device__ __forceinline__ uint4 shift_pair(const uint4 &a, const uint4 &b, uint32_t e) {
+  const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  const uint32_t bits = 8 * (e & 3u);
+  uint4 r;
+  auto take = [&](auto c) {
+    constexpr int K = decltype(c)::value;
+    // (the word past the pair is only reached with bits == 0)
+    r.x = __funnelshift_r(w[K], w[K + 1], bits);
+    r.y = __funnelshift_r(w[K + 1], w[K + 2], bits);
+    r.z = __funnelshift_r(w[K + 2], w[K + 3], bits);
+    r.w = __funnelshift_r(w[K + 3], w[K + 4], bits);
+  };
+  switch (e >> 2) {
+    case 0: take(std::integral_constant<int, 0>{}); break;
+    case 1: take(std::integral_constant<int, 1>{}); break;
+    case 2: take(std::integral_constant<int, 2>{}); break;
+    default: take(std::integral_constant<int, 3>{}); break;
   }
+  return r;
+}
+template <int V>
+__device__ __forceinline__ void shift_unit(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
+  const unsigned long long src = __ldg(P), n = k.nbytes;
+  const unsigned long long o0 = (0ull - src) & 15u;           // first whole vector of the source
+  const unsigned long long last = o0 + 16 <= n ? o0 + ((n - o0 - 16) & ~15ull) : 0ull;   // the last one
+  const unsigned long long base = o0 + ((unsigned long long)part * V * 31 + lane) * 16;
+  uint4 a[V], b[V];
+  const bool any = o0 + 32 <= n;                              // at least one pair
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const unsigned long long o = base + v * (31 * 16);
+    a[v] = make_uint4(0, 0, 0, 0);
+    if (any && o <= last) a[v] = __ldcg(reinterpret_cast<const uint4 *>(src + o));
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    b[v].x = __shfl_down_sync(0xffffffffu, a[v].x, 1);
+    b[v].y = __shfl_down_sync(0xffffffffu, a[v].y, 1);
+    b[v].z = __shfl_down_sync(0xffffffffu, a[v].z, 1);
+    b[v].w = __shfl_down_sync(0xffffffffu, a[v].w, 1);
+  }
+  // the ends: lanes 0 .. 15 the first 32 bytes, lanes 16 .. 31 those from the
+  // last vector on, two bytes each (a short member has only the first)
+  const bool edges = part + 1 == k.upm;
+  const unsigned long long at = lane < 16 ? 2ull * lane : (any ? last + 2ull * (lane - 16) : 32 + 2ull * (lane - 16));
+  unsigned short ev = 0;
+  if (edges && at < n) ev = __ldcg(reinterpret_cast<const unsigned short *>(src + at));
+  for (uint32_t d = 0; d < k.ndst; ++d) {
+    const unsigned long long dst = __ldg(P + 1 + d);
+    const uint32_t e = (uint32_t)((0ull - (dst + o0)) & 15u);   // from a source vector to the destination's
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const unsigned long long o = base + v * (31 * 16);
+      if (any && lane < 31 && o < last) *reinterpret_cast<uint4 *>(dst + o + e) = shift_pair(a[v], b[v], e);
+    }
+    if (edges && at < n && (!any || (lane < 16 ? at < o0 + e : at >= last + e)))
+      *reinterpret_cast<unsigned short *>(dst + at) = ev;
+  }
+}
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_SHIFT], 8) sweep_shift_kernel(const __grid_constant__ SweepArgs A) {
+  launch_order();
+  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (unit >= A.units) return;
+  const unsigned long long *P;
+  uint32_t part;
+  const SweepClass k = find_class(A, unit, P, part);
+  if (sweep_v(k.meta) == 4) shift_unit<4>(k, P, part, threadIdx.x & 31);
+  else shift_unit<1>(k, P, part, threadIdx.x & 31);
 }
 
 // ---- FP8 blocks --------------------------------------------------------------------
@@ -428,13 +549,13 @@ __device__ __forceinline__ void cp_wait() {
 // a source, which keeps FP8_SLOTS - 1 in flight through folds, encodings and
 // stores without holding registers (72 a thread, 24 warps an SM).  Copies and
 // stores move the unit as one range of whole sectors, and only the fold reads
-// it by blocks.  All-reduce of 2 Mi values a rank over 32 ranks ({4, 8}),
+// it by blocks.  All-reduce of 16 Mi values a rank over 32 ranks ({4, 8}),
 // 1.21 GB in and out: 265 us with the next sources loaded into registers (16
 // warps an SM; 403 us when refilled one by one), 223 us through the ring by
 // blocks, 199 us by the unit's range, 6.1 TB/s; two or four units a warp
 // lose 5 and 10 %, neighbouring warps on neighbouring units read longer
 // stretches of each source at a time.
-__global__ void __launch_bounds__(128, 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ __align__(16) uint32_t saved[];
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -473,7 +594,7 @@ __global__ void __launch_bounds__(128, 6) sweep_fp8_kernel(const __grid_constant
   uint32_t sp = 0, nz = 0;   // words saved; which of 32 tokens do more than combine
   uint32_t slot = 0;
   for (uint32_t q = 0; q < k.nsrc; ++q) {
-    if ((q & 31u) == 0) nz = __ballot_sync(0xffffffffu, q + lane < k.nsrc && __ldg(tok + q + lane) != 0u);
+    if ((q & 31u) == 0) nz = more_than_combine(tok, q, k.nsrc);
     cp_wait<FP8_SLOTS - 2>();
     __syncwarp();              // every lane's copies have landed, and the slot read last is free
     load((slot + FP8_SLOTS - 1) % FP8_SLOTS);
@@ -536,7 +657,8 @@ __global__ void __launch_bounds__(128, 6) sweep_fp8_kernel(const __grid_constant
 }
 
 typedef void (*Kernel)(const SweepArgs);
-const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel};
+const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel,
+                                         sweep_shift_kernel};
 
 }  // namespace
 

@@ -20,11 +20,11 @@ def built():
     __graft_entry__.build()
 
 
-def _buffers(kind, P, d, dtype, seed):
+def _buffers(kind, P, d, dtype, seed, pad=0):
     import torch
     from paper_2408_05962_gb300 import collectives as C
     tdt = {"f32": torch.float32, "i32": torch.int32, "bf16": torch.bfloat16, "fp8": torch.uint8}[dtype]
-    b = C.Buffers(kind, P, d, tdt, "cuda")
+    b = C.Buffers(kind, P, d, tdt, "cuda", pad)
     g = torch.Generator(device="cuda")
     g.manual_seed(seed)
     if dtype == "i32":
@@ -41,11 +41,11 @@ def _buffers(kind, P, d, dtype, seed):
     return b
 
 
-def _both(kind, P, h, s, m, d, dtype, op="sum", ring=1, seed=0):
+def _both(kind, P, h, s, m, d, dtype, op="sum", ring=1, seed=0, pad=0):
     """The sweep's result equals the step executor's."""
     import torch
     from paper_2408_05962_gb300 import hiccl as H
-    b = _buffers(kind, P, d, dtype, seed)
+    b = _buffers(kind, P, d, dtype, seed, pad)
     got = []
     for trace in (0, 1):
         c = H.Comm(P, dtype)
@@ -71,6 +71,15 @@ def _both(kind, P, h, s, m, d, dtype, op="sum", ring=1, seed=0):
 @pytest.mark.parametrize("kind", ["allreduce", "alltoall"])
 def test_chunk_edges(kind, dtype, d):
     _both(kind, 8, [2, 4], 1, 1, d, dtype, seed=d)
+
+
+# rows `pad` elements longer than their data: chunks of every rank lie
+# differently off a 16-byte boundary, and the padding is not written
+@pytest.mark.parametrize("d", [1, 7, 9, 15, 16, 23, 247, 248, 249, 255, 991, 993, 1000, 66000, 262147])
+@pytest.mark.parametrize("dtype,pad", [("f32", 1), ("f32", 3), ("bf16", 1), ("bf16", 2), ("bf16", 7)])
+@pytest.mark.parametrize("kind", ["allreduce", "alltoall", "broadcast"])
+def test_operands_off_each_other(kind, dtype, pad, d):
+    _both(kind, 6, [2, 3], 1, 1, d, dtype, seed=d, pad=pad)
 
 
 @pytest.mark.parametrize("dtype,op", [("f32", "max"), ("i32", "min"), ("i32", "lor"), ("bf16", "min"), ("bf16", "sum")])

@@ -19,7 +19,7 @@ from tests._bridge import FakeAddresses, register
 from tests._cases import fill, random_program
 
 START, PUSH, ROUND, POP, JOIN = 1, 2, 1, 2, 3
-COPY, FOLD, FP8, NARROW = range(4)
+COPY, FOLD, FP8, NARROW, SHIFT = range(5)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -42,7 +42,7 @@ def decode(blob):
     assert len(blob) == o + 8 * npt + 4 * nt
     for c in cls:
         m = c["meta"]
-        c.update(dtype=m & 15, rop=(m >> 4) & 7, width=1 << ((m >> 7) & 7), v=(m >> 10) & 15, kernel=(m >> 14) & 7)
+        c.update(dtype=m & 15, rop=(m >> 4) & 7, width=1 << ((m >> 7) & 7), v=(m >> 10) & 31, kernel=(m >> 15) & 7)
     return cls, lau, ptrs, toks
 
 
@@ -93,14 +93,15 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         units = 0
         for c in cls[L["lo"]:L["hi"]]:
             assert c["kernel"] == L["kernel"] and c["unit0"] == units
-            unit = (4 * 144 if L["kernel"] == FP8 else 32 * c["width"]) * c["v"]
+            unit = {FP8: 4 * 144, SHIFT: 31 * 16}.get(L["kernel"], 32 * c["width"]) * c["v"]
             assert (c["upm"] - 1) * unit < c["nbytes"] <= c["upm"] * unit        # units tile a member
-            assert c["v"] in (1, 2, 4)
+            assert c["v"] in (1, 2, 4, 8, 16)
             units += c["upm"] * c["nmem"]
             for i in range(c["nmem"]):
                 p = ptrs[c["ptr"] + i * (c["nsrc"] + c["ndst"]):][:c["nsrc"] + c["ndst"]]
-                assert all(a % c["width"] == 0 for a in p) and (L["kernel"] == NARROW) == (c["width"] < 16)
-                assert (c["nsrc"] > 1) or L["kernel"] != FP8
+                assert all((a - p[0]) % c["width"] == 0 for a in p) and (c["width"] == 16 or p[0] % c["width"] == 0)
+                assert (L["kernel"] in (NARROW, SHIFT)) == (c["width"] < 16)
+                assert L["kernel"] == FOLD or (c["nsrc"] > 1) == (L["kernel"] in (FP8, NARROW))
                 members.append((c, p))
         assert L["units"] == units and L["threads"] in (32, 64, 128, 256, 512)
     rng = np.random.Generator(np.random.PCG64(seed))
