@@ -384,17 +384,16 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
  * `out` receives, without padding: the counts of classes, launches, operand
  * pointers and tokens (u64 each); the classes (48 bytes: bytes per operand
  * u64, first pointer u64, then u32 first unit, units per member, members,
- * sources, destinations, first token, meta, 0); the launches (24 bytes: u32
- * kernel, first and end class, units, threads, saved words per thread); the
- * pointers (u64; per member its sources in evaluation order, then its
+ * sources, destinations, first token, meta, destinations per unit); the
+ * launches (24 bytes: u32 kernel, first and end class, units, threads, saved
+ * words per thread); the pointers (u64; per member its sources in evaluation order, then its
  * destinations); the tokens (u32, one per source: bit 0 the source starts the
  * accumulator, bit 1 after the old one was saved, else it is combined in;
  * then two-bit operations from bit 8 on: 1 round the accumulator to the
  * payload, 2 combine (saved, accumulator), 3 combine (accumulator, saved)).
  * meta: dtype 4 bits, operator 3, log2 of the access width 3, vectors per lane 5,
- * kernel 3 (0 copies, 1 folds, 2 FP8 folds; operands
- * that lie differently off a 16-byte boundary: 3 folds, 4 copies).  *bytes
- * receives the size (0: the plan has no sweep); a NULL or too small `out` is
+ * kernel 3 (0 copies, 1 folds, 2 FP8 folds; of operands that lie differently
+ * off a 16-byte boundary: 3 folds, 4 copies).  *bytes receives the size (0: the plan has no sweep); a NULL or too small `out` is
  * left alone.  HICCL_ERR_STATE without a plan. */
 hiccl_status_t hiccl_debug_sweep(hiccl_comm_t comm, void *out, size_t capacity, size_t *bytes);
 

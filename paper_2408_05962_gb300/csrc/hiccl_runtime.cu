@@ -1089,6 +1089,7 @@ static hiccl_status_t upload_sweep(hiccl_comm *c) {
     A.nclass = L.class_hi - L.class_lo;
     A.units = L.units;
     for (uint32_t k = 0; k < A.nclass && k < SWEEP_PREFIX; ++k) A.unit0[k] = w.classes[L.class_lo + k].unit0;
+    for (uint32_t k = 0; k < A.nclass && k < SWEEP_INLINE; ++k) A.first[k] = w.classes[L.class_lo + k];
     d->sweeps.push_back(A);
   }
   // the upload must have landed before the first start (on any stream)

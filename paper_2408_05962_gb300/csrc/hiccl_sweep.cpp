@@ -200,6 +200,11 @@ unsigned long long row_bytes(uint32_t kern, const SweepClass &k) {
   return kern == SWEEP_SHIFT ? 31 * 16 : 32ull << sweep_lw(k.meta);
 }
 
+// units that store one range of a member to all its destinations
+unsigned long long groups(const SweepClass &k) {
+  return k.nsrc > 1 ? 1 : (k.ndst + SWEEP_GROUP - 1) / SWEEP_GROUP;
+}
+
 // Launches, vectors per lane and units of a sweep's classes.
 void plan_launches(Sweep &sw) {
   bool folds = false;
@@ -219,7 +224,7 @@ void plan_launches(Sweep &sw) {
     for (; z < sw.classes.size() && kernel_of(sw.classes[z]) == kern; ++z) {
       const SweepClass &k = sw.classes[z];
       const unsigned long long row = row_bytes(kern, k);
-      rows += (k.nbytes + row - 1) / row * k.nmem;
+      rows += (k.nbytes + row - 1) / row * k.nmem * groups(k);
     }
     unsigned long long units = 0;
     uint32_t words = 0;
@@ -230,13 +235,13 @@ void plan_launches(Sweep &sw) {
       if (kern == SWEEP_SHIFT) v = rows >= 4 * 2432 ? 4 : 1;
       else if (kern == SWEEP_NARROW) v = rows >= 8 * 2432 ? 8 : rows >= 2 * 2432 ? 2 : 1;
       else if (kern != SWEEP_FP8 && k.nsrc == 1) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
-      else if (kern == SWEEP_FOLD) v = rows >= 2 * 2432 ? 2 : 1;
       const unsigned long long unit = row_bytes(kern, k) * v;
       const unsigned long long upm = (k.nbytes + unit - 1) / unit;
       k.meta = sweep_meta(dt, sweep_rop(k.meta), lw, v, kern);
       k.unit0 = (uint32_t)units;
       k.upm = (uint32_t)upm;
-      units += upm * k.nmem;
+      k.group = k.nsrc > 1 ? k.ndst : SWEEP_GROUP;
+      units += upm * k.nmem * groups(k);
       if (units > 0xF0000000ull) {   // far beyond device memory
         sw.valid = false;
         return;

@@ -4,24 +4,25 @@
 //
 // What bounds a pass is memory: every input is read once and every output
 // written once, with at most one add per value between.  A warp takes one
-// unit -- V vectors of 32 lanes of one member -- and loads up to eight
-// sources before it folds the first, so that 16 warps an SM hold 64 to 128
-// KiB in flight; the value goes to every destination straight from
-// registers.  CTAs are small (64 threads for folds), so that a finished warp's
-// registers are not held by its slower neighbours: 635 against 641 us for the
-// All-reduce below at 256 threads, 557 against 572 us for a group of 48
-// collectives.  Nothing waits on another CTA, so the grid is one warp per unit
-// and the hardware's CTA scheduler balances the tail: measured against a
-// persistent grid of the same code, 41.3 against 74 us for a 4 MiB Broadcast
-// to 64 ranks, 624 against 676 us for the All-reduce below; bulk (TMA) loads
-// and stores through shared-memory rings measured 48.9 and 672 us.
+// unit of one member.  Folds bring their sources through a ring of
+// asynchronous copies in shared memory, one 16-byte vector a lane and source,
+// so that the loads in flight (30 warps x 4 to 6 KiB an SM) need no registers
+// and never wait for a fold; copies load up to four vectors a lane.  The
+// value goes to its destinations straight from registers.  Nothing waits on
+// another CTA, so the grid is one warp per unit, in CTAs of two to four warps
+// that free their SM as they finish, and the hardware's CTA scheduler
+// balances the tail.  Measured against: a persistent grid of the same code,
+// 74 against 41 us for a 4 MiB Broadcast to 64 ranks; bulk (TMA) loads and
+// stores through shared-memory rings, 672 against 624 us for the All-reduce
+// below; eight sources in registers, 53.9 against 46.7 us for a BF16
+// Reduce-scatter of 16 ranks x 16 MiB.
 //
 // Against the step executor, GB300, a start as a program times it: All-reduce
-// of 64 MiB a rank over 32 ranks 769 -> 646 us (626 us, 6.87 TB/s of the
+// of 64 MiB a rank over 32 ranks 769 -> 644 us (623 us, 6.89 TB/s of the
 // inputs read and outputs written once, without the host), All-reduce of 64
-// KiB of BF16 over 8 ranks (graph replay) 22.6 -> 6.8 us, the seven
-// collectives of 64 ranks x 4 MiB (graph replay) 456 -> 306 us, an odd-length
-// 6 MiB All-reduce over 16 ranks 531 -> 54 us.
+// KiB of BF16 over 8 ranks (graph replay) 22.7 -> 6.2 us, the seven
+// collectives of 64 ranks x 4 MiB (graph replay) 456 -> 290 us, an odd-length
+// 6 MiB All-reduce over 16 ranks 534 -> 54 us.
 
 #include <cuda_runtime.h>
 
@@ -34,6 +35,63 @@
 namespace hiccl {
 
 namespace {
+
+// Groups of a fold's ring: three hold 6 KiB a warp, 30 warps an SM.  A pass
+// with fewer units than half of those warps (SHORT_UNITS) deepens it instead.
+// Measured with two / three / four groups: 45.1 / 43.6 / 50 us for a
+// Reduce-scatter of 64 ranks x 4 MiB, 48.7 / 46.7 / 56 us for 16 ranks x
+// 16 MiB of BF16.
+constexpr int FOLD_GROUPS = 3, FOLD_GROUPS_SHORT = 5;
+constexpr uint32_t SHORT_UNITS = 152 * 16;
+
+// ---- units -----------------------------------------------------------------------
+
+// What a unit does: part `part` of a member of class k with operand pointers
+// P, stored to the destinations P[d0 .. d1).
+struct Unit {
+  SweepClass k;
+  const unsigned long long *P;
+  uint32_t part, d0, d1;
+};
+__device__ __forceinline__ Unit find_unit(const SweepArgs &A, uint32_t unit) {
+  uint32_t lo = 0, hi = A.nclass;
+  while (hi - lo > 1) {   // last class whose first unit is not past `unit`
+    const uint32_t mid = (lo + hi) >> 1;
+    const uint32_t u0 = A.nclass <= SWEEP_PREFIX ? A.unit0[mid] : __ldg(&A.classes[mid].unit0);
+    if (u0 <= unit) lo = mid;
+    else hi = mid;
+  }
+  Unit r;
+  if (A.nclass <= SWEEP_INLINE) {
+    r.k = A.first[lo];
+  } else {
+    const uint4 *q = reinterpret_cast<const uint4 *>(A.classes + lo);
+    uint4 *z = reinterpret_cast<uint4 *>(&r.k);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) z[i] = __ldg(q + i);
+  }
+  const SweepClass &k = r.k;
+  uint32_t at = unit - k.unit0, g = 0;
+  if (k.group < k.ndst) {   // destination groups, tile by tile of the source
+    const uint32_t all = k.upm * k.nmem, tile = SWEEP_TILE / sweep_v(k.meta);
+    uint32_t base = 0, cur = all;
+    if (all > tile) {
+      const unsigned long long per = (unsigned long long)tile * ((k.ndst + k.group - 1) / k.group);
+      const uint32_t t = (uint32_t)(at / per);
+      at -= (uint32_t)(t * per);
+      base = t * tile;
+      cur = min(tile, all - base);
+    }
+    g = at / cur;
+    at = base + (at - g * cur);
+  }
+  const uint32_t mem = at / k.upm;
+  r.part = at - mem * k.upm;
+  r.P = A.ptrs + k.ptr + (unsigned long long)mem * (k.nsrc + k.ndst);
+  r.d0 = k.nsrc + g * k.group;
+  r.d1 = k.nsrc + min(k.ndst, (g + 1) * k.group);
+  return r;
+}
 
 // ---- accesses of W bytes per lane ----------------------------------------------
 
@@ -103,6 +161,21 @@ struct Acc {
   }
 };
 
+// two binary32 values in one 64-bit register pair
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpack2(unsigned long long d, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(d));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 // a[i] = a[i] op b(i) over n words, the operator's branch taken once (once per
 // word, a 64-way int32 maximum of 1 MiB a rank took 39 us instead of 26)
 template <int FAM, int N, typename F>
@@ -115,7 +188,15 @@ __device__ __forceinline__ void combine(uint32_t *a, F b, uint32_t dt, uint32_t 
   auto add = [&](uint32_t x, uint32_t y) { return __float_as_uint(__fadd_rn(f(x), f(y))); };
   auto fmx = [&](uint32_t x, uint32_t y) { return __float_as_uint(fmaxf(f(x), f(y))); };
   auto fmn = [&](uint32_t x, uint32_t y) { return __float_as_uint(fminf(f(x), f(y))); };
-  if constexpr (FAM == F32_SUM || FAM == BF16_SUM) {
+  if constexpr ((FAM == F32_SUM || FAM == BF16_SUM) && N % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {   // two sums an instruction
+      float lo, hi;
+      unpack2(add2(pack2(f(a[i]), f(a[i + 1])), pack2(f(b(i)), f(b(i + 1)))), lo, hi);
+      a[i] = __float_as_uint(lo);
+      a[i + 1] = __float_as_uint(hi);
+    }
+  } else if constexpr (FAM == F32_SUM || FAM == BF16_SUM) {
     each(add);
   } else if constexpr (FAM == BF16_ANY) {
     if (rop == HICCL_MAX) each(fmx);
@@ -133,11 +214,18 @@ __device__ __forceinline__ void combine(uint32_t *a, F b, uint32_t dt, uint32_t 
   }
 }
 
-// the sources q .. q + 31 whose tokens are not plain combines, one bit each
-__device__ __forceinline__ uint32_t more_than_combine(const uint32_t *tok, uint32_t q, uint32_t nsrc) {
-  const uint32_t i = q + (threadIdx.x & 31);
-  return __ballot_sync(0xffffffffu, i < nsrc && __ldg(tok + i) != 0u);
-}
+// The tokens of 32 sources, one a lane: a bit for each that is not a plain
+// combine, and the token itself on request.
+struct Tokens {
+  uint32_t mine = 0, nz = 0;
+  __device__ __forceinline__ void read(const uint32_t *tok, uint32_t q, uint32_t nsrc) {   // q a multiple of 32
+    const uint32_t i = q + (threadIdx.x & 31);
+    mine = i < nsrc ? __ldg(tok + i) : 0u;
+    nz = __ballot_sync(0xffffffffu, mine != 0u);
+  }
+  __device__ __forceinline__ bool plain(uint32_t q) const { return !((nz >> (q & 31u)) & 1u); }
+  __device__ __forceinline__ uint32_t at(uint32_t q) const { return __shfl_sync(0xffffffffu, mine, q & 31u); }
+};
 
 // One unit of a fold: V vectors of W bytes per lane, at byte offset `off` of
 // the lane's first vector, vectors 32 * W bytes apart, those ending past
@@ -155,10 +243,11 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
 #pragma unroll
   for (int v = 0; v < V; ++v) on[v] = off + v * (32 * W) + W <= end;
   static_assert(32 % U == 0, "the sources in flight lie in one 32-bit mask");
-  uint32_t sp = 0, nz = 0;   // words saved; which of 32 tokens do more than combine
+  uint32_t sp = 0;   // words saved
+  Tokens t;
   for (uint32_t q = 0; q < nsrc; q += U) {
     Raw<W> x[U][V];
-    if ((q & 31u) == 0) nz = more_than_combine(tok, q, nsrc);
+    if ((q & 31u) == 0) t.read(tok, q, nsrc);
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (q + u < nsrc) {
@@ -171,11 +260,11 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
     for (int u = 0; u < U; ++u)
       if (q + u < nsrc) {
         auto src = [&](int i) { return A::widen(x[u][i / N], i % N); };
-        if (!((nz >> ((q & 31u) + u)) & 1u)) {
+        if (t.plain(q + u)) {
           combine<FAM, V * N>(acc, src, dt, rop);
           continue;
         }
-        const uint32_t tk = __ldg(tok + q + u);
+        const uint32_t tk = t.at(q + u);
         if (tk & TOK_START) {
           if (tk & TOK_PUSH) {
 #pragma unroll
@@ -194,18 +283,9 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
             continue;
           }
           sp -= V * N;
-          const bool pop = (o & 3u) == TOK_POP;   // the saved value is the left operand
 #pragma unroll
-          for (int v = 0; v < V; ++v) {
-            uint32_t y[N];
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-              const uint32_t z = stack[(sp + v * N + i) * threads], w = acc[v * N + i];
-              acc[v * N + i] = pop ? z : w;
-              y[i] = pop ? w : z;
-            }
-            combine<FAM, N>(acc + v * N, [&](int i) { return y[i]; }, dt, rop);
-          }
+          for (int v = 0; v < V; ++v)
+            combine<FAM, N>(acc + v * N, [&](int i) { return stack[(sp + v * N + i) * threads]; }, dt, rop);
         }
       }
   }
@@ -221,8 +301,9 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
   }
 }
 
+// V vectors of the source at P[0] to the destinations P[d0 .. d1)
 template <int W, int V>
-__device__ __forceinline__ void copy_unit(const unsigned long long *__restrict__ P, uint32_t ndst,
+__device__ __forceinline__ void copy_unit(const unsigned long long *__restrict__ P, uint32_t d0, uint32_t d1,
                                           unsigned long long off, unsigned long long end) {
   Raw<W> r[V];
   bool on[V];
@@ -233,19 +314,136 @@ __device__ __forceinline__ void copy_unit(const unsigned long long *__restrict__
     if (on[v]) r[v] = ld_raw<W>(s + v * (32 * W));
   }
 #pragma unroll 4
-  for (uint32_t d = 0; d < ndst; ++d) {
-    const unsigned long long a = __ldg(P + 1 + d) + off;
+  for (uint32_t d = d0; d < d1; ++d) {
+    const unsigned long long a = __ldg(P + d) + off;
 #pragma unroll
     for (int v = 0; v < V; ++v)
       if (on[v]) st_raw<W>(a + v * (32 * W), r[v]);
   }
 }
 
+__device__ __forceinline__ void cp_async16(uint32_t dst, unsigned long long src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// pointer q of a list of n that the warp reads 32 at a time, lane i holding
+// the i-th of the block that q lies in; every lane takes part.  (The rings
+// leave so little L1 that a load per pointer goes to L2: 57 instead of 51 us
+// for a BF16 Reduce-scatter of 16 ranks x 16 MiB.)
+__device__ __forceinline__ unsigned long long pointer_at(const unsigned long long *P, uint32_t q, uint32_t n,
+                                                         unsigned long long &held) {
+  const uint32_t lane = threadIdx.x & 31;
+  if ((q & 31u) == 0) held = q + lane < n ? __ldg(P + q + lane) : 0ull;
+  return __shfl_sync(0xffffffffu, held, q & 31u);
+}
+
+// One unit of a fold of 16-byte vectors, one per lane at byte offset `off`.
+// Sources pass through a ring of G groups of RING_GROUP slots of the warp, an
+// asynchronous copy group each, so that G - 1 groups stay in flight without
+// registers for them.  (Waiting and committing takes about 250 cycles; per
+// source, not per group, it was most of the 366 a source took.)
+constexpr uint32_t RING_GROUP = 4;
+static_assert(32 % RING_GROUP == 0, "a group lies in one block of 32 sources");
+
+template <int FAM, int G>
+__device__ __forceinline__ void fold_ring(const SweepArgs &A, const Unit &u, unsigned long long off, bool on,
+                                          uint32_t dt, uint32_t rop, char *ring, uint4 *stack, uint32_t threads) {
+  using C = Acc<FAM, 16>;
+  constexpr int N = C::N;
+  const SweepClass &k = u.k;
+  const uint32_t *tok = A.toks + k.tok;
+  const uint32_t ring_at = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
+  unsigned long long held = 0;
+  uint32_t lq = 0;   // next source to load
+  auto load = [&](uint32_t g) {
+#pragma unroll
+    for (uint32_t i = 0; i < RING_GROUP; ++i)
+      if (lq + i < k.nsrc) {
+        const unsigned long long s = pointer_at(u.P, lq + i, k.nsrc, held) + off;
+        if (on) cp_async16(ring_at + (g * RING_GROUP + i) * 512, s);
+      }
+    lq += RING_GROUP;
+    cp_commit();
+  };
+#pragma unroll 1
+  for (uint32_t g = 0; g < G - 1; ++g) load(g);
+  uint32_t acc[N];
+  uint32_t sp = 0;   // saved values end here
+  Tokens t;
+  uint32_t g = 0;
+#pragma unroll 1
+  for (uint32_t q = 0; q < k.nsrc; q += RING_GROUP) {
+    if ((q & 31u) == 0) t.read(tok, q, k.nsrc);
+    cp_wait<G - 2>();
+    load(g == 0 ? G - 1 : g - 1);   // the group read last
+    Raw<16> x[RING_GROUP];
+#pragma unroll
+    for (uint32_t i = 0; i < RING_GROUP; ++i) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(ring + (g * RING_GROUP + i) * 512);
+      x[i].w[0] = v.x;
+      x[i].w[1] = v.y;
+      x[i].w[2] = v.z;
+      x[i].w[3] = v.w;
+    }
+    if (++g == G) g = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < RING_GROUP; ++i) {
+      auto src = [&](int j) { return C::widen(x[i], j); };
+      if (q + i >= k.nsrc) break;
+      if (t.plain(q + i)) {
+        combine<FAM, N>(acc, src, dt, rop);
+        continue;
+      }
+      const uint32_t tk = t.at(q + i);
+      if (tk & TOK_START) {
+        if (tk & TOK_PUSH) {
+#pragma unroll
+          for (int j = 0; j < N; j += 4, sp += threads)
+            stack[sp] = make_uint4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) acc[j] = src(j);
+      } else {
+        combine<FAM, N>(acc, src, dt, rop);
+      }
+      for (uint32_t o = tk >> TOK_OPS; o; o >>= 2) {
+        if ((o & 3u) == TOK_ROUND) {
+          C::round(acc);
+          continue;
+        }
+        sp -= threads * (N / 4);
+        uint32_t y[N];
+#pragma unroll
+        for (int j = 0; j < N; j += 4) {
+          const uint4 z = stack[sp + j / 4 * threads];
+          y[j] = z.x;
+          y[j + 1] = z.y;
+          y[j + 2] = z.z;
+          y[j + 3] = z.w;
+        }
+        combine<FAM, N>(acc, [&](int j) { return y[j]; }, dt, rop);
+      }
+    }
+  }
+  const Raw<16> r = C::pack(acc);
+#pragma unroll 4
+  for (uint32_t d = 0; d < k.ndst; ++d) {
+    const unsigned long long a = pointer_at(u.P + k.nsrc, d, k.ndst, held) + off;
+    if (on) st_raw<16>(a, r);
+  }
+}
+
 // the family's fold for a class of any payload but FP8
 template <int W, int V, int U>
 __device__ __forceinline__ void fold_any(const SweepArgs &A, const SweepClass &k, const unsigned long long *P,
-                                         unsigned long long off, unsigned long long end, uint32_t *stack) {
-  const uint32_t dt = sweep_dtype(k.meta), rop = sweep_rop(k.meta), threads = blockDim.x;
+                                         unsigned long long off, unsigned long long end, uint32_t *stack,
+                                         uint32_t threads) {
+  const uint32_t dt = sweep_dtype(k.meta), rop = sweep_rop(k.meta);
   const uint32_t *tok = A.toks + k.tok;
   if (dt == HICCL_BF16) {
     if (rop == HICCL_SUM) fold_unit<BF16_SUM, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
@@ -255,32 +453,6 @@ __device__ __forceinline__ void fold_any(const SweepArgs &A, const SweepClass &k
       fold_unit<F32_SUM, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
     else fold_unit<ANY_32, W, V, U>(P, tok, k.nsrc, k.ndst, off, end, dt, rop, stack, threads);
   }
-}
-
-// ---- units -----------------------------------------------------------------------
-
-// The class and member of a unit; operand pointers at P, the unit's index
-// inside the member in `part`.
-__device__ __forceinline__ SweepClass find_class(const SweepArgs &A, uint32_t unit, const unsigned long long *&P,
-                                                 uint32_t &part) {
-  uint32_t lo = 0, hi = A.nclass;
-  while (hi - lo > 1) {   // last class whose first unit is not past `unit`
-    const uint32_t mid = (lo + hi) >> 1;
-    const uint32_t u0 = A.nclass <= SWEEP_PREFIX ? A.unit0[mid] : __ldg(&A.classes[mid].unit0);
-    if (u0 <= unit) lo = mid;
-    else hi = mid;
-  }
-  SweepClass k;
-  {
-    const uint4 *q = reinterpret_cast<const uint4 *>(A.classes + lo);
-    uint4 *z = reinterpret_cast<uint4 *>(&k);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) z[i] = __ldg(q + i);
-  }
-  const uint32_t at = unit - k.unit0, mem = at / k.upm;
-  part = at - mem * k.upm;
-  P = A.ptrs + k.ptr + (unsigned long long)mem * (k.nsrc + k.ndst);
-  return k;
 }
 
 // Launches overlap the previous kernel's tail: the next kernel's CTAs may
@@ -311,50 +483,58 @@ __device__ __forceinline__ unsigned long long edge_of(const SweepClass &k, const
 }
 
 // a copy's unit, and with the last one the member's edges
-__device__ __forceinline__ void copy_member(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
+__device__ __forceinline__ void copy_member(const Unit &u, int lane) {
+  const SweepClass &k = u.k;
   const uint32_t v = sweep_v(k.meta);
-  const Body b = body_of(k, P);
-  const unsigned long long off = b.head + (unsigned long long)part * 512 * v + lane * 16;
-  if (v == 4) copy_unit<16, 4>(P, k.ndst, off, b.end);
-  else if (v == 2) copy_unit<16, 2>(P, k.ndst, off, b.end);
-  else copy_unit<16, 1>(P, k.ndst, off, b.end);
-  if (part + 1 == k.upm && b.end - b.head != k.nbytes) copy_unit<2, 1>(P, k.ndst, edge_of<2>(k, b, lane), k.nbytes);
+  const Body b = body_of(k, u.P);
+  const unsigned long long off = b.head + (unsigned long long)u.part * 512 * v + lane * 16;
+  if (v == 4) copy_unit<16, 4>(u.P, u.d0, u.d1, off, b.end);
+  else if (v == 2) copy_unit<16, 2>(u.P, u.d0, u.d1, off, b.end);
+  else copy_unit<16, 1>(u.P, u.d0, u.d1, off, b.end);
+  if (u.part + 1 == k.upm && b.end - b.head != k.nbytes)
+    copy_unit<2, 1>(u.P, u.d0, u.d1, edge_of<2>(k, b, lane), k.nbytes);
 }
 
-// V vectors a lane in flight, stored to every destination
+// V vectors a lane in flight, stored to a group of destinations
 __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_COPY], 8) sweep_copy_kernel(const __grid_constant__ SweepArgs A) {
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (unit >= A.units) return;
-  const unsigned long long *P;
-  uint32_t part;
-  const SweepClass k = find_class(A, unit, P, part);
-  copy_member(k, P, part, threadIdx.x & 31);
+  copy_member(find_unit(A, unit), threadIdx.x & 31);
 }
 
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FOLD], 8) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
-  extern __shared__ uint32_t saved[];
+template <int G>
+__device__ __forceinline__ void fold_member(const SweepArgs &A, const Unit &u, int lane) {
+  extern __shared__ __align__(16) uint32_t saved[];
+  const SweepClass &k = u.k;
+  const uint32_t dt = sweep_dtype(k.meta), rop = sweep_rop(k.meta), threads = blockDim.x;
+  char *ring = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (G * RING_GROUP * 512) + lane * 16;
+  uint4 *stack = reinterpret_cast<uint4 *>(saved) + (threads >> 5) * (G * RING_GROUP * 32) + threadIdx.x;   // saved values
+  const Body b = body_of(k, u.P);
+  const unsigned long long off = b.head + (unsigned long long)u.part * 512 + lane * 16;
+  const bool on = off + 16 <= b.end;
+  if (dt == HICCL_BF16) {
+    if (rop == HICCL_SUM) fold_ring<BF16_SUM, G>(A, u, off, on, dt, rop, ring, stack, threads);
+    else fold_ring<BF16_ANY, G>(A, u, off, on, dt, rop, ring, stack, threads);
+  } else {
+    if (dt == HICCL_F32 && rop == HICCL_SUM) fold_ring<F32_SUM, G>(A, u, off, on, dt, rop, ring, stack, threads);
+    else fold_ring<ANY_32, G>(A, u, off, on, dt, rop, ring, stack, threads);
+  }
+  if (u.part + 1 == k.upm && b.end - b.head != k.nbytes) {
+    uint32_t *words = reinterpret_cast<uint32_t *>(stack);   // one of each of this thread's own vectors
+    if (dt == HICCL_BF16) fold_any<2, 1, 8>(A, k, u.P, edge_of<2>(k, b, lane), k.nbytes, words, 4 * threads);
+    else fold_any<4, 1, 8>(A, k, u.P, edge_of<4>(k, b, lane), k.nbytes, words, 4 * threads);
+  }
+}
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FOLD], 16) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (unit >= A.units) return;
-  const unsigned long long *P;
-  uint32_t part;
-  const SweepClass k = find_class(A, unit, P, part);
-  if (k.nsrc == 1) {
-    copy_member(k, P, part, lane);
-    return;
-  }
-  uint32_t *stack = saved + threadIdx.x;
-  const uint32_t v = sweep_v(k.meta);
-  const Body b = body_of(k, P);
-  const unsigned long long off = b.head + (unsigned long long)part * 512 * v + lane * 16;
-  if (v == 2) fold_any<16, 2, 8>(A, k, P, off, b.end, stack);
-  else fold_any<16, 1, 16>(A, k, P, off, b.end, stack);
-  if (part + 1 == k.upm && b.end - b.head != k.nbytes) {
-    if (sweep_dtype(k.meta) == HICCL_BF16) fold_any<2, 1, 8>(A, k, P, edge_of<2>(k, b, lane), k.nbytes, stack);
-    else fold_any<4, 1, 8>(A, k, P, edge_of<4>(k, b, lane), k.nbytes, stack);
-  }
+  const Unit u = find_unit(A, unit);
+  if (u.k.nsrc == 1) copy_member(u, lane);
+  else if (A.groups == FOLD_GROUPS) fold_member<FOLD_GROUPS>(A, u, lane);
+  else fold_member<FOLD_GROUPS_SHORT>(A, u, lane);
 }
 
 // folds of operands that lie differently off a 16-byte boundary: W-byte
@@ -365,9 +545,9 @@ __device__ __forceinline__ void narrow_unit(const SweepArgs &A, const SweepClass
                                             uint32_t part, int lane, uint32_t *stack) {
   const uint32_t v = sweep_v(k.meta);
   const unsigned long long off = (unsigned long long)part * (32 * W) * v + lane * W;
-  if (v == 8) fold_any<W, 8, 4>(A, k, P, off, k.nbytes, stack);
-  else if (v == 2) fold_any<W, 2, 8>(A, k, P, off, k.nbytes, stack);
-  else fold_any<W, 1, 16>(A, k, P, off, k.nbytes, stack);
+  if (v == 8) fold_any<W, 8, 4>(A, k, P, off, k.nbytes, stack, blockDim.x);
+  else if (v == 2) fold_any<W, 2, 8>(A, k, P, off, k.nbytes, stack, blockDim.x);
+  else fold_any<W, 1, 16>(A, k, P, off, k.nbytes, stack, blockDim.x);
 }
 __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_NARROW], 10) sweep_narrow_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ uint32_t saved[];
@@ -375,9 +555,10 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_NARROW], 10) sweep_narrow_
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (unit >= A.units) return;
-  const unsigned long long *P;
-  uint32_t part;
-  const SweepClass k = find_class(A, unit, P, part);
+  const Unit u = find_unit(A, unit);
+  const SweepClass &k = u.k;
+  const unsigned long long *P = u.P;
+  const uint32_t part = u.part;
   if (sweep_lw(k.meta) == 2) narrow_unit<4>(A, k, P, part, lane, saved + threadIdx.x);
   else narrow_unit<2>(A, k, P, part, lane, saved + threadIdx.x);
 }
@@ -413,7 +594,10 @@ __device__ __forceinline__ uint4 shift_pair(const uint4 &a, const uint4 &b, uint
   return r;
 }
 template <int V>
-__device__ __forceinline__ void shift_unit(const SweepClass &k, const unsigned long long *P, uint32_t part, int lane) {
+__device__ __forceinline__ void shift_unit(const Unit &u, int lane) {
+  const SweepClass &k = u.k;
+  const unsigned long long *P = u.P;
+  const uint32_t part = u.part;
   const unsigned long long src = __ldg(P), n = k.nbytes;
   const unsigned long long o0 = (0ull - src) & 15u;           // first whole vector of the source
   const unsigned long long last = o0 + 16 <= n ? o0 + ((n - o0 - 16) & ~15ull) : 0ull;   // the last one
@@ -439,8 +623,8 @@ __device__ __forceinline__ void shift_unit(const SweepClass &k, const unsigned l
   const unsigned long long at = lane < 16 ? 2ull * lane : (any ? last + 2ull * (lane - 16) : 32 + 2ull * (lane - 16));
   unsigned short ev = 0;
   if (edges && at < n) ev = __ldcg(reinterpret_cast<const unsigned short *>(src + at));
-  for (uint32_t d = 0; d < k.ndst; ++d) {
-    const unsigned long long dst = __ldg(P + 1 + d);
+  for (uint32_t d = u.d0; d < u.d1; ++d) {
+    const unsigned long long dst = __ldg(P + d);
     const uint32_t e = (uint32_t)((0ull - (dst + o0)) & 15u);   // from a source vector to the destination's
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -455,11 +639,9 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_SHIFT], 8) sweep_shift_ker
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (unit >= A.units) return;
-  const unsigned long long *P;
-  uint32_t part;
-  const SweepClass k = find_class(A, unit, P, part);
-  if (sweep_v(k.meta) == 4) shift_unit<4>(k, P, part, threadIdx.x & 31);
-  else shift_unit<1>(k, P, part, threadIdx.x & 31);
+  const Unit u = find_unit(A, unit);
+  if (sweep_v(u.k.meta) == 4) shift_unit<4>(u, threadIdx.x & 31);
+  else shift_unit<1>(u, threadIdx.x & 31);
 }
 
 // ---- FP8 blocks --------------------------------------------------------------------
@@ -471,20 +653,6 @@ struct Fp8Raw {
   float scale;
 };
 
-// two binary32 values in one 64-bit register pair
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-  unsigned long long d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-  return d;
-}
-__device__ __forceinline__ void unpack2(unsigned long long d, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(d));
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 // rounded products: fma with -0, which a kernel argument supplies so that the
 // product is not contracted into the add that follows it
 __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b,
@@ -531,95 +699,91 @@ __device__ __forceinline__ Fp8Raw fp8_encode(const unsigned long long *v) {
   return r;
 }
 
-constexpr int FP8_SLOTS = 8;                                    // sources a warp keeps in flight
+constexpr int FP8_GROUPS = 2;                                   // of the ring of an FP8 fold
+constexpr uint32_t FP8_SLOTS = FP8_GROUPS * RING_GROUP;
 constexpr uint32_t FP8_STEP = 4 * FP8_BLOCK_BYTES;              // bytes of a source in one slot
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, unsigned long long src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 // A unit is four blocks, 576 bytes of every operand.  A source takes about 100
 // instructions, so a warp is busy while its loads should fly; they
-// pass through a ring of slots in shared memory, one asynchronous copy group
-// a source, which keeps FP8_SLOTS - 1 in flight through folds, encodings and
-// stores without holding registers (72 a thread, 24 warps an SM).  Copies and
+// pass through a ring of slots in shared memory, an asynchronous copy group
+// for every RING_GROUP sources, which keeps loads in flight through folds,
+// encodings and stores without holding registers (72 a thread, 24 warps an SM).  Copies and
 // stores move the unit as one range of whole sectors, and only the fold reads
 // it by blocks.  All-reduce of 16 Mi values a rank over 32 ranks ({4, 8}),
 // 1.21 GB in and out: 265 us with the next sources loaded into registers (16
 // warps an SM; 403 us when refilled one by one), 223 us through the ring by
-// blocks, 199 us by the unit's range, 6.1 TB/s; two or four units a warp
-// lose 5 and 10 %, neighbouring warps on neighbouring units read longer
-// stretches of each source at a time.
+// blocks, 199 us by the unit's range, 186 us (6.5 TB/s) with copy groups of
+// four sources; two or four units a warp lose 5 and 10 %, neighbouring warps
+// on neighbouring units read longer stretches of each source at a time.
 __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ __align__(16) uint32_t saved[];
   launch_order();
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (unit >= A.units) return;
-  const unsigned long long *P;
-  uint32_t part;
-  const SweepClass k = find_class(A, unit, P, part);
+  const Unit u = find_unit(A, unit);
+  const SweepClass &k = u.k;
+  const unsigned long long *P = u.P;
+  const uint32_t part = u.part;
   const uint32_t *tok = A.toks + k.tok;
   const uint32_t threads = blockDim.x, sub = lane & 7;
   const unsigned long long minus0 = A.minus0;
   char *ring = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (FP8_SLOTS * FP8_STEP);
   char *mine = ring + (lane >> 3) * FP8_BLOCK_BYTES;   // this group's block in slot 0
   const uint32_t ring_at = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + 16 * lane;
-  float *stack = reinterpret_cast<float *>(saved) + (threads >> 5) * (FP8_SLOTS * FP8_STEP / 4) + threadIdx.x;
+  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + (threads >> 5) * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
 
   // this lane's 16 bytes of the unit, and (lanes 0 .. 3) 16 of its last 64
   const unsigned long long off = (unsigned long long)part * FP8_STEP + 16 * lane;
   const bool on = off < k.nbytes, on2 = lane < 4 && off + 512 < k.nbytes;
-  unsigned long long lptr = __ldg(P);   // of source lq
-  uint32_t lq = 0;
-  auto load = [&](int slot) {
-    if (lq < k.nsrc) {
-      const unsigned long long s = lptr + off;
-      if (on) cp_async16(ring_at + slot * FP8_STEP, s);
-      if (on2) cp_async16(ring_at + slot * FP8_STEP + 512, s + 512);
-      if (++lq < k.nsrc) lptr = __ldg(P + lq);
-    }
+  unsigned long long held = 0;
+  uint32_t lq = 0;   // next source to load
+  auto load = [&](uint32_t g) {
+#pragma unroll
+    for (uint32_t i = 0; i < RING_GROUP; ++i)
+      if (lq + i < k.nsrc) {
+        const unsigned long long s = pointer_at(P, lq + i, k.nsrc, held) + off;
+        const uint32_t to = ring_at + (g * RING_GROUP + i) * FP8_STEP;
+        if (on) cp_async16(to, s);
+        if (on2) cp_async16(to + 512, s + 512);
+      }
+    lq += RING_GROUP;
     cp_commit();
   };
-#pragma unroll
-  for (int u = 0; u < FP8_SLOTS - 1; ++u) load(u);
+#pragma unroll 1
+  for (uint32_t g = 0; g < FP8_GROUPS - 1; ++g) load(g);
   unsigned long long acc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0ull;
-  uint32_t sp = 0, nz = 0;   // words saved; which of 32 tokens do more than combine
-  uint32_t slot = 0;
+  uint32_t sp = 0;   // saved values end here
+  Tokens t;
+  uint32_t g = 0, slot = 0;
+#pragma unroll 1
   for (uint32_t q = 0; q < k.nsrc; ++q) {
-    if ((q & 31u) == 0) nz = more_than_combine(tok, q, k.nsrc);
-    cp_wait<FP8_SLOTS - 2>();
-    __syncwarp();              // every lane's copies have landed, and the slot read last is free
-    load((slot + FP8_SLOTS - 1) % FP8_SLOTS);
+    if ((q & 31u) == 0) t.read(tok, q, k.nsrc);
+    if (q % RING_GROUP == 0) {
+      cp_wait<FP8_GROUPS - 2>();
+      __syncwarp();            // every lane's copies have landed, and the group read last is free
+      load(g == 0 ? FP8_GROUPS - 1 : g - 1);
+      slot = g * RING_GROUP;
+      if (++g == FP8_GROUPS) g = 0;
+    }
     Fp8Raw x;
     x.c = *reinterpret_cast<const uint4 *>(mine + slot * FP8_STEP + 16 * sub);
     x.scale = *reinterpret_cast<const float *>(mine + slot * FP8_STEP + 128);
-    slot = (slot + 1) % FP8_SLOTS;
+    ++slot;
     unsigned long long y[8];
     fp8_widen(x, minus0, y);
-    if (!((nz >> (q & 31u)) & 1u)) {
+    if (t.plain(q)) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) acc[i] = add2(acc[i], y[i]);
       continue;
     }
-    const uint32_t tk = __ldg(tok + q);
+    const uint32_t tk = t.at(q);
     if (tk & TOK_START) {
       if (tk & TOK_PUSH) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float lo, hi;
-          unpack2(acc[i], lo, hi);
-          stack[(sp + 2 * i) * threads] = lo;
-          stack[(sp + 2 * i + 1) * threads] = hi;
-        }
-        sp += 16;
+        for (int i = 0; i < 8; i += 2, sp += threads) stack[sp] = make_ulonglong2(acc[i], acc[i + 1]);
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) acc[i] = y[i];
@@ -631,11 +795,12 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(
       if ((o & 3u) == TOK_ROUND) {
         fp8_widen(fp8_encode(acc), minus0, acc);
       } else {
-        sp -= 16;
+        sp -= 4 * threads;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {   // (a sum of two is the same in both orders)
-          const float lo = stack[(sp + 2 * i) * threads], hi = stack[(sp + 2 * i + 1) * threads];
-          acc[i] = add2(pack2(lo, hi), acc[i]);
+        for (int i = 0; i < 8; i += 2) {
+          const ulonglong2 z = stack[sp + i / 2 * threads];
+          acc[i] = add2(z.x, acc[i]);
+          acc[i + 1] = add2(z.y, acc[i + 1]);
         }
       }
     }
@@ -682,6 +847,11 @@ cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_
   cfg.blockDim = dim3(L.threads);
   cfg.dynamicSmemBytes = (size_t)L.stack_words * 4 * L.threads;
   if (L.kernel == SWEEP_FP8) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;
+  SweepArgs B = A;
+  if (L.kernel == SWEEP_FOLD) {
+    B.groups = L.units < SHORT_UNITS ? FOLD_GROUPS_SHORT : FOLD_GROUPS;
+    cfg.dynamicSmemBytes += warps * B.groups * RING_GROUP * 512;
+  }
   if (one_per_sm && cfg.dynamicSmemBytes < SWEEP_HALF_SM) cfg.dynamicSmemBytes = SWEEP_HALF_SM;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -689,7 +859,7 @@ cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, KERNELS[L.kernel], A);
+  return cudaLaunchKernelEx(&cfg, KERNELS[L.kernel], B);
 }
 
 }  // namespace hiccl

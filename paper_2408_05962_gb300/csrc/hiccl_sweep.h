@@ -13,8 +13,10 @@ struct SweepArgs {
   const unsigned long long *ptrs;
   uint32_t nclass;
   uint32_t units;
+  uint32_t groups = 0;                  // of a fold's ring
   unsigned long long minus0 = 0x8000000080000000ull;   // two binary32 -0 (see mul2)
   uint32_t unit0[SWEEP_PREFIX];         // first units, for searching without a memory access
+  SweepClass first[SWEEP_INLINE];       // the classes themselves, where there are few
 };
 
 cudaError_t sweep_prepare();            // once per device, with it current

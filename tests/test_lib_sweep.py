@@ -31,7 +31,7 @@ def decode(blob):
     """(classes, launches, pointers, tokens) of a sweep's inspection blob."""
     nc, nl, npt, nt = struct.unpack_from("<4Q", blob, 0)
     o = 32
-    cls = [dict(zip(("nbytes", "ptr", "unit0", "upm", "nmem", "nsrc", "ndst", "tok", "meta", "_"),
+    cls = [dict(zip(("nbytes", "ptr", "unit0", "upm", "nmem", "nsrc", "ndst", "tok", "meta", "group"),
                     struct.unpack_from("<2Q8I", blob, o + 48 * k))) for k in range(nc)]
     o += 48 * nc
     lau = [dict(zip(("kernel", "lo", "hi", "units", "threads", "words"), struct.unpack_from("<6I", blob, o + 24 * k)))
@@ -96,7 +96,8 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
             unit = {FP8: 4 * 144, SHIFT: 31 * 16}.get(L["kernel"], 32 * c["width"]) * c["v"]
             assert (c["upm"] - 1) * unit < c["nbytes"] <= c["upm"] * unit        # units tile a member
             assert c["v"] in (1, 2, 4, 8, 16)
-            units += c["upm"] * c["nmem"]
+            assert c["group"] == (c["ndst"] if c["nsrc"] > 1 else 2)
+            units += c["upm"] * c["nmem"] * -(-c["ndst"] // c["group"])
             for i in range(c["nmem"]):
                 p = ptrs[c["ptr"] + i * (c["nsrc"] + c["ndst"]):][:c["nsrc"] + c["ndst"]]
                 assert all((a - p[0]) % c["width"] == 0 for a in p) and (c["width"] == 16 or p[0] % c["width"] == 0)
