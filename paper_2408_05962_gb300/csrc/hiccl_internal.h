@@ -170,12 +170,13 @@ enum : uint32_t {
   SWEEP_KERNELS = 5
 };
 // A copy's destinations are stored in groups of SWEEP_GROUP, group after group
-// over SWEEP_TILE / (vectors per lane) units of source (16 MiB, which stay in
+// over SWEEP_TILE / (vectors per lane) units of source (4 MiB, which stay in
 // L2 between the groups): few, long streams of writes instead of one per
 // destination.  Measured, 4 MiB to 64 destinations in turn over three sets of
 // buffers: all 64 a unit 54 us, 16 44 us, 8 43 us, 4 40.7 us, 2 38.0 us
-// (7.2 TB/s), 1 40.4 us.
-constexpr uint32_t SWEEP_GROUP = 2, SWEEP_TILE = 32768;
+// (7.2 TB/s), 1 40.4 us.  16 MiB to 16 destinations by tiles of 1 / 2 / 4 / 8 /
+// 16 MiB: 43.1 / 42.5 / 41.2 / 42.4 / 45.9 us.
+constexpr uint32_t SWEEP_GROUP = 2, SWEEP_TILE = 8192;
 constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128};   // most threads of a CTA
 
 // token of one source, in evaluation order: START the accumulator with it

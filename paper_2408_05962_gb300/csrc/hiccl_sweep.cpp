@@ -184,20 +184,21 @@ struct TouchIndex {
 
 // Width of the accesses that every operand of a member allows: 16 bytes when
 // all lie equally far off a 16-byte boundary (whole vectors between a few
-// elements at both ends), else the widest of 4 and 2 that the addresses (and
-// the length) share.
+// elements at both ends), told as 32 when they lie equally far off a 32-byte
+// sector (the vectors then start with one), else the widest of 4 and 2 that
+// the addresses (and the length) share.
 uint32_t width_log2(const Member &m) {
   unsigned long long a = 0, off = 0;
   for (unsigned long long v : m.src) a |= v, off |= v ^ m.src[0];
   for (unsigned long long v : m.dst) a |= v, off |= v ^ m.src[0];
-  if (off % 16 == 0) return 4;
+  if (off % 16 == 0) return off % 32 == 0 ? 5 : 4;
   return a % 4 == 0 && m.nbytes % 4 == 0 ? 2 : 1;
 }
 
 // bytes of a member that a warp moves with one vector per lane
 unsigned long long row_bytes(uint32_t kern, const SweepClass &k) {
   if (kern == SWEEP_FP8) return 4 * FP8_BLOCK_BYTES;
-  return kern == SWEEP_SHIFT ? 31 * 16 : 32ull << sweep_lw(k.meta);
+  return kern == SWEEP_SHIFT ? 31 * 16 : 32ull << std::min(sweep_lw(k.meta), 4u);
 }
 
 // units that store one range of a member to all its destinations
@@ -208,9 +209,9 @@ unsigned long long groups(const SweepClass &k) {
 // Launches, vectors per lane and units of a sweep's classes.
 void plan_launches(Sweep &sw) {
   bool folds = false;
-  for (const SweepClass &k : sw.classes) folds |= k.nsrc > 1 && sweep_lw(k.meta) == 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
+  for (const SweepClass &k : sw.classes) folds |= k.nsrc > 1 && sweep_lw(k.meta) >= 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
   auto kernel_of = [&](const SweepClass &k) -> uint32_t {
-    if (sweep_lw(k.meta) != 4) return k.nsrc > 1 ? SWEEP_NARROW : SWEEP_SHIFT;
+    if (sweep_lw(k.meta) < 4) return k.nsrc > 1 ? SWEEP_NARROW : SWEEP_SHIFT;
     if (k.nsrc > 1 && sweep_dtype(k.meta) == HICCL_FP8E4M3) return SWEEP_FP8;
     return k.nsrc > 1 || folds ? SWEEP_FOLD : SWEEP_COPY;
   };
@@ -247,7 +248,7 @@ void plan_launches(Sweep &sw) {
         return;
       }
       // accumulator words of a lane: 32-bit values, or BF16 / FP8 values widened to 32 bits
-      const uint32_t acc = kern == SWEEP_FP8 ? 16 : lw == 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
+      const uint32_t acc = kern == SWEEP_FP8 ? 16 : lw >= 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
       if (k.nsrc > 1) words = std::max(words, sw.depth * acc * v);
     }
     SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words};

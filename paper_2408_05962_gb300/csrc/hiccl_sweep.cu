@@ -464,15 +464,17 @@ __device__ __forceinline__ void launch_order() {
 }
 
 // Where the whole 16-byte vectors of a member lie: all its operands are
-// equally far off a boundary, so they start at byte `head` and end at `end`
-// of each; the elements before and after are at most 14 + 14 bytes.  (Rows of
+// equally far off a boundary (of 32 bytes where they agree that far, so that no
+// sector is written by two warps), so they start at byte `head` and end at
+// `end` of each; the elements before and after are at most 30 + 14 bytes.  (Rows of
 // a multiple of 16 bytes with odd chunk lengths are such operands: an odd
-// 6 MiB All-reduce over 16 ranks takes 38 us, 55 us by 4-byte accesses.)
+// 6 MiB All-reduce over 16 ranks takes 36 us, 38 us from 16-byte boundaries
+// and 55 us by 4-byte accesses.)
 struct Body {
   unsigned long long head, end;
 };
 __device__ __forceinline__ Body body_of(const SweepClass &k, const unsigned long long *P) {
-  const unsigned long long h = min((0ull - __ldg(P)) & 15u, k.nbytes);
+  const unsigned long long h = min((0ull - __ldg(P)) & ((1u << sweep_lw(k.meta)) - 1u), k.nbytes);
   return Body{h, h + ((k.nbytes - h) & ~15ull)};
 }
 // byte offset of this lane's element of W bytes outside the body (nbytes: none)

@@ -93,14 +93,14 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         units = 0
         for c in cls[L["lo"]:L["hi"]]:
             assert c["kernel"] == L["kernel"] and c["unit0"] == units
-            unit = {FP8: 4 * 144, SHIFT: 31 * 16}.get(L["kernel"], 32 * c["width"]) * c["v"]
+            unit = {FP8: 4 * 144, SHIFT: 31 * 16}.get(L["kernel"], 32 * min(c["width"], 16)) * c["v"]
             assert (c["upm"] - 1) * unit < c["nbytes"] <= c["upm"] * unit        # units tile a member
             assert c["v"] in (1, 2, 4, 8, 16)
             assert c["group"] == (c["ndst"] if c["nsrc"] > 1 else 2)
             units += c["upm"] * c["nmem"] * -(-c["ndst"] // c["group"])
             for i in range(c["nmem"]):
                 p = ptrs[c["ptr"] + i * (c["nsrc"] + c["ndst"]):][:c["nsrc"] + c["ndst"]]
-                assert all((a - p[0]) % c["width"] == 0 for a in p) and (c["width"] == 16 or p[0] % c["width"] == 0)
+                assert all((a - p[0]) % c["width"] == 0 for a in p) and (c["width"] >= 16 or p[0] % c["width"] == 0)
                 assert (L["kernel"] in (NARROW, SHIFT)) == (c["width"] < 16)
                 assert L["kernel"] == FOLD or (c["nsrc"] > 1) == (L["kernel"] in (FP8, NARROW))
                 members.append((c, p))
@@ -112,7 +112,7 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         out = vals[0]
         if c["nsrc"] > 1:
             out, most = evaluate(vals, toks[c["tok"]:c["tok"] + c["nsrc"]], H.OP_NAMES[c["rop"]], dtype)
-            acc = 16 if dtype == "fp8" else (c["width"] // 2 if dtype == "bf16" else c["width"] // 4)
+            acc = 16 if dtype == "fp8" else (min(c["width"], 16) // (2 if dtype == "bf16" else 4))
             L = next(x for x in lau if x["kernel"] == c["kernel"])
             assert most * max(acc, 1) * c["v"] <= L["words"]   # saved values fit
         for a in p[c["nsrc"]:]:
