@@ -167,15 +167,34 @@ def _check(comm, st: int):
         raise HicclError(st, msg)
 
 
+_raw_stream = None      # device index -> handle of PyTorch's current stream, once known to work
+
+
+def _current_stream() -> int | None:
+    """Handle of PyTorch's current stream on the current device (None without
+    CUDA).  Looking it up as a number takes 0.2 us where building the Stream
+    object takes 3.8, a quarter of a small collective's start and wait."""
+    global _raw_stream
+    import torch
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch._C._cuda_getDevice())
+    if not torch.cuda.is_available():
+        return None
+    handle = int(torch.cuda.current_stream().cuda_stream)
+    try:
+        if torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) == handle:
+            _raw_stream = torch._C._cuda_getCurrentRawStream
+    except AttributeError:
+        pass
+    return handle
+
+
 def _stream_handle(stream) -> int | None:
     if stream is None:
         try:
-            import torch
-            if torch.cuda.is_available():
-                return int(torch.cuda.current_stream().cuda_stream)
+            return _current_stream()
         except Exception:
-            pass
-        return None
+            return None
     if isinstance(stream, int):
         return stream
     return int(stream.cuda_stream)

@@ -124,6 +124,30 @@ def test_step_executor(name, dtype, d, mis):
             assert_bit_equal(ref, out)
 
 
+def test_current_stream_of_a_start():
+    """A start without a stream goes to PyTorch's current one, as it changes."""
+    import torch
+    from paper_2408_05962_gb300 import hiccl as H
+    streams = [torch.cuda.default_stream(), torch.cuda.Stream(), torch.cuda.Stream(priority=-1)]
+    for s in streams + streams:
+        with torch.cuda.stream(s):
+            assert H._stream_handle(None) == torch.cuda.current_stream().cuda_stream == s.cuda_stream
+    b = _buffers("allreduce", 8, 50000, "f32", 3)
+    c = H.Comm(8, "f32")
+    c.add_collective("allreduce", 50000, b.send_ptrs(), b.recv_ptrs())
+    c.init([2, 4], 1, 1)
+    c.start()
+    c.wait()
+    want = b.recv.clone()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(streams[1]):
+        torch.cuda._sleep(20_000_000)                      # the fill is still queued when the start is issued
+        b.recv.zero_()
+        c.start()
+        c.wait()
+    assert torch.equal(b.recv, want)
+
+
 def test_sweep_replayed_and_restarted():
     """Captured starts of two communicators on forked streams, replayed beside
     direct starts; one CTA per SM (CTAS_PER_SM = 1) gives the same result."""
