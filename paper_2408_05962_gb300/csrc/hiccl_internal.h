@@ -167,7 +167,8 @@ enum : uint32_t {
   SWEEP_FP8 = 2,      // folds of FP8 blocks
   SWEEP_NARROW = 3,   // folds of other operands: 4- or 2-byte accesses
   SWEEP_SHIFT = 4,    // copies of other operands: vectors shifted in registers
-  SWEEP_KERNELS = 5
+  SWEEP_TEAM = 5,     // folds as SWEEP_FOLD's, a CTA to a unit
+  SWEEP_KERNELS = 6
 };
 // A copy's destinations are stored in groups of SWEEP_GROUP, group after group
 // over SWEEP_TILE / (vectors per lane) units of source (4 MiB, which stay in
@@ -177,7 +178,16 @@ enum : uint32_t {
 // (7.2 TB/s), 1 40.4 us.  16 MiB to 16 destinations by tiles of 1 / 2 / 4 / 8 /
 // 16 MiB: 43.1 / 42.5 / 41.2 / 42.4 / 45.9 us.
 constexpr uint32_t SWEEP_GROUP = 2, SWEEP_TILE = 8192;
-constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128};   // most threads of a CTA
+constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128, 512};   // most threads of a CTA
+
+constexpr uint32_t SWEEP_TEAM_MAX = 32;    // sections of an expression
+// In a fold pass of few units every warp folds one source after the other,
+// about 300 cycles each, while most of an SM idles: below eight units an SM
+// the sections go to the warps of a CTA, as many as fill the SMs
+// (SWEEP_TEAM_WARPS in all).  Measured without / with, All-reduce of 64 ranks
+// x 64 KiB 12.7 / 9.4 us, Reduce of 64 ranks x 16 KiB 10.8 / 6.1 us; at 1024
+// units (16 ranks x 512 KiB) 7.3 / 5.2 us, at 2048 (1 MiB) 8.6 / 10.6 us.
+constexpr uint32_t SWEEP_TEAM_UNITS = 152 * 8, SWEEP_TEAM_WARPS = 152 * 32;
 
 // token of one source, in evaluation order: START the accumulator with it
 // (first saving the old one when PUSH is set), else combine it; then up to
@@ -201,8 +211,14 @@ struct SweepClass {
   uint32_t tok;                // first of the nsrc tokens
   uint32_t meta;               // sweep_meta
   uint32_t group;              // destinations that one unit stores (copies; folds store all)
+  // an expression in two steps (team > 1): `team` sections of consecutive
+  // sources, evaluated apart, then an expression of their values.  From token
+  // ttok: the sections' nsrc tokens, their team + 1 bounds, team tokens.
+  uint32_t team;
+  uint32_t ttok;
+  uint32_t pad[2];
 };
-static_assert(sizeof(SweepClass) == 48, "class layout");
+static_assert(sizeof(SweepClass) == 64, "class layout");
 // dtype (4 bits) | operator (3) | log2 of the access width (3) | vectors per lane (5) | kernel (3)
 HICCL_HD inline uint32_t sweep_meta(uint32_t dt, uint32_t rop, uint32_t lw, uint32_t v, uint32_t kern) {
   return dt | (rop << 4) | (lw << 7) | (v << 10) | (kern << 15);

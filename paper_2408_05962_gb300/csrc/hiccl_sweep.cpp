@@ -55,10 +55,11 @@ struct Expr {
     toks.back() |= o << (TOK_OPS + 2 * nops.back()++);
   }
   // ends of the level-l subgroups inside leaves[lo, hi)
-  size_t next(size_t lo, size_t hi, int l) const {
-    const long long q = leaves[lo] / G[l + 1];
+  size_t next(size_t lo, size_t hi, int l) const { return next_in(leaves, lo, hi, l); }
+  size_t next_in(const std::vector<int> &v, size_t lo, size_t hi, int l) const {
+    const long long q = v[lo] / G[l + 1];
     size_t k = lo + 1;
-    while (k < hi && leaves[k] / G[l + 1] == q) ++k;
+    while (k < hi && v[k] / G[l + 1] == q) ++k;
     return k;
   }
   // the value of a group: the left fold of its non-empty subgroups'
@@ -135,15 +136,69 @@ struct Expr {
 struct Program {   // an expression shared by members: evaluation order and tokens
   std::vector<int> leaves;
   long long node;  // the chain's first node (-1: tree)
-  bool rounds;
+  bool rounds, exact;
   std::vector<int> order;
-  uint32_t tok;
+  uint32_t tok, team, ttok;
 };
+
+// The two-step form of a program's expression (see SweepClass::team): the
+// groups of the level that makes a section and the list of sections shortest
+// together, or equal parts where the operator is exact (the order of exact
+// operations does not change the result).  Returns the number of sections (0: none) and
+// appends their tokens, bounds and the tokens of their values.
+uint32_t two_steps(const std::vector<int> &h, const std::vector<int> &leaves, bool rounds, bool exact, bool chained,
+                   std::vector<uint32_t> &toks, uint32_t &depth) {
+  const uint32_t n = (uint32_t)leaves.size();
+  if (n < 8 || (chained && !exact)) return 0;
+  std::vector<uint32_t> lower, bounds, upper;
+  if (exact) {
+    uint32_t T = 2;
+    while (T < SWEEP_TEAM_MAX && (T + 1) * (T + 1) <= n) ++T;
+    for (uint32_t s = 0; s <= T; ++s) bounds.push_back((uint32_t)((unsigned long long)n * s / T));
+    lower.assign(n, 0);
+    for (uint32_t s = 0; s < T; ++s) lower[bounds[s]] = TOK_START;
+    upper.assign(T, 0);
+    upper[0] = TOK_START;
+  } else {
+    std::vector<int> reps;
+    Expr top(h, reps, rounds);
+    int level = -1;
+    for (int l = 0; l < (int)h.size(); ++l) {
+      std::vector<uint32_t> b;
+      for (size_t a = 0; a < n; a = top.next_in(leaves, a, n, l)) b.push_back((uint32_t)a);
+      if (b.size() > SWEEP_TEAM_MAX || b.size() == n) break;
+      if (b.size() < 2) continue;
+      if (level >= 0 && n / b.size() + b.size() >= n / bounds.size() + bounds.size()) continue;
+      level = l;
+      bounds = b;
+    }
+    if (level < 0) return 0;
+    for (uint32_t a : bounds) reps.push_back(leaves[a]);
+    bounds.push_back(n);
+    for (size_t s = 0; s + 1 < bounds.size(); ++s) {
+      Expr e(h, leaves, rounds);
+      e.group(bounds[s], bounds[s + 1], level + 1, false);
+      uint32_t d = 0;
+      if (!e.finish(d)) return 0;
+      depth = std::max(depth, d);
+      lower.insert(lower.end(), e.toks.begin(), e.toks.end());
+    }
+    top.group(0, reps.size(), 0, false);
+    uint32_t d = 0;
+    if (!top.finish(d)) return 0;
+    depth = std::max(depth, d);
+    upper = top.toks;
+  }
+  toks.insert(toks.end(), lower.begin(), lower.end());
+  toks.insert(toks.end(), bounds.begin(), bounds.end());
+  toks.insert(toks.end(), upper.begin(), upper.end());
+  return (uint32_t)upper.size();
+}
 
 struct Member {
   std::vector<unsigned long long> src, dst;
   unsigned long long nbytes;
-  uint32_t rop, tok;
+  uint32_t rop, tok, team, ttok;
 };
 
 // ---- ranges ------------------------------------------------------------------
@@ -209,10 +264,18 @@ unsigned long long groups(const SweepClass &k) {
 // Launches, vectors per lane and units of a sweep's classes.
 void plan_launches(Sweep &sw) {
   bool folds = false;
-  for (const SweepClass &k : sw.classes) folds |= k.nsrc > 1 && sweep_lw(k.meta) >= 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
+  unsigned long long fold_units = 0;
+  auto folded = [](const SweepClass &k) {
+    return k.nsrc > 1 && sweep_lw(k.meta) >= 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
+  };
+  for (const SweepClass &k : sw.classes)
+    if (folded(k)) fold_units += (k.nbytes + 511) / 512 * k.nmem;
+  auto teamed = [&](const SweepClass &k) { return k.team > 1 && fold_units < SWEEP_TEAM_UNITS; };
+  for (const SweepClass &k : sw.classes) folds |= folded(k) && !teamed(k);
   auto kernel_of = [&](const SweepClass &k) -> uint32_t {
     if (sweep_lw(k.meta) < 4) return k.nsrc > 1 ? SWEEP_NARROW : SWEEP_SHIFT;
     if (k.nsrc > 1 && sweep_dtype(k.meta) == HICCL_FP8E4M3) return SWEEP_FP8;
+    if (folded(k) && teamed(k)) return SWEEP_TEAM;
     return k.nsrc > 1 || folds ? SWEEP_FOLD : SWEEP_COPY;
   };
   std::stable_sort(sw.classes.begin(), sw.classes.end(),
@@ -255,7 +318,12 @@ void plan_launches(Sweep &sw) {
     const uint32_t most = SWEEP_THREADS[kern];
     // a short pass uses small CTAs, so that its units reach every SM
     uint32_t warps = most / 32;
-    while (warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
+    while (kern != SWEEP_TEAM && warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
+    // a team's warps: no more than sections, and enough for SWEEP_TEAM_WARPS in all
+    uint32_t sections = 1;
+    for (size_t i = a; i < z; ++i) sections = std::max(sections, sw.classes[i].team);
+    while (kern == SWEEP_TEAM && warps > sections) warps /= 2;
+    while (kern == SWEEP_TEAM && warps > 1 && units * (warps / 2) >= SWEEP_TEAM_WARPS) warps /= 2;
     L.threads = warps * 32;
     sw.launches.push_back(L);
     a = z;
@@ -277,7 +345,7 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
     Member m;
     m.nbytes = (unsigned long long)p.count * c.esize;
     m.rop = 0;
-    m.tok = 0;
+    m.tok = m.team = m.ttok = 0;
     if (p.epoch != epoch) {
       epoch = p.epoch;
       idx.build(ms, ms.size());
@@ -293,25 +361,32 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
       m.dst.push_back(p.recv[p.root]);
     } else {
       const bool rounds = p.op == HICCL_SUM && (c.dtype == HICCL_BF16 || c.dtype == HICCL_FP8E4M3);
+      const bool exact = p.op != HICCL_SUM || c.dtype == HICCL_I32;
       const long long node = c.ring > 1 ? p.root / node_ranks : -1;
       const Program *pg = nullptr;
       for (size_t k = progs.size(); k-- > 0 && !pg && k + 64 > progs.size();)
-        if (progs[k].node == node && progs[k].rounds == rounds && progs[k].leaves == p.leaves) pg = &progs[k];
+        if (progs[k].node == node && progs[k].rounds == rounds && progs[k].exact == exact && progs[k].leaves == p.leaves) pg = &progs[k];
       if (!pg) {
         Expr e(hierarchy, p.leaves, rounds);
         if (c.ring > 1) e.chain(c.ring, ring_lvl, node);
         else e.group(0, p.leaves.size(), 0, false);
         uint32_t depth = 0;
         if (!e.finish(depth)) return;
-        sw.depth = std::max(sw.depth, depth);
-        progs.push_back(Program{p.leaves, node, rounds, e.order, (uint32_t)sw.toks.size()});
+        const uint32_t tok = (uint32_t)sw.toks.size();
         sw.toks.insert(sw.toks.end(), e.toks.begin(), e.toks.end());
+        const uint32_t ttok = (uint32_t)sw.toks.size();
+        const uint32_t team =
+            c.dtype == HICCL_FP8E4M3 ? 0 : two_steps(hierarchy, p.leaves, rounds, exact, c.ring > 1, sw.toks, depth);
+        sw.depth = std::max(sw.depth, depth);
+        progs.push_back(Program{p.leaves, node, rounds, exact, e.order, tok, team, ttok});
         pg = &progs.back();
       }
       for (int r : pg->order) m.src.push_back(p.send[r]);
       m.dst.push_back(p.recv[p.root]);
       m.rop = (uint32_t)p.op;
       m.tok = pg->tok;
+      m.team = pg->team;
+      m.ttok = pg->ttok;
     }
     // earlier epochs: no conflict, or a copy of exactly what one expression
     // stores (whose sources it may overwrite in place)
@@ -367,6 +442,8 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
     k.nsrc = (uint32_t)m0.src.size();
     k.ndst = (uint32_t)m0.dst.size();
     k.tok = m0.tok;
+    k.team = m0.team;
+    k.ttok = m0.ttok;
     k.meta = sweep_meta((uint32_t)c.dtype, m0.rop, widths[v[0]], 1, 0);
     for (uint32_t i : v) {
       sw.ptrs.insert(sw.ptrs.end(), ms[i].src.begin(), ms[i].src.end());
@@ -386,6 +463,7 @@ void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw) {
     for (SweepClass k : m->classes) {
       k.ptr += sw.ptrs.size();
       k.tok += (uint32_t)sw.toks.size();
+      k.ttok += (uint32_t)sw.toks.size();
       sw.classes.push_back(k);
     }
     sw.ptrs.insert(sw.ptrs.end(), m->ptrs.begin(), m->ptrs.end());

@@ -68,7 +68,7 @@ __device__ __forceinline__ Unit find_unit(const SweepArgs &A, uint32_t unit) {
     const uint4 *q = reinterpret_cast<const uint4 *>(A.classes + lo);
     uint4 *z = reinterpret_cast<uint4 *>(&r.k);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) z[i] = __ldg(q + i);
+    for (int i = 0; i < 4; ++i) z[i] = __ldg(q + i);
   }
   const SweepClass &k = r.k;
   uint32_t at = unit - k.unit0, g = 0;
@@ -227,21 +227,16 @@ struct Tokens {
   __device__ __forceinline__ uint32_t at(uint32_t q) const { return __shfl_sync(0xffffffffu, mine, q & 31u); }
 };
 
-// One unit of a fold: V vectors of W bytes per lane, at byte offset `off` of
-// the lane's first vector, vectors 32 * W bytes apart, those ending past
-// `end` left out.  U sources are in flight; every source's token says how it
-// enters the accumulator (see TOK_*).  `stack` holds this thread's saved
-// values, word k at stack[k * threads].
-template <int FAM, int W, int V, int U>
-__device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__ P, const uint32_t *__restrict__ tok,
-                                          uint32_t nsrc, uint32_t ndst, unsigned long long off, unsigned long long end,
-                                          uint32_t dt, uint32_t rop, uint32_t *stack, uint32_t threads) {
+// The value of an expression of nsrc sources: V vectors of W bytes a lane,
+// load(q, x) filling source q's.  U sources are in flight; every source's
+// token says how it enters the accumulator (see TOK_*).  `stack` holds this
+// thread's saved values, word k at stack[k * threads].
+template <int FAM, int W, int V, int U, typename LD>
+__device__ __forceinline__ void fold_value(LD load, const uint32_t *__restrict__ tok, uint32_t nsrc, uint32_t dt,
+                                           uint32_t rop, uint32_t *stack, uint32_t threads, Raw<W> (&r)[V]) {
   using A = Acc<FAM, W>;
   constexpr int N = A::N;
   uint32_t acc[V * N];
-  bool on[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v) on[v] = off + v * (32 * W) + W <= end;
   static_assert(32 % U == 0, "the sources in flight lie in one 32-bit mask");
   uint32_t sp = 0;   // words saved
   Tokens t;
@@ -250,12 +245,7 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
     if ((q & 31u) == 0) t.read(tok, q, nsrc);
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (q + u < nsrc) {
-        const unsigned long long s = __ldg(P + q + u) + off;
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-          if (on[v]) x[u][v] = ld_raw<W>(s + v * (32 * W));
-      }
+      if (q + u < nsrc) load(q + u, x[u]);
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (q + u < nsrc) {
@@ -289,9 +279,28 @@ __device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__
         }
       }
   }
-  Raw<W> r[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) r[v] = A::pack(acc + v * N);
+}
+
+// One unit of a fold: the lane's first vector at byte offset `off` of every
+// operand, vectors 32 * W bytes apart, those ending past `end` left out.
+template <int FAM, int W, int V, int U>
+__device__ __forceinline__ void fold_unit(const unsigned long long *__restrict__ P, const uint32_t *__restrict__ tok,
+                                          uint32_t nsrc, uint32_t ndst, unsigned long long off, unsigned long long end,
+                                          uint32_t dt, uint32_t rop, uint32_t *stack, uint32_t threads) {
+  bool on[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) on[v] = off + v * (32 * W) + W <= end;
+  Raw<W> r[V];
+  fold_value<FAM, W, V, U>(
+      [&](uint32_t q, Raw<W> (&x)[V]) {
+        const unsigned long long s = __ldg(P + q) + off;
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          if (on[v]) x[v] = ld_raw<W>(s + v * (32 * W));
+      },
+      tok, nsrc, dt, rop, stack, threads, r);
 #pragma unroll 4
   for (uint32_t d = 0; d < ndst; ++d) {
     const unsigned long long a = __ldg(P + nsrc + d) + off;
@@ -537,6 +546,66 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FOLD], 16) sweep_fold_kern
   if (u.k.nsrc == 1) copy_member(u, lane);
   else if (A.groups == FOLD_GROUPS) fold_member<FOLD_GROUPS>(A, u, lane);
   else fold_member<FOLD_GROUPS_SHORT>(A, u, lane);
+}
+
+// A short fold pass: a CTA to a unit.  Its warps evaluate the expression's
+// sections (SweepClass::team), leave their values in shared memory, and after
+// a barrier every warp evaluates the expression of those and stores its share
+// of the destinations.
+template <int FAM, int W>
+__device__ __forceinline__ void team_unit(const SweepArgs &A, const Unit &u, unsigned long long off,
+                                          unsigned long long end, uint32_t dt, uint32_t rop, uint4 *parts,
+                                          uint32_t *stack) {
+  const SweepClass &k = u.k;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const uint32_t *tok = A.toks + k.ttok, *bounds = tok + k.nsrc, *upper = bounds + k.team + 1;
+  const bool on = off + W <= end;
+  auto part = [&](uint32_t s) { return reinterpret_cast<Raw<W> *>(parts + s * 32 + lane); };
+  Raw<W> r[1];
+  for (uint32_t s = warp; s < k.team; s += warps) {
+    const uint32_t q0 = __ldg(bounds + s), q1 = __ldg(bounds + s + 1);
+    fold_value<FAM, W, 1, 8>(
+        [&](uint32_t q, Raw<W> (&x)[1]) {
+          const unsigned long long a = __ldg(u.P + q0 + q) + off;
+          if (on) x[0] = ld_raw<W>(a);
+        },
+        tok + q0, q1 - q0, dt, rop, stack, blockDim.x, r);
+    *part(s) = r[0];
+  }
+  __syncthreads();
+  fold_value<FAM, W, 1, 8>([&](uint32_t s, Raw<W> (&x)[1]) { x[0] = *part(s); }, upper, k.team, dt, rop, stack,
+                           blockDim.x, r);
+  if (!on) return;
+#pragma unroll 4
+  for (uint32_t d = warp; d < k.ndst; d += warps) st_raw<W>(__ldg(u.P + k.nsrc + d) + off, r[0]);
+}
+template <int W>
+__device__ __forceinline__ void team_any(const SweepArgs &A, const Unit &u, unsigned long long off,
+                                         unsigned long long end, uint4 *parts, uint32_t *stack) {
+  const uint32_t dt = sweep_dtype(u.k.meta), rop = sweep_rop(u.k.meta);
+  if (dt == HICCL_BF16) {
+    if (rop == HICCL_SUM) team_unit<BF16_SUM, W>(A, u, off, end, dt, rop, parts, stack);
+    else team_unit<BF16_ANY, W>(A, u, off, end, dt, rop, parts, stack);
+  } else if constexpr (W >= 4) {
+    if (dt == HICCL_F32 && rop == HICCL_SUM) team_unit<F32_SUM, W>(A, u, off, end, dt, rop, parts, stack);
+    else team_unit<ANY_32, W>(A, u, off, end, dt, rop, parts, stack);
+  }
+}
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_TEAM], 2)
+    sweep_team_kernel(const __grid_constant__ SweepArgs A) {
+  __shared__ uint4 parts[SWEEP_TEAM_MAX * 32];
+  extern __shared__ __align__(16) uint32_t saved[];
+  launch_order();
+  const int lane = threadIdx.x & 31;
+  const Unit u = find_unit(A, blockIdx.x);
+  uint32_t *stack = saved + threadIdx.x;
+  const Body b = body_of(u.k, u.P);
+  team_any<16>(A, u, b.head + (unsigned long long)u.part * 512 + lane * 16, b.end, parts, stack);
+  if (u.part + 1 == u.k.upm && b.end - b.head != u.k.nbytes) {
+    __syncthreads();   // the parts have been read
+    if (sweep_dtype(u.k.meta) == HICCL_BF16) team_any<2>(A, u, edge_of<2>(u.k, b, lane), u.k.nbytes, parts, stack);
+    else team_any<4>(A, u, edge_of<4>(u.k, b, lane), u.k.nbytes, parts, stack);
+  }
 }
 
 // folds of operands that lie differently off a 16-byte boundary: W-byte
@@ -825,7 +894,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(
 
 typedef void (*Kernel)(const SweepArgs);
 const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel,
-                                         sweep_shift_kernel};
+                                         sweep_shift_kernel, sweep_team_kernel};
 
 }  // namespace
 
@@ -845,7 +914,7 @@ cudaError_t sweep_prepare() {
 cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_sm, cudaStream_t s) {
   const unsigned warps = L.threads / 32;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((L.units + warps - 1) / warps);
+  cfg.gridDim = dim3(L.kernel == SWEEP_TEAM ? L.units : (L.units + warps - 1) / warps);
   cfg.blockDim = dim3(L.threads);
   cfg.dynamicSmemBytes = (size_t)L.stack_words * 4 * L.threads;
   if (L.kernel == SWEEP_FP8) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;

@@ -19,7 +19,7 @@ from tests._bridge import FakeAddresses, register
 from tests._cases import fill, random_program
 
 START, PUSH, ROUND, POP, JOIN = 1, 2, 1, 2, 3
-COPY, FOLD, FP8, NARROW, SHIFT = range(5)
+COPY, FOLD, FP8, NARROW, SHIFT, TEAM = range(6)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -31,9 +31,10 @@ def decode(blob):
     """(classes, launches, pointers, tokens) of a sweep's inspection blob."""
     nc, nl, npt, nt = struct.unpack_from("<4Q", blob, 0)
     o = 32
-    cls = [dict(zip(("nbytes", "ptr", "unit0", "upm", "nmem", "nsrc", "ndst", "tok", "meta", "group"),
-                    struct.unpack_from("<2Q8I", blob, o + 48 * k))) for k in range(nc)]
-    o += 48 * nc
+    cls = [dict(zip(("nbytes", "ptr", "unit0", "upm", "nmem", "nsrc", "ndst", "tok", "meta", "group",
+                     "team", "ttok"),
+                    struct.unpack_from("<2Q10I", blob, o + 64 * k))) for k in range(nc)]
+    o += 64 * nc
     lau = [dict(zip(("kernel", "lo", "hi", "units", "threads", "words"), struct.unpack_from("<6I", blob, o + 24 * k)))
            for k in range(nl)]
     o += 24 * nl
@@ -102,7 +103,7 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
                 p = ptrs[c["ptr"] + i * (c["nsrc"] + c["ndst"]):][:c["nsrc"] + c["ndst"]]
                 assert all((a - p[0]) % c["width"] == 0 for a in p) and (c["width"] >= 16 or p[0] % c["width"] == 0)
                 assert (L["kernel"] in (NARROW, SHIFT)) == (c["width"] < 16)
-                assert L["kernel"] == FOLD or (c["nsrc"] > 1) == (L["kernel"] in (FP8, NARROW))
+                assert L["kernel"] == FOLD or (c["nsrc"] > 1) == (L["kernel"] in (FP8, NARROW, TEAM))
                 members.append((c, p))
         assert L["units"] == units and L["threads"] in (32, 64, 128, 256, 512)
     rng = np.random.Generator(np.random.PCG64(seed))
@@ -111,7 +112,16 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         vals = [view(a, c["nbytes"]).copy().view(dt) for a in p[:c["nsrc"]]]
         out = vals[0]
         if c["nsrc"] > 1:
-            out, most = evaluate(vals, toks[c["tok"]:c["tok"] + c["nsrc"]], H.OP_NAMES[c["rop"]], dtype)
+            op, n, T = H.OP_NAMES[c["rop"]], c["nsrc"], c["team"]
+            out, most = evaluate(vals, toks[c["tok"]:c["tok"] + n], op, dtype)
+            assert T > 1 or c["kernel"] != TEAM
+            if T:                                        # in two steps, whichever the launch takes
+                lower, bounds, upper = np.split(np.array(toks[c["ttok"]:c["ttok"] + n + 2 * T + 1]), [n, n + T + 1])
+                assert bounds[0] == 0 and bounds[-1] == n and T <= 32 and n >= 8
+                parts = [evaluate(vals[a:z], lower[a:z].tolist(), op, dtype) for a, z in zip(bounds, bounds[1:])]
+                two, m2 = evaluate([p for p, _ in parts], upper.tolist(), op, dtype)
+                assert np.array_equal(two.view(np.uint8), out.view(np.uint8))
+                most = max([most, m2] + [m for _, m in parts])
             acc = 16 if dtype == "fp8" else (min(c["width"], 16) // (2 if dtype == "bf16" else 4))
             L = next(x for x in lau if x["kernel"] == c["kernel"])
             assert most * max(acc, 1) * c["v"] <= L["words"]   # saved values fit
@@ -238,6 +248,27 @@ def test_a_repeated_copy_and_a_disjoint_one_are_swept():
     assert check(two_epochs(build), [2, 2], 1, 1)
 
 
+@pytest.mark.parametrize("P,h,dtype,op,ring,T", [(64, [4, 4, 4], "f32", "sum", 1, 4), (64, [8, 8], "bf16", "sum", 1, 8),
+                                                 (12, [2, 2, 3], "bf16", "sum", 1, 4), (8, [2, 4], "f32", "sum", 1, 2),
+                                                 (16, [16], "f32", "sum", 1, 0), (16, [16], "i32", "sum", 1, 4),
+                                                 (64, [64], "i32", "max", 1, 8), (16, [4, 4], "f32", "min", 4, 4),
+                                                 (16, [4, 4], "f32", "sum", 4, 0), (6, [2, 3], "f32", "sum", 1, 0),
+                                                 (16, [4, 4], "fp8", "sum", 1, 0)])
+def test_two_step_forms(P, h, dtype, op, ring, T):
+    """Sections at a level's groups, or anywhere for exact operators; none for
+    chains and one-level sums, whose order is sequential, nor for few sources."""
+    prog = PR.reducescatter(P, 2 if dtype == "fp8" else 37, dtype=dtype, op=op)
+    assert check(prog, h, 1, 1, seed=P, ring=ring, zero_frac=0.25)
+    fake = FakeAddresses(prog)
+    comm = register(prog, fake.addr)
+    comm.set_option(H.OPT_RING, ring)
+    comm.plan(h, 1, 1)
+    cls, lau, _, _ = decode(comm.sweep())
+    assert {c["team"] for c in cls} == {T}
+    if T and all(c["width"] >= 16 for c in cls):
+        assert [x["kernel"] for x in lau] == [TEAM]
+
+
 def test_deep_hierarchies_fall_back():
     """Eight levels of two need seven saved values, more than the kernels hold."""
     assert check(PR.reduce(64, 8), [2] * 6, 1, 1)
@@ -260,4 +291,4 @@ def test_group_sweep_is_the_union():
     cls, lau, ptrs, _ = decode(g.sweep())
     assert sum(k["nmem"] for k in cls) == total
     assert sorted(ptrs) == sorted(p for c in members for p in decode(c.sweep())[2])
-    assert len(lau) == 1 and lau[0]["kernel"] == FOLD
+    assert [x["kernel"] for x in lau] == [FOLD, TEAM]         # the flat sum is sequential
