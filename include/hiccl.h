@@ -394,7 +394,7 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
  * payload, 2 combine (saved, accumulator), 3 combine (accumulator, saved)).
  * meta: dtype 4 bits, operator 3, log2 of the access width 3, vectors per lane 5,
  * kernel 3 (0 copies, 1 folds, 2 FP8 folds; of operands that lie differently
- * off a 16-byte boundary: 3 folds, 4 copies; 5 folds in two steps).  A two-step
+ * off a 16-byte boundary: 3 folds, 4 copies; 5, 6 folds in two steps).  A two-step
  * form evaluates `sections` runs of sources apart and then an expression of
  * their values: the sections' tokens, sections + 1 bounds, tokens of the values.  *bytes receives the size (0: the plan has no sweep); a NULL or too small `out` is
  * left alone.  HICCL_ERR_STATE without a plan. */

@@ -168,7 +168,8 @@ enum : uint32_t {
   SWEEP_NARROW = 3,   // folds of other operands: 4- or 2-byte accesses
   SWEEP_SHIFT = 4,    // copies of other operands: vectors shifted in registers
   SWEEP_TEAM = 5,     // folds as SWEEP_FOLD's, a CTA to a unit
-  SWEEP_KERNELS = 6
+  SWEEP_FP8_TEAM = 6, // folds as SWEEP_FP8's, a CTA to a unit
+  SWEEP_KERNELS = 7
 };
 // A copy's destinations are stored in groups of SWEEP_GROUP, group after group
 // over SWEEP_TILE / (vectors per lane) units of source (4 MiB, which stay in
@@ -178,7 +179,7 @@ enum : uint32_t {
 // (7.2 TB/s), 1 40.4 us.  16 MiB to 16 destinations by tiles of 1 / 2 / 4 / 8 /
 // 16 MiB: 43.1 / 42.5 / 41.2 / 42.4 / 45.9 us.
 constexpr uint32_t SWEEP_GROUP = 2, SWEEP_TILE = 8192;
-constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128, 512};   // most threads of a CTA
+constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128, 512, 256};   // most threads of a CTA
 
 constexpr uint32_t SWEEP_TEAM_MAX = 32;    // sections of an expression
 // In a fold pass of few units every warp folds one source after the other,

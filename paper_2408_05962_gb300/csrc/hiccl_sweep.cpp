@@ -252,7 +252,7 @@ uint32_t width_log2(const Member &m) {
 
 // bytes of a member that a warp moves with one vector per lane
 unsigned long long row_bytes(uint32_t kern, const SweepClass &k) {
-  if (kern == SWEEP_FP8) return 4 * FP8_BLOCK_BYTES;
+  if (kern == SWEEP_FP8 || kern == SWEEP_FP8_TEAM) return 4 * FP8_BLOCK_BYTES;
   return kern == SWEEP_SHIFT ? 31 * 16 : 32ull << std::min(sweep_lw(k.meta), 4u);
 }
 
@@ -263,20 +263,21 @@ unsigned long long groups(const SweepClass &k) {
 
 // Launches, vectors per lane and units of a sweep's classes.
 void plan_launches(Sweep &sw) {
-  bool folds = false;
+  bool folds = false;   // a launch of SWEEP_FOLD, which copies can join
   unsigned long long fold_units = 0;
-  auto folded = [](const SweepClass &k) {
-    return k.nsrc > 1 && sweep_lw(k.meta) >= 4 && sweep_dtype(k.meta) != HICCL_FP8E4M3;
+  auto fold_kernel = [](const SweepClass &k) -> uint32_t {
+    return sweep_dtype(k.meta) == HICCL_FP8E4M3 ? SWEEP_FP8 : SWEEP_FOLD;
   };
+  auto folded = [](const SweepClass &k) { return k.nsrc > 1 && sweep_lw(k.meta) >= 4; };
   for (const SweepClass &k : sw.classes)
-    if (folded(k)) fold_units += (k.nbytes + 511) / 512 * k.nmem;
+    if (folded(k)) fold_units += (k.nbytes + row_bytes(fold_kernel(k), k) - 1) / row_bytes(fold_kernel(k), k) * k.nmem;
   auto teamed = [&](const SweepClass &k) { return k.team > 1 && fold_units < SWEEP_TEAM_UNITS; };
-  for (const SweepClass &k : sw.classes) folds |= folded(k) && !teamed(k);
+  for (const SweepClass &k : sw.classes) folds |= folded(k) && !teamed(k) && fold_kernel(k) == SWEEP_FOLD;
   auto kernel_of = [&](const SweepClass &k) -> uint32_t {
     if (sweep_lw(k.meta) < 4) return k.nsrc > 1 ? SWEEP_NARROW : SWEEP_SHIFT;
-    if (k.nsrc > 1 && sweep_dtype(k.meta) == HICCL_FP8E4M3) return SWEEP_FP8;
-    if (folded(k) && teamed(k)) return SWEEP_TEAM;
-    return k.nsrc > 1 || folds ? SWEEP_FOLD : SWEEP_COPY;
+    if (!folded(k)) return folds ? SWEEP_FOLD : SWEEP_COPY;
+    if (teamed(k)) return fold_kernel(k) == SWEEP_FP8 ? SWEEP_FP8_TEAM : SWEEP_TEAM;
+    return fold_kernel(k);
   };
   std::stable_sort(sw.classes.begin(), sw.classes.end(),
                    [&](const SweepClass &a, const SweepClass &b) { return kernel_of(a) < kernel_of(b); });
@@ -298,7 +299,7 @@ void plan_launches(Sweep &sw) {
       uint32_t v = 1;
       if (kern == SWEEP_SHIFT) v = rows >= 4 * 2432 ? 4 : 1;
       else if (kern == SWEEP_NARROW) v = rows >= 8 * 2432 ? 8 : rows >= 2 * 2432 ? 2 : 1;
-      else if (kern != SWEEP_FP8 && k.nsrc == 1) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
+      else if (k.nsrc == 1) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
       const unsigned long long unit = row_bytes(kern, k) * v;
       const unsigned long long upm = (k.nbytes + unit - 1) / unit;
       k.meta = sweep_meta(dt, sweep_rop(k.meta), lw, v, kern);
@@ -311,19 +312,20 @@ void plan_launches(Sweep &sw) {
         return;
       }
       // accumulator words of a lane: 32-bit values, or BF16 / FP8 values widened to 32 bits
-      const uint32_t acc = kern == SWEEP_FP8 ? 16 : lw >= 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
+      const uint32_t acc = kern == SWEEP_FP8 || kern == SWEEP_FP8_TEAM ? 16 : lw >= 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
       if (k.nsrc > 1) words = std::max(words, sw.depth * acc * v);
     }
     SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words};
     const uint32_t most = SWEEP_THREADS[kern];
     // a short pass uses small CTAs, so that its units reach every SM
     uint32_t warps = most / 32;
-    while (kern != SWEEP_TEAM && warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
+    const bool team = kern == SWEEP_TEAM || kern == SWEEP_FP8_TEAM;
+    while (!team && warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
     // a team's warps: no more than sections, and enough for SWEEP_TEAM_WARPS in all
     uint32_t sections = 1;
     for (size_t i = a; i < z; ++i) sections = std::max(sections, sw.classes[i].team);
-    while (kern == SWEEP_TEAM && warps > sections) warps /= 2;
-    while (kern == SWEEP_TEAM && warps > 1 && units * (warps / 2) >= SWEEP_TEAM_WARPS) warps /= 2;
+    while (team && warps > sections) warps /= 2;
+    while (team && warps > 1 && units * (warps / 2) >= SWEEP_TEAM_WARPS) warps /= 2;
     L.threads = warps * 32;
     sw.launches.push_back(L);
     a = z;
@@ -375,8 +377,7 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
         const uint32_t tok = (uint32_t)sw.toks.size();
         sw.toks.insert(sw.toks.end(), e.toks.begin(), e.toks.end());
         const uint32_t ttok = (uint32_t)sw.toks.size();
-        const uint32_t team =
-            c.dtype == HICCL_FP8E4M3 ? 0 : two_steps(hierarchy, p.leaves, rounds, exact, c.ring > 1, sw.toks, depth);
+        const uint32_t team = two_steps(hierarchy, p.leaves, rounds, exact, c.ring > 1, sw.toks, depth);
         sw.depth = std::max(sw.depth, depth);
         progs.push_back(Program{p.leaves, node, rounds, exact, e.order, tok, team, ttok});
         pg = &progs.back();

@@ -774,77 +774,90 @@ constexpr int FP8_GROUPS = 2;                                   // of the ring o
 constexpr uint32_t FP8_SLOTS = FP8_GROUPS * RING_GROUP;
 constexpr uint32_t FP8_STEP = 4 * FP8_BLOCK_BYTES;              // bytes of a source in one slot
 
+// blocks in shared memory: this lane's 16 codes (and the scale) of its group's
+__device__ __forceinline__ Fp8Raw fp8_read(const char *block) {
+  Fp8Raw x;
+  x.c = *reinterpret_cast<const uint4 *>(block + 16 * (threadIdx.x & 7));
+  x.scale = *reinterpret_cast<const float *>(block + 128);
+  return x;
+}
+__device__ __forceinline__ void fp8_write(char *block, const Fp8Raw &r) {
+  const uint32_t sub = threadIdx.x & 7;
+  *reinterpret_cast<uint4 *>(block + 16 * sub) = r.c;
+  if (sub == 0) *reinterpret_cast<uint4 *>(block + 128) = make_uint4(__float_as_uint(r.scale), 0u, 0u, 0u);
+}
 // A unit is four blocks, 576 bytes of every operand.  A source takes about 100
-// instructions, so a warp is busy while its loads should fly; they
-// pass through a ring of slots in shared memory, an asynchronous copy group
-// for every RING_GROUP sources, which keeps loads in flight through folds,
-// encodings and stores without holding registers (72 a thread, 24 warps an SM).  Copies and
-// stores move the unit as one range of whole sectors, and only the fold reads
-// it by blocks.  All-reduce of 16 Mi values a rank over 32 ranks ({4, 8}),
+// instructions, so a warp is busy while its loads should fly; they pass
+// through a ring of slots in shared memory, an asynchronous copy group for
+// every RING_GROUP sources, which keeps loads in flight through folds,
+// encodings and stores without holding registers (72 a thread, 24 warps an
+// SM).  Copies and stores move the unit as one range of whole sectors, and
+// only the fold reads it by blocks.  All-reduce of 16 Mi values a rank over 32 ranks ({4, 8}),
 // 1.21 GB in and out: 265 us with the next sources loaded into registers (16
 // warps an SM; 403 us when refilled one by one), 223 us through the ring by
 // blocks, 199 us by the unit's range, 186 us (6.5 TB/s) with copy groups of
 // four sources; two or four units a warp lose 5 and 10 %, neighbouring warps
 // on neighbouring units read longer stretches of each source at a time.
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
-  extern __shared__ __align__(16) uint32_t saved[];
-  launch_order();
-  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (unit >= A.units) return;
-  const Unit u = find_unit(A, unit);
-  const SweepClass &k = u.k;
-  const unsigned long long *P = u.P;
-  const uint32_t part = u.part;
-  const uint32_t *tok = A.toks + k.tok;
-  const uint32_t threads = blockDim.x, sub = lane & 7;
-  const unsigned long long minus0 = A.minus0;
-  char *ring = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (FP8_SLOTS * FP8_STEP);
-  char *mine = ring + (lane >> 3) * FP8_BLOCK_BYTES;   // this group's block in slot 0
-  const uint32_t ring_at = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + 16 * lane;
-  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + (threads >> 5) * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
+struct Fp8Ring {
+  const unsigned long long *P;
+  uint32_t nsrc, lq, g, slot, ring_at;
+  const char *mine;              // this lane's block in slot 0
+  unsigned long long off;        // this lane's 16 bytes of the unit
+  bool on, on2;                  // ... lie in the member; and 512 bytes further on (lanes 0 .. 3)
 
-  // this lane's 16 bytes of the unit, and (lanes 0 .. 3) 16 of its last 64
-  const unsigned long long off = (unsigned long long)part * FP8_STEP + 16 * lane;
-  const bool on = off < k.nbytes, on2 = lane < 4 && off + 512 < k.nbytes;
-  unsigned long long held = 0;
-  uint32_t lq = 0;   // next source to load
-  auto load = [&](uint32_t g) {
+  __device__ __forceinline__ void load(uint32_t to_group) {
 #pragma unroll
     for (uint32_t i = 0; i < RING_GROUP; ++i)
-      if (lq + i < k.nsrc) {
-        const unsigned long long s = pointer_at(P, lq + i, k.nsrc, held) + off;
-        const uint32_t to = ring_at + (g * RING_GROUP + i) * FP8_STEP;
+      if (lq + i < nsrc) {
+        const unsigned long long s = pointer_at(P, lq + i, nsrc, held) + off;
+        const uint32_t to = ring_at + (to_group * RING_GROUP + i) * FP8_STEP;
         if (on) cp_async16(to, s);
         if (on2) cp_async16(to + 512, s + 512);
       }
     lq += RING_GROUP;
     cp_commit();
-  };
+  }
+  __device__ __forceinline__ void start(const unsigned long long *sources, uint32_t n) {
+    P = sources;
+    nsrc = n;
+    lq = g = 0;
 #pragma unroll 1
-  for (uint32_t g = 0; g < FP8_GROUPS - 1; ++g) load(g);
-  unsigned long long acc[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] = 0ull;
-  uint32_t sp = 0;   // saved values end here
-  Tokens t;
-  uint32_t g = 0, slot = 0;
-#pragma unroll 1
-  for (uint32_t q = 0; q < k.nsrc; ++q) {
-    if ((q & 31u) == 0) t.read(tok, q, k.nsrc);
+    for (uint32_t i = 0; i < FP8_GROUPS - 1; ++i) load(i);
+  }
+  __device__ __forceinline__ Fp8Raw next(uint32_t q) {   // q = 0, 1, ...
     if (q % RING_GROUP == 0) {
       cp_wait<FP8_GROUPS - 2>();
-      __syncwarp();            // every lane's copies have landed, and the group read last is free
+      __syncwarp();              // every lane's copies have landed, and the group read last is free
       load(g == 0 ? FP8_GROUPS - 1 : g - 1);
       slot = g * RING_GROUP;
       if (++g == FP8_GROUPS) g = 0;
     }
-    Fp8Raw x;
-    x.c = *reinterpret_cast<const uint4 *>(mine + slot * FP8_STEP + 16 * sub);
-    x.scale = *reinterpret_cast<const float *>(mine + slot * FP8_STEP + 128);
+    const Fp8Raw x = fp8_read(mine + slot * FP8_STEP);
     ++slot;
+    return x;
+  }
+  __device__ __forceinline__ void drain() {              // the ring is free afterwards
+    cp_wait<0>();
+    __syncwarp();
+  }
+
+ private:
+  unsigned long long held;
+};
+
+// the value of an expression, next(q) giving source q
+template <typename NEXT>
+__device__ __forceinline__ void fp8_fold(NEXT next, const uint32_t *tok, uint32_t nsrc, unsigned long long minus0,
+                                         ulonglong2 *stack, uint32_t threads, unsigned long long (&acc)[8]) {
+  uint32_t sp = 0;   // saved values end here
+  Tokens t;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i] = 0ull;
+#pragma unroll 1
+  for (uint32_t q = 0; q < nsrc; ++q) {
+    if ((q & 31u) == 0) t.read(tok, q, nsrc);
     unsigned long long y[8];
-    fp8_widen(x, minus0, y);
+    fp8_widen(next(q), minus0, y);
     if (t.plain(q)) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) acc[i] = add2(acc[i], y[i]);
@@ -876,25 +889,84 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(
       }
     }
   }
-  const Fp8Raw r = fp8_encode(acc);
-  cp_wait<0>();
-  __syncwarp();   // the ring is free: the result takes slot 0
-  *reinterpret_cast<uint4 *>(mine + 16 * sub) = r.c;
-  if (sub == 0) *reinterpret_cast<uint4 *>(mine + 128) = make_uint4(__float_as_uint(r.scale), 0u, 0u, 0u);
+}
+
+// the unit in slot 0 of the ring, as one range, to destinations d0, d0 + step, ...
+__device__ __forceinline__ void fp8_store(const Unit &u, const Fp8Ring &ring, const char *slot0, uint32_t d0,
+                                          uint32_t step) {
+  const uint32_t lane = threadIdx.x & 31;
   __syncwarp();
-  const uint4 v = *reinterpret_cast<const uint4 *>(ring + 16 * lane);
-  const uint4 v2 = *reinterpret_cast<const uint4 *>(ring + 512 + 16 * (lane & 3));
+  const uint4 v = *reinterpret_cast<const uint4 *>(slot0 + 16 * lane);
+  const uint4 v2 = *reinterpret_cast<const uint4 *>(slot0 + 512 + 16 * (lane & 3));
 #pragma unroll 4
-  for (uint32_t d = 0; d < k.ndst; ++d) {
-    const unsigned long long a = __ldg(P + k.nsrc + d) + off;
-    if (on) *reinterpret_cast<uint4 *>(a) = v;
-    if (on2) *reinterpret_cast<uint4 *>(a + 512) = v2;
+  for (uint32_t d = d0; d < u.k.ndst; d += step) {
+    const unsigned long long a = __ldg(u.P + u.k.nsrc + d) + ring.off;
+    if (ring.on) *reinterpret_cast<uint4 *>(a) = v;
+    if (ring.on2) *reinterpret_cast<uint4 *>(a + 512) = v2;
   }
+}
+__device__ __forceinline__ void fp8_ring_at(Fp8Ring &r, const Unit &u, char *base) {
+  const uint32_t lane = threadIdx.x & 31;
+  r.ring_at = static_cast<uint32_t>(__cvta_generic_to_shared(base)) + 16 * lane;
+  r.mine = base + (lane >> 3) * FP8_BLOCK_BYTES;
+  r.off = (unsigned long long)u.part * FP8_STEP + 16 * lane;
+  r.on = r.off < u.k.nbytes;
+  r.on2 = lane < 4 && r.off + 512 < u.k.nbytes;
+}
+
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
+  extern __shared__ __align__(16) uint32_t saved[];
+  launch_order();
+  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (unit >= A.units) return;
+  const Unit u = find_unit(A, unit);
+  char *base = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (FP8_SLOTS * FP8_STEP);
+  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + (blockDim.x >> 5) * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
+  Fp8Ring ring;
+  fp8_ring_at(ring, u, base);
+  ring.start(u.P, u.k.nsrc);
+  unsigned long long acc[8];
+  fp8_fold([&](uint32_t q) { return ring.next(q); }, A.toks + u.k.tok, u.k.nsrc, A.minus0, stack, blockDim.x, acc);
+  const Fp8Raw r = fp8_encode(acc);
+  ring.drain();
+  fp8_write(const_cast<char *>(ring.mine), r);
+  fp8_store(u, ring, base, 0, 1);
+}
+
+// a short pass: a CTA to a unit, as sweep_team_kernel
+__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8_TEAM], 2)
+    sweep_fp8_team_kernel(const __grid_constant__ SweepArgs A) {
+  __shared__ __align__(16) char parts[SWEEP_TEAM_MAX * FP8_STEP];
+  extern __shared__ __align__(16) uint32_t saved[];
+  launch_order();
+  const Unit u = find_unit(A, blockIdx.x);
+  const SweepClass &k = u.k;
+  const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5, grp = (threadIdx.x & 31) >> 3;
+  char *base = reinterpret_cast<char *>(saved) + warp * (FP8_SLOTS * FP8_STEP);
+  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + warps * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
+  const uint32_t *tok = A.toks + k.ttok, *bounds = tok + k.nsrc, *upper = bounds + k.team + 1;
+  Fp8Ring ring;
+  fp8_ring_at(ring, u, base);
+  unsigned long long acc[8];
+  for (uint32_t s = warp; s < k.team; s += warps) {
+    const uint32_t q0 = __ldg(bounds + s), n = __ldg(bounds + s + 1) - q0;
+    ring.start(u.P + q0, n);
+    Fp8Raw only;   // a section of one source passes its block through
+    fp8_fold([&](uint32_t q) { return only = ring.next(q); }, tok + q0, n, A.minus0, stack, blockDim.x, acc);
+    const Fp8Raw r = fp8_encode(acc);
+    fp8_write(parts + s * FP8_STEP + grp * FP8_BLOCK_BYTES, n == 1 ? only : r);
+    ring.drain();
+  }
+  __syncthreads();
+  fp8_fold([&](uint32_t s) { return fp8_read(parts + s * FP8_STEP + grp * FP8_BLOCK_BYTES); }, upper, k.team, A.minus0,
+           stack, blockDim.x, acc);
+  fp8_write(const_cast<char *>(ring.mine), fp8_encode(acc));
+  fp8_store(u, ring, base, warp, warps);
 }
 
 typedef void (*Kernel)(const SweepArgs);
 const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel,
-                                         sweep_shift_kernel, sweep_team_kernel};
+                                         sweep_shift_kernel, sweep_team_kernel, sweep_fp8_team_kernel};
 
 }  // namespace
 
@@ -914,10 +986,10 @@ cudaError_t sweep_prepare() {
 cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_sm, cudaStream_t s) {
   const unsigned warps = L.threads / 32;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(L.kernel == SWEEP_TEAM ? L.units : (L.units + warps - 1) / warps);
+  cfg.gridDim = dim3(L.kernel == SWEEP_TEAM || L.kernel == SWEEP_FP8_TEAM ? L.units : (L.units + warps - 1) / warps);
   cfg.blockDim = dim3(L.threads);
   cfg.dynamicSmemBytes = (size_t)L.stack_words * 4 * L.threads;
-  if (L.kernel == SWEEP_FP8) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;
+  if (L.kernel == SWEEP_FP8 || L.kernel == SWEEP_FP8_TEAM) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;
   SweepArgs B = A;
   if (L.kernel == SWEEP_FOLD) {
     B.groups = L.units < SHORT_UNITS ? FOLD_GROUPS_SHORT : FOLD_GROUPS;

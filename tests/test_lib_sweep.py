@@ -19,7 +19,7 @@ from tests._bridge import FakeAddresses, register
 from tests._cases import fill, random_program
 
 START, PUSH, ROUND, POP, JOIN = 1, 2, 1, 2, 3
-COPY, FOLD, FP8, NARROW, SHIFT, TEAM = range(6)
+COPY, FOLD, FP8, NARROW, SHIFT, TEAM, FP8_TEAM = range(7)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -94,7 +94,7 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         units = 0
         for c in cls[L["lo"]:L["hi"]]:
             assert c["kernel"] == L["kernel"] and c["unit0"] == units
-            unit = {FP8: 4 * 144, SHIFT: 31 * 16}.get(L["kernel"], 32 * min(c["width"], 16)) * c["v"]
+            unit = {FP8: 4 * 144, FP8_TEAM: 4 * 144, SHIFT: 31 * 16}.get(L["kernel"], 32 * min(c["width"], 16)) * c["v"]
             assert (c["upm"] - 1) * unit < c["nbytes"] <= c["upm"] * unit        # units tile a member
             assert c["v"] in (1, 2, 4, 8, 16)
             assert c["group"] == (c["ndst"] if c["nsrc"] > 1 else 2)
@@ -103,7 +103,7 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
                 p = ptrs[c["ptr"] + i * (c["nsrc"] + c["ndst"]):][:c["nsrc"] + c["ndst"]]
                 assert all((a - p[0]) % c["width"] == 0 for a in p) and (c["width"] >= 16 or p[0] % c["width"] == 0)
                 assert (L["kernel"] in (NARROW, SHIFT)) == (c["width"] < 16)
-                assert L["kernel"] == FOLD or (c["nsrc"] > 1) == (L["kernel"] in (FP8, NARROW, TEAM))
+                assert L["kernel"] == FOLD or (c["nsrc"] > 1) == (L["kernel"] not in (COPY, SHIFT))
                 members.append((c, p))
         assert L["units"] == units and L["threads"] in (32, 64, 128, 256, 512)
     rng = np.random.Generator(np.random.PCG64(seed))
@@ -114,11 +114,12 @@ def run_sweep(comm, fake, mem, dtype, seed=0):
         if c["nsrc"] > 1:
             op, n, T = H.OP_NAMES[c["rop"]], c["nsrc"], c["team"]
             out, most = evaluate(vals, toks[c["tok"]:c["tok"] + n], op, dtype)
-            assert T > 1 or c["kernel"] != TEAM
+            assert T > 1 or c["kernel"] not in (TEAM, FP8_TEAM)
             if T:                                        # in two steps, whichever the launch takes
                 lower, bounds, upper = np.split(np.array(toks[c["ttok"]:c["ttok"] + n + 2 * T + 1]), [n, n + T + 1])
                 assert bounds[0] == 0 and bounds[-1] == n and T <= 32 and n >= 8
-                parts = [evaluate(vals[a:z], lower[a:z].tolist(), op, dtype) for a, z in zip(bounds, bounds[1:])]
+                parts = [evaluate(vals[a:z], lower[a:z].tolist(), op, dtype) if z - a > 1 else (vals[a], 0)
+                         for a, z in zip(bounds, bounds[1:])]
                 two, m2 = evaluate([p for p, _ in parts], upper.tolist(), op, dtype)
                 assert np.array_equal(two.view(np.uint8), out.view(np.uint8))
                 most = max([most, m2] + [m for _, m in parts])
@@ -253,7 +254,7 @@ def test_a_repeated_copy_and_a_disjoint_one_are_swept():
                                                  (16, [16], "f32", "sum", 1, 0), (16, [16], "i32", "sum", 1, 4),
                                                  (64, [64], "i32", "max", 1, 8), (16, [4, 4], "f32", "min", 4, 4),
                                                  (16, [4, 4], "f32", "sum", 4, 0), (6, [2, 3], "f32", "sum", 1, 0),
-                                                 (16, [4, 4], "fp8", "sum", 1, 0)])
+                                                 (16, [4, 4], "fp8", "sum", 1, 4)])
 def test_two_step_forms(P, h, dtype, op, ring, T):
     """Sections at a level's groups, or anywhere for exact operators; none for
     chains and one-level sums, whose order is sequential, nor for few sources."""
@@ -266,7 +267,7 @@ def test_two_step_forms(P, h, dtype, op, ring, T):
     cls, lau, _, _ = decode(comm.sweep())
     assert {c["team"] for c in cls} == {T}
     if T and all(c["width"] >= 16 for c in cls):
-        assert [x["kernel"] for x in lau] == [TEAM]
+        assert [x["kernel"] for x in lau] == [FP8_TEAM if dtype == "fp8" else TEAM]
 
 
 def test_deep_hierarchies_fall_back():
