@@ -7,19 +7,22 @@ of fp32 per rank (uniform[-1, 1], seed 0), stripe 4, pipeline 8; each
 collective is one start of its own persistent communicator.  The seven
 starts of a step are captured once in a CUDA graph, each on its own stream
 forked from the step's stream (independent collectives started back to back
-on separate streams, so that one launch's last work items run beside the
-next one's first); the timed region is a series of blocks of K graph
+on separate streams, so that one launch's last units run beside the next
+one's first); the timed region is a series of blocks of K graph
 replays (at least one second in all) and the median block gives the step
 time (Sec. 6.2 reports the median of its measured rounds).  Beside it: the
 same step with the starts in order on one stream ("serial_step"), the same
 steps through start / wait on the host ("eager"), and the seven collectives
 as one grouped communicator, one launch per step ("grouped_step").
 
-Metric: device-memory GB/s of the schedule (each copy reads its bytes once
-and writes them once per destination; an f-input reduce reads f times and
-writes once), with the fraction of the measured HBM bandwidth; per
-collective GB/s, the semantic-minimum bytes and the paper-style d*p/t are
-reported beside it.  The default line also carries, each under its own
+Metric: GB/s of the schedule (each copy reads its bytes once and writes them
+once per destination; an f-input reduce reads f times and writes once): the
+factorized schedule's work over time.  A start runs it as one pass that reads
+every input once and writes every output once, so the schedule's rate can
+exceed the memory's; the roofline fraction therefore divides those minimum
+bytes ("min_bytes") by the time and the measured HBM bandwidth.  Per
+collective GB/s, the minimum bytes and the paper-style d*p/t are reported
+beside it.  The default line also carries, each under its own
 timing: the 64 MiB-per-rank All-reduce as FP32, BF16 and FP8 payloads with
 their FP64 errors; the batch of 256 mixed collectives (one launch each,
 grouped, graph); and a short served run with p50 / p99 latency.
@@ -287,7 +290,8 @@ def measured_peak():
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("hiccl_runtime.cu", "hiccl_internal.h"):
+    for f in ("hiccl_sweep.cu", "hiccl_sweep.cpp", "hiccl_sweep.h", "hiccl_device.cuh", "hiccl_runtime.cu",
+              "hiccl_internal.h"):
         with open(os.path.join(ROOT, "paper_2408_05962_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -295,7 +299,7 @@ def kernel_hash():
 
 def recorded_traffic():
     """DRAM bytes per launch from the committed ncu summary, if it was taken
-    on the current executor source (else None)."""
+    on the current kernel sources (else None)."""
     try:
         vals = {}
         with open(TRAFFIC_FILE) as f:
@@ -558,11 +562,11 @@ def _make_comm(H, P, dtype, args):
 def _graph_of(comms, kinds, device, concurrent=False):
     """One CUDA graph holding one start of the communicator of every name in
     ``kinds`` (names may repeat; a start under capture records only the
-    executor launch, and each replay is a complete execution): in order on
+    launch, and each replay is a complete execution): in order on
     one stream, or (``concurrent``) each on its own stream forked from the
     graph's stream and joined back, as independent collectives started back
     to back on separate streams run -- the launches then overlap on the
-    device (one's last work items beside the next one's first) instead of
+    device (one's last units beside the next one's first) instead of
     each waiting for the previous grid to complete."""
     import torch
     gs = torch.cuda.Stream(device)
@@ -663,7 +667,7 @@ def measure_collectives(args, device, world, workload, dtype, xs=None, e2e=True)
     torch.cuda.synchronize(device)
 
     # the same collectives as one grouped communicator (hiccl_group): one
-    # persistent launch per step whose tickets interleave the seven by depth
+    # launch per step
     grouped = None
     if len(kinds) > 1:
         gcomm = H.Comm.group([comms[k] for k in kinds])
@@ -726,13 +730,16 @@ def measure_collectives(args, device, world, workload, dtype, xs=None, e2e=True)
         gm = per_kind_graph[kind]
         coll[kind] = {"ms": med, "gbs": nbytes[kind] / med / 1e6, "frac": nbytes[kind] / med / 1e6 / peak,
                       "graph_ms": gm, "graph_gbs": nbytes[kind] / gm / 1e6, "graph_frac": nbytes[kind] / gm / 1e6 / peak,
+                      "graph_min_frac": mbytes[kind] / gm / 1e6 / peak,
                       "dp_over_t_gbs": pbytes[kind] / med / 1e6, "schedule_bytes": nbytes[kind],
                       "min_bytes": mbytes[kind], "min_gbs": mbytes[kind] / med / 1e6,
                       "level_bytes": comms[kind].level_bytes(), "steps": comms[kind].plan_info()["steps"]}
     accuracy = None
     if dtype in ("bf16", "fp8") and "allreduce" in bufs:
         accuracy = _lowprec_accuracy(bufs["allreduce"], dtype, xs, device)
-    out = {"value": gbs, "frac": gbs / world / peak, "peak": peak, "peak_kind": peak_kind,
+    step_min = sum(mbytes.values())
+    out = {"value": gbs, "frac": gbs / world / peak, "min_gbs": gbs / world * step_min / step_bytes,
+           "step_min_bytes": step_min, "peak": peak, "peak_kind": peak_kind,
            "ms_per_step": block_ms / args.steps, "blocks": len(blocks), "steps_per_block": args.steps,
            "block_ms": blocks, "timed_s": sum(blocks) / 1e3, "wall_s": wall, "clocks": clk,
            "launches": len(kinds) * args.steps * len(blocks), "step_bytes": step_bytes,
@@ -821,7 +828,8 @@ def measure_allreduce64(args, device, dtypes=("f32", "bf16", "fp8")):
     out = {}
     for dt in dtypes:
         r = measure_collectives(sub, device, 1, "allreduce64", dt, xs=xs, e2e=False)
-        out[dt] = {"gbs": r["value"], "frac": r["frac"], "ms": r["ms_per_step"],
+        out[dt] = {"gbs": r["value"], "frac": r["frac"], "min_gbs": r["min_gbs"], "min_frac": r["min_gbs"] / r["peak"],
+                   "ms": r["ms_per_step"],
                    "schedule_bytes": r["step_bytes"], "eager_gbs": r["eager"]["value"],
                    **({"accuracy": r["accuracy"]} if r["accuracy"] else {})}
     out["config"] = workload_config("allreduce64", 1, "f32+bf16+fp8")
@@ -848,7 +856,7 @@ def measure_batch(args, device, steps):
     gen.manual_seed(0)
     comms, bufs, tuned = [], [], {}
     stream = torch.cuda.current_stream(device)
-    total_bytes = 0
+    total_bytes = total_min = 0
     t_setup = time.perf_counter()
     for dsc in descs:
         P, h, dt = dsc["P"], dsc["hierarchy"], dsc["dtype"]
@@ -871,6 +879,7 @@ def measure_batch(args, device, steps):
             tuned[key] = comm.autotune(stream, tune_method=True)
         rd, wr = comm.hbm_bytes()
         total_bytes += rd + wr
+        total_min += min_bytes(dsc["kind"], P, dsc["bytes_per_rank"])
         comms.append(comm)
         bufs.append(b)
     t_setup = time.perf_counter() - t_setup
@@ -904,7 +913,8 @@ def measure_batch(args, device, steps):
     out = {"schedule_bytes": total_bytes, "one_launch_each_ms": t_sep * 1e3,
            "grouped_ms": t_grp * 1e3, "graph_ms": t_graph * 1e3,
            "one_launch_each_gbs": total_bytes / t_sep / 1e9, "grouped_gbs": total_bytes / t_grp / 1e9,
-           "graph_gbs": total_bytes / t_graph / 1e9, "speedup_vs_one_launch_each": t_sep / t_graph,
+           "graph_gbs": total_bytes / t_graph / 1e9, "min_bytes": total_min,
+           "graph_min_gbs": total_min / t_graph / 1e9, "speedup_vs_one_launch_each": t_sep / t_graph,
            "tuned_configs": len(tuned), "setup_s": t_setup,
            "config": "256 collectives (All-gather/Reduce-scatter/All-reduce), P in {8,16,32}, two-level "
                      "hierarchies, 4 KiB..16 MiB per rank log-uniform, fp32/bf16, one persistent launch "
@@ -1038,9 +1048,9 @@ def run_ours(args):
     default_run = (args.workload == "seven" and not args.kinds and args.ring == 1 and not args.bytes_per_rank
                    and not args.item_bytes and not args.ctas_per_sm and not args.threads and args.order is None
                    and not args.slot_items)
-    # DRAM bytes of an average executor launch of the default workload, from
-    # the committed ncu capture (null for other workloads or options, or once
-    # the executor sources have changed since the capture)
+    # DRAM bytes of an average launch of the default workload, from the
+    # committed ncu capture (null for other workloads or options, or once the
+    # kernel sources have changed since the capture)
     step_traffic = recorded_traffic() if default_run else None
     nk = len(r["collectives"])
     traffic = step_traffic / nk if step_traffic else None
@@ -1062,10 +1072,13 @@ def run_ours(args):
                              "'graph_ms' from a graph of ten starts of that collective, replayed",
                    "blocks": r["blocks"], "timed_s": r["timed_s"],
                    "block_ms": r["block_ms"], "eager": r["eager"]},
-        "roofline": {"bound": "hbm", "achieved": r["value"] / world, "peak": peak, "unit": "GB/s",
-                     "frac": r["frac"], "peak_source": r["peak_kind"],
+        "roofline": {"bound": "hbm", "achieved": r["min_gbs"], "peak": peak, "unit": "GB/s",
+                     "frac": r["min_gbs"] / peak, "peak_source": r["peak_kind"],
+                     "bytes": "every input read once, every output written once (what the sweep kernels move)",
                      "traffic": traffic, "traffic_per_step": step_traffic,
-                     "schedule_bytes_per_launch": r["step_bytes"] / nk, "kernel": "hiccl_exec_kernel"},
+                     "min_bytes_per_launch": r["step_min_bytes"] / nk,
+                     "schedule_bytes_per_launch": r["step_bytes"] / nk,
+                     "schedule_frac": r["frac"], "kernel": "sweep_copy_kernel, sweep_fold_kernel"},
         "clocks": r["clocks"], "gpu_launches": r["launches"] * world,
         "e2e": r["e2e"], "collectives": r["collectives"], "cpu_baseline": cpu,
     }
@@ -1113,9 +1126,11 @@ def run_batch(args):
         "vs_baseline": None, "dtype": "f32+bf16", "data": "synthetic",
         "config": {"workload": b["config"], "collectives": 256, "parallelism": f"replicas{world}",
                    "tuned_configs": b["tuned_configs"]},
-        "roofline": {"bound": "hbm", "achieved": gbs / world, "peak": peak, "unit": "GB/s",
-                     "frac": gbs / world / peak, "peak_source": peak_kind, "traffic": None,
-                     "kernel": "hiccl_exec_kernel"},
+        "roofline": {"bound": "hbm", "achieved": b["graph_min_gbs"], "peak": peak, "unit": "GB/s",
+                     "frac": b["graph_min_gbs"] / peak, "schedule_frac": gbs / world / peak,
+                     "bytes": "every input read once, every output written once",
+                     "peak_source": peak_kind, "traffic": None,
+                     "kernel": "sweep_copy_kernel, sweep_fold_kernel"},
         "clocks": clk, "gpu_launches": args.steps * world, "batch": b,
     }
     if rank == 0:
@@ -1161,7 +1176,7 @@ def run_serve(args):
                                f"{args.budget_gb} GB budget, continuous batching", "parallelism": f"replicas{world}"},
         "roofline": {"bound": "hbm", "achieved": head["gbs"], "peak": peak, "unit": "GB/s",
                      "frac": head["gbs"] / peak, "peak_source": peak_kind, "traffic": None,
-                     "kernel": "hiccl_exec_kernel"},
+                     "kernel": "sweep_copy_kernel, sweep_fold_kernel"},
         "clocks": clk, "serving": out, "p50_ms": head.get("p50_ms"), "p99_ms": head.get("p99_ms"),
     }
     if rank == 0:
