@@ -382,12 +382,12 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
  * a copy or a nested fold over equal byte ranges (every collective of Table 2
  * does; TRACE and hiccl_debug_withhold select the step-by-step executor).
  * `out` receives, without padding: the counts of classes, launches, operand
- * pointers and tokens (u64 each); the classes (64 bytes: bytes per operand
+ * pointers, tokens and hints (u64 each); the classes (64 bytes: bytes per operand
  * u64, first pointer u64, then u32 first unit, units per member, members,
  * sources, destinations, first token, meta, destinations per unit, sections,
  * first token of the two-step form, 0, 0); the
- * launches (24 bytes: u32 kernel, first and end class, units, threads, saved
- * words per thread); the pointers (u64; per member its sources in evaluation order, then its
+ * launches (32 bytes: u32 kernel, first and end class, units, threads, saved
+ * words per thread, first hint, 0); the pointers (u64; per member its sources in evaluation order, then its
  * destinations); the tokens (u32, one per source: bit 0 the source starts the
  * accumulator, bit 1 after the old one was saved, else it is combined in;
  * then two-bit operations from bit 8 on: 1 round the accumulator to the
@@ -396,7 +396,9 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
  * kernel 3 (0 copies, 1 folds, 2 FP8 folds; of operands that lie differently
  * off a 16-byte boundary: 3 folds, 4 copies; 5, 6 folds in two steps).  A two-step
  * form evaluates `sections` runs of sources apart and then an expression of
- * their values: the sections' tokens, sections + 1 bounds, tokens of the values.  *bytes receives the size (0: the plan has no sweep); a NULL or too small `out` is
+ * their values: the sections' tokens, sections + 1 bounds, tokens of the values.
+ * Last come the hints (u32) of launches of more than 96 classes: hint i is the
+ * class, from the launch's first, of unit 128 i.  *bytes receives the size (0: the plan has no sweep); a NULL or too small `out` is
  * left alone.  HICCL_ERR_STATE without a plan. */
 hiccl_status_t hiccl_debug_sweep(hiccl_comm_t comm, void *out, size_t capacity, size_t *bytes);
 

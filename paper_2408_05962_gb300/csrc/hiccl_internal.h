@@ -230,12 +230,20 @@ HICCL_HD inline uint32_t sweep_lw(uint32_t m) { return (m >> 7) & 7u; }
 HICCL_HD inline uint32_t sweep_v(uint32_t m) { return (m >> 10) & 31u; }
 HICCL_HD inline uint32_t sweep_kernel(uint32_t m) { return (m >> 15) & 7u; }
 
+// A launch of more than SWEEP_PREFIX classes finds a unit's class from hints:
+// hint i is the class (within the launch) of unit i << SWEEP_HINT_SHIFT, so
+// the class lies between two of them.  (By a binary search over the classes in
+// memory, eight dependent loads a warp, the group of 256 collectives of 4 KiB to
+// 16 MiB took 2.21 ms instead of 1.92.)
+constexpr uint32_t SWEEP_HINT_SHIFT = 7;
 struct SweepLaunch {
   uint32_t kernel;
   uint32_t class_lo, class_hi;
   uint32_t units;
   uint32_t threads;
   uint32_t stack_words;        // 32-bit words of saved values per thread
+  uint32_t hint;               // first hint
+  uint32_t pad;
 };
 
 // ---------------------------------------------------------------------------
@@ -247,7 +255,7 @@ struct SweepLaunch {
 struct Sweep {
   bool valid = false;
   std::vector<SweepClass> classes;            // grouped by launch
-  std::vector<uint32_t> toks;
+  std::vector<uint32_t> toks, hints;
   std::vector<unsigned long long> ptrs;
   std::vector<SweepLaunch> launches;
   uint32_t depth = 0;                         // saved values of the deepest expression

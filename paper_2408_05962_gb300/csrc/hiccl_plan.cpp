@@ -1715,8 +1715,9 @@ hiccl_status_t hiccl_debug_sweep(hiccl_comm_t c, void *out, size_t capacity, siz
     if (!c->plan.valid) return fail(c, HICCL_ERR_STATE, "no plan");
     const Sweep &w = c->plan.sweep;
     if (!w.valid) return HICCL_OK;
-    const unsigned long long n[4] = {w.classes.size(), w.launches.size(), w.ptrs.size(), w.toks.size()};
-    *bytes = sizeof(n) + n[0] * sizeof(SweepClass) + n[1] * sizeof(SweepLaunch) + n[2] * 8 + n[3] * 4;
+    const unsigned long long n[5] = {w.classes.size(), w.launches.size(), w.ptrs.size(), w.toks.size(),
+                                     w.hints.size()};
+    *bytes = sizeof(n) + n[0] * sizeof(SweepClass) + n[1] * sizeof(SweepLaunch) + n[2] * 8 + n[3] * 4 + n[4] * 4;
     if (!out || capacity < *bytes) return HICCL_OK;
     char *q = static_cast<char *>(out);
     auto put = [&](const void *src, size_t len) {
@@ -1728,6 +1729,7 @@ hiccl_status_t hiccl_debug_sweep(hiccl_comm_t c, void *out, size_t capacity, siz
     put(w.launches.data(), n[1] * sizeof(SweepLaunch));
     put(w.ptrs.data(), n[2] * 8);
     put(w.toks.data(), n[3] * 4);
+    put(w.hints.data(), n[4] * 4);
     return HICCL_OK;
   });
 }

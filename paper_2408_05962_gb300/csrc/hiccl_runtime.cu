@@ -1070,11 +1070,13 @@ static hiccl_status_t dev_alloc(hiccl_comm *c, void **ptr, size_t bytes, const c
 static hiccl_status_t upload_sweep(hiccl_comm *c) {
   const Sweep &w = c->plan.sweep;
   DevState *d = c->dev;
-  const size_t cb = w.classes.size() * sizeof(SweepClass), pb = w.ptrs.size() * 8, tb = w.toks.size() * 4;
-  std::vector<char> img(std::max<size_t>(cb + pb + tb, 16));
+  const size_t cb = w.classes.size() * sizeof(SweepClass), pb = w.ptrs.size() * 8, tb = w.toks.size() * 4,
+               hb = w.hints.size() * 4;
+  std::vector<char> img(std::max<size_t>(cb + pb + tb + hb, 16));
   if (cb) std::memcpy(img.data(), w.classes.data(), cb);
   if (pb) std::memcpy(img.data() + cb, w.ptrs.data(), pb);
   if (tb) std::memcpy(img.data() + cb + pb, w.toks.data(), tb);
+  if (hb) std::memcpy(img.data() + cb + pb + tb, w.hints.data(), hb);
   const hiccl_status_t st = dev_alloc(c, &d->sweep_table, img.size(), "sweep table");
   if (st != HICCL_OK) return st;
   cudaError_t e = cudaMemcpyAsync(d->sweep_table, img.data(), img.size(), cudaMemcpyHostToDevice, d->upload);
@@ -1086,6 +1088,7 @@ static hiccl_status_t upload_sweep(hiccl_comm *c) {
     A.classes = reinterpret_cast<const SweepClass *>(base) + L.class_lo;
     A.ptrs = reinterpret_cast<const unsigned long long *>(base + cb);
     A.toks = reinterpret_cast<const uint32_t *>(base + cb + pb);
+    A.hints = A.toks + w.toks.size() + L.hint;
     A.nclass = L.class_hi - L.class_lo;
     A.units = L.units;
     for (uint32_t k = 0; k < A.nclass && k < SWEEP_PREFIX; ++k) A.unit0[k] = w.classes[L.class_lo + k].unit0;

@@ -282,6 +282,7 @@ void plan_launches(Sweep &sw) {
   std::stable_sort(sw.classes.begin(), sw.classes.end(),
                    [&](const SweepClass &a, const SweepClass &b) { return kernel_of(a) < kernel_of(b); });
   sw.launches.clear();
+  sw.hints.clear();
   for (size_t a = 0; a < sw.classes.size();) {
     const uint32_t kern = kernel_of(sw.classes[a]);
     size_t z = a;
@@ -315,7 +316,12 @@ void plan_launches(Sweep &sw) {
       const uint32_t acc = kern == SWEEP_FP8 || kern == SWEEP_FP8_TEAM ? 16 : lw >= 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
       if (k.nsrc > 1) words = std::max(words, sw.depth * acc * v);
     }
-    SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words};
+    SweepLaunch L{kern, (uint32_t)a, (uint32_t)z, (uint32_t)units, 0, words, (uint32_t)sw.hints.size(), 0};
+    if (z - a > SWEEP_PREFIX)
+      for (size_t i = a, u = 0; u <= units + (1u << SWEEP_HINT_SHIFT); u += 1u << SWEEP_HINT_SHIFT) {
+        while (i + 1 < z && sw.classes[i + 1].unit0 <= u) ++i;
+        sw.hints.push_back((uint32_t)(i - a));
+      }
     const uint32_t most = SWEEP_THREADS[kern];
     // a short pass uses small CTAs, so that its units reach every SM
     uint32_t warps = most / 32;

@@ -55,6 +55,10 @@ struct Unit {
 };
 __device__ __forceinline__ Unit find_unit(const SweepArgs &A, uint32_t unit) {
   uint32_t lo = 0, hi = A.nclass;
+  if (hi > SWEEP_PREFIX) {
+    lo = __ldg(A.hints + (unit >> SWEEP_HINT_SHIFT));
+    hi = __ldg(A.hints + (unit >> SWEEP_HINT_SHIFT) + 1) + 1;
+  }
   while (hi - lo > 1) {   // last class whose first unit is not past `unit`
     const uint32_t mid = (lo + hi) >> 1;
     const uint32_t u0 = A.nclass <= SWEEP_PREFIX ? A.unit0[mid] : __ldg(&A.classes[mid].unit0);

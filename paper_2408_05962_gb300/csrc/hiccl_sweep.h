@@ -11,6 +11,7 @@ struct SweepArgs {
   const SweepClass *classes;            // of this launch
   const uint32_t *toks;
   const unsigned long long *ptrs;
+  const uint32_t *hints;                // of this launch
   uint32_t nclass;
   uint32_t units;
   uint32_t groups = 0;                  // of a fold's ring

@@ -192,3 +192,27 @@ def test_sweep_replayed_and_restarted():
                 c.start()
                 c.wait()
             assert all(torch.equal(b.recv, w) for b, w in zip(bufs, want))
+
+
+def test_many_classes():
+    """A program of 300 primitives of different lengths: copies and folds whose
+    classes are found through hints."""
+    from oracle.model import Program
+    prog = Program(4)
+    n = [1 + 13 * k % 2200 for k in range(300)]
+    a = [prog.buffer(("send", r), sum(n)) for r in range(4)]
+    b = [prog.buffer(("recv", r), sum(n)) for r in range(4)]
+    o = 0
+    for k, m in enumerate(n):
+        if k % 3:
+            prog.multicast(k % 4, [0, 1, 2, 3], m, a[k % 4].shift(o), {j: b[j].shift(o) for j in range(4)})
+        else:
+            prog.reduction([0, 1, 2, 3], k % 4, m, {j: a[j].shift(o) for j in range(4)}, b[k % 4].shift(o))
+        o += m
+    mem0 = fill(prog, 11)
+    ref = {k: v.copy() for k, v in mem0.items()}
+    S.run_program(prog, ref, [2, 2])
+    outs, comm = run_on_gpu(prog, [2, 2], 1, 1, mem0, repeats=2)
+    assert comm.sweep()
+    for out in outs:
+        assert_bit_equal(ref, out)

@@ -29,18 +29,26 @@ def built():
 
 def decode(blob):
     """(classes, launches, pointers, tokens) of a sweep's inspection blob."""
-    nc, nl, npt, nt = struct.unpack_from("<4Q", blob, 0)
-    o = 32
+    nc, nl, npt, nt, nh = struct.unpack_from("<5Q", blob, 0)
+    o = 40
     cls = [dict(zip(("nbytes", "ptr", "unit0", "upm", "nmem", "nsrc", "ndst", "tok", "meta", "group",
                      "team", "ttok"),
                     struct.unpack_from("<2Q10I", blob, o + 64 * k))) for k in range(nc)]
     o += 64 * nc
-    lau = [dict(zip(("kernel", "lo", "hi", "units", "threads", "words"), struct.unpack_from("<6I", blob, o + 24 * k)))
+    lau = [dict(zip(("kernel", "lo", "hi", "units", "threads", "words", "hint"), struct.unpack_from("<7I", blob, o + 32 * k)))
            for k in range(nl)]
-    o += 24 * nl
+    o += 32 * nl
     ptrs = np.frombuffer(blob, np.uint64, npt, o).tolist()
     toks = np.frombuffer(blob, np.uint32, nt, o + 8 * npt).tolist()
-    assert len(blob) == o + 8 * npt + 4 * nt
+    assert len(blob) == o + 8 * npt + 4 * (nt + nh)
+    hints = np.frombuffer(blob, np.uint32, nh, o + 8 * npt + 4 * nt)
+    for L in lau:                                        # the class of every unit lies between two hints
+        first = [c["unit0"] for c in cls[L["lo"]:L["hi"]]]
+        if len(first) > 96:
+            at = np.searchsorted(first, np.arange(L["units"]), side="right") - 1
+            h = hints[L["hint"]:]
+            i = np.arange(L["units"]) >> 7
+            assert (h[i] <= at).all() and (at <= h[i + 1]).all() and (h[i + 1] < len(first)).all()
     for c in cls:
         m = c["meta"]
         c.update(dtype=m & 15, rop=(m >> 4) & 7, width=1 << ((m >> 7) & 7), v=(m >> 10) & 31, kernel=(m >> 15) & 7)
@@ -268,6 +276,20 @@ def test_two_step_forms(P, h, dtype, op, ring, T):
     assert {c["team"] for c in cls} == {T}
     if T and all(c["width"] >= 16 for c in cls):
         assert [x["kernel"] for x in lau] == [FP8_TEAM if dtype == "fp8" else TEAM]
+
+
+def test_many_classes_have_hints():
+    """A program of 150 multicasts of different lengths: classes beyond the
+    argument prefix are found through hints, and the sweep is the oracle's."""
+    prog = Program(4)
+    n = [3 + 7 * k % 1500 for k in range(150)]
+    a = [prog.buffer(("send", r), sum(n)) for r in range(4)]
+    b = [prog.buffer(("recv", r), sum(n)) for r in range(4)]
+    o = 0
+    for k, m in enumerate(n):
+        prog.multicast(k % 4, [0, 1, 2, 3], m, a[k % 4].shift(o), {j: b[j].shift(o) for j in range(4)})
+        o += m
+    assert check(prog, [2, 2], 1, 1, seed=3)
 
 
 def test_deep_hierarchies_fall_back():
