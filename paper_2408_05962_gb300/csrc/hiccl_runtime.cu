@@ -1398,7 +1398,13 @@ hiccl_status_t hiccl_debug_withhold(hiccl_comm_t c, unsigned long long index, in
       if (index >= c->plan.steps.size() || extra < 0 || extra > 1000)
         return fail(c, HICCL_ERR_INVALID, "bad step or count");
       const hiccl_status_t st = upload_steps(c);
-      if (st != HICCL_OK) return st;
+      if (st != HICCL_OK) {   // the sweep stays
+        for (void **p : {&d->table, &d->counters, &d->scratch}) {
+          if (*p) cudaFreeAsync(*p, d->upload);
+          *p = nullptr;
+        }
+        return st;
+      }
     }
     if (index >= d->indeg.size() || extra < 0 || extra > 1000) return fail(c, HICCL_ERR_INVALID, "bad step or count");
     // the dependency count is stored in every record entry of the step

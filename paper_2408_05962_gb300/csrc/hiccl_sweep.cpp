@@ -433,8 +433,19 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
   std::map<Key, uint32_t> at;
   std::vector<std::vector<uint32_t>> members;
   std::vector<uint32_t> widths(ms.size());
+  // copies of one shape go together, as misaligned as the worst of them: in an
+  // All-to-all of odd chunks one pair of ranks in eight happens to agree, and a
+  // launch of its own costs its ramp (64 ranks x 1 MiB of BF16: 27.5 us with
+  // it, 25.1 us without)
+  std::map<std::pair<unsigned long long, size_t>, uint32_t> shape;
   for (size_t i = 0; i < ms.size(); ++i) {
     widths[i] = width_log2(ms[i]);
+    if (ms[i].src.size() > 1) continue;
+    uint32_t &w = shape.emplace(std::make_pair(ms[i].nbytes, ms[i].dst.size()), widths[i]).first->second;
+    w = std::min(w, widths[i]);
+  }
+  for (size_t i = 0; i < ms.size(); ++i) {
+    if (ms[i].src.size() == 1) widths[i] = shape[{ms[i].nbytes, ms[i].dst.size()}];
     const Key k(ms[i].nbytes, ms[i].src.size(), ms[i].dst.size(), ms[i].rop, ms[i].tok, widths[i]);
     auto it = at.emplace(k, (uint32_t)members.size()).first;
     if (it->second == members.size()) members.emplace_back();

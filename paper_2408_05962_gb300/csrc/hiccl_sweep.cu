@@ -37,10 +37,11 @@ namespace hiccl {
 namespace {
 
 // Groups of a fold's ring: three hold 6 KiB a warp, 30 warps an SM.  A pass
-// with fewer units than half of those warps (SHORT_UNITS) deepens it instead.
-// Measured with two / three / four groups: 45.1 / 43.6 / 50 us for a
-// Reduce-scatter of 64 ranks x 4 MiB, 48.7 / 46.7 / 56 us for 16 ranks x
-// 16 MiB of BF16.
+// with fewer units than half of those warps (SHORT_UNITS) deepens it instead
+// (a 64-way int32 maximum of 1 MiB a rank, 2048 units: 19.2 us with three,
+// 17.2 us with five).  Measured with two / three / four groups: 45.1 / 43.6 /
+// 50 us for a Reduce-scatter of 64 ranks x 4 MiB, 48.7 / 46.7 / 56 us for 16
+// ranks x 16 MiB of BF16.
 constexpr int FOLD_GROUPS = 3, FOLD_GROUPS_SHORT = 5;
 constexpr uint32_t SHORT_UNITS = 152 * 16;
 
@@ -104,7 +105,7 @@ struct Raw {
   uint32_t w[W >= 4 ? W / 4 : 1];
 };
 // (L2 only: under programmatic launch another kernel may just have written
-// these lines, and no input is read twice)
+// these lines, and no SM reads a line twice)
 template <int W>
 __device__ __forceinline__ Raw<W> ld_raw(unsigned long long a) {
   Raw<W> r;
@@ -643,8 +644,8 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_NARROW], 10) sweep_narrow_
 // vector takes straddle two of them, the lane's own and the next lane's, and
 // are shifted out of the pair.  (Element accesses are bound by latency: 64
 // bytes a warp request, 90 us for an odd-length BF16 All-to-all of 64 ranks x
-// 1 MiB at four requests in flight and 45 us at sixteen, against 27 us here,
-// 4.9 TB/s.)  A unit is V rows of 31 destination vectors
+// 1 MiB at four requests in flight and 45 us at sixteen, against 25 us here,
+// 5.4 TB/s; aligned, it takes 23 us.  Two vectors a lane 27.2, eight 25.9 us.)  A unit is V rows of 31 destination vectors
 // (lane 31 loads only for lane 30) -- 496 source bytes a row; the elements
 // that no whole pair covers, at most 31 bytes at each end, go one by one with
 // the member's last unit.
@@ -974,9 +975,9 @@ const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, swe
 
 }  // namespace
 
-// dynamic shared memory: at most SWEEP_MAX_DEPTH values of 16 words for each
-// of 128 threads and four rings, or of 16 words for 256; more than half an SM's keeps a second CTA
-// off it
+// dynamic shared memory: at most SWEEP_MAX_DEPTH saved values of 16 words for
+// each of 256 threads beside the rings of eight warps; more than half an SM's
+// keeps a second CTA off it
 constexpr size_t SWEEP_MAX_SMEM = SWEEP_MAX_DEPTH * 16 * 4 * 256 + 8 * FP8_SLOTS * FP8_STEP, SWEEP_HALF_SM = 120 * 1024;
 
 cudaError_t sweep_prepare() {
