@@ -54,8 +54,8 @@ METRIC = "HBM GB/s (% of GB300 peak) per collective; p50/p99 latency of served r
 KINDS = ("broadcast", "scatter", "gather", "allgather", "reducescatter", "allreduce", "alltoall")
 P, HIER, STRIPE, PIPE = 64, [4, 4, 4], 4, 8
 BYTES_PER_RANK = 4 << 20
-KERNEL_SRC = os.path.join(ROOT, "paper_2408_05962_gb300", "csrc", "hiccl_runtime.cu")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "executor_traffic_seven_p64.txt")
+
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "sweep_traffic_seven_p64.txt")
 
 
 # the two single-GPU workloads: the seven collectives (the headline), and the
