@@ -38,8 +38,8 @@ namespace {
 
 // Groups of a fold's ring: three hold 6 KiB a warp, 30 warps an SM.  A pass
 // with fewer units than half of those warps (SHORT_UNITS) deepens it instead
-// (a 64-way int32 maximum of 1 MiB a rank, 2048 units: 19.2 us with three,
-// 17.2 us with five).  Measured with two / three / four groups: 45.1 / 43.6 /
+// (a 64-way int32 maximum of 1 MiB a rank, 2048 units: 15.1 us with three,
+// 13.7 us with five).  Measured with two / three / four groups: 45.1 / 43.6 /
 // 50 us for a Reduce-scatter of 64 ranks x 4 MiB, 48.7 / 46.7 / 56 us for 16
 // ranks x 16 MiB of BF16.
 constexpr int FOLD_GROUPS = 3, FOLD_GROUPS_SHORT = 5;
@@ -181,23 +181,24 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
   return d;
 }
 
-// a[i] = a[i] op b(i) over n words, the operator's branch taken once (once per
-// word, a 64-way int32 maximum of 1 MiB a rank took 39 us instead of 26)
-template <int FAM, int N, typename F>
+// a[i] = a[i] op b(i) over N words of S sources in turn (source j's are
+// b(j * N) ..), the operator's branch taken once for all of them
+template <int FAM, int N, int S = 1, typename F>
 __device__ __forceinline__ void combine(uint32_t *a, F b, uint32_t dt, uint32_t rop) {
   auto f = [](uint32_t x) { return __uint_as_float(x); };
   auto each = [&](auto op) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = op(a[i], b(i));
+    for (int i = 0; i < N * S; ++i) a[i % N] = op(a[i % N], b(i));
   };
   auto add = [&](uint32_t x, uint32_t y) { return __float_as_uint(__fadd_rn(f(x), f(y))); };
   auto fmx = [&](uint32_t x, uint32_t y) { return __float_as_uint(fmaxf(f(x), f(y))); };
   auto fmn = [&](uint32_t x, uint32_t y) { return __float_as_uint(fminf(f(x), f(y))); };
   if constexpr ((FAM == F32_SUM || FAM == BF16_SUM) && N % 2 == 0) {
 #pragma unroll
-    for (int i = 0; i < N; i += 2) {   // two sums an instruction
+    for (int j = 0; j < N * S; j += 2) {   // two sums an instruction
+      const int i = j % N;
       float lo, hi;
-      unpack2(add2(pack2(f(a[i]), f(a[i + 1])), pack2(f(b(i)), f(b(i + 1)))), lo, hi);
+      unpack2(add2(pack2(f(a[i]), f(a[i + 1])), pack2(f(b(j)), f(b(j + 1)))), lo, hi);
       a[i] = __float_as_uint(lo);
       a[i + 1] = __float_as_uint(hi);
     }
@@ -229,6 +230,7 @@ struct Tokens {
     nz = __ballot_sync(0xffffffffu, mine != 0u);
   }
   __device__ __forceinline__ bool plain(uint32_t q) const { return !((nz >> (q & 31u)) & 1u); }
+  __device__ __forceinline__ bool plain4(uint32_t q) const { return !((nz >> (q & 31u)) & 15u); }
   __device__ __forceinline__ uint32_t at(uint32_t q) const { return __shfl_sync(0xffffffffu, mine, q & 31u); }
 };
 
@@ -405,6 +407,16 @@ __device__ __forceinline__ void fold_ring(const SweepArgs &A, const Unit &u, uns
       x[i].w[3] = v.w;
     }
     if (++g == G) g = 0;
+    // A group of plain combines takes its operator's branch once: the chain of
+    // tests between sources bounds a short pass (a 64-way int32 maximum of 1 MiB
+    // a rank 17.4 -> 13.7 us).  Sums have no such branch and would only pay for
+    // a second copy of the loop in registers (spills, 2 to 4 % slower).
+    static_assert(RING_GROUP == 4, "plain4");
+    if constexpr (FAM == ANY_32 || FAM == BF16_ANY)
+      if (q + RING_GROUP <= k.nsrc && t.plain4(q)) {
+        combine<FAM, N, RING_GROUP>(acc, [&](int j) { return C::widen(x[j / N], j % N); }, dt, rop);
+        continue;
+      }
 #pragma unroll
     for (uint32_t i = 0; i < RING_GROUP; ++i) {
       auto src = [&](int j) { return C::widen(x[i], j); };

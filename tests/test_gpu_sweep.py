@@ -90,6 +90,15 @@ def test_operators_and_fan_ins(dtype, op, d):
     _both("allreduce", 9, [9], 1, 1, d, dtype, op, seed=d + 2)
 
 
+# folds whose plain combines fill, straddle or miss a group of four, in the first
+# 32 sources and after them; enough units for a warp, not a block, to own each
+@pytest.mark.parametrize("dtype,op", [("f32", "max"), ("i32", "max"), ("bf16", "max"), ("i32", "sum")])
+@pytest.mark.parametrize("P,h", [(3, [3]), (5, [5]), (8, [8]), (9, [9]), (24, [4, 6]), (35, [35]), (36, [3, 12]), (70, [7, 10])])
+def test_groups_of_plain_combines(P, h, dtype, op):
+    d = 330000 // P + 3                                    # 2600 units, 1300 of BF16
+    _both("reduce", P, h, 1, 1, d, dtype, op, seed=P, pad=-(P * d) % 8)
+
+
 @pytest.mark.parametrize("blocks", [1, 3, 4, 5, 64, 2051])
 @pytest.mark.parametrize("P,h,ring", [(8, [2, 4], 1), (12, [2, 2, 3], 1), (16, [16], 1), (12, [4, 3], 4)])
 def test_fp8_blocks(P, h, ring, blocks):
