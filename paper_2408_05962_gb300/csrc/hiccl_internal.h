@@ -296,6 +296,26 @@ struct Prim {
   int epoch;
 };
 
+// A range that a primitive reads or writes, and those of a program: primitive
+// i has all[of[i]] .. all[of[i + 1] - 1], its reads first.
+struct Range {
+  unsigned long long lo, hi;
+  int prim;
+  bool write;
+  int rank = -1;   // owner of the buffer
+};
+struct Ranges {
+  std::vector<Range> all;
+  std::vector<size_t> of;
+};
+
+// Byte ranges of two primitives that overlap across a fence, one of them written.
+struct Conflict {
+  uint32_t later, earlier;   // primitives
+  bool same;                 // the ranges are equal
+  bool rewrites;             // both write
+};
+
 struct DevState;   // defined by the runtime
 
 struct Plan {
@@ -380,8 +400,10 @@ hiccl_status_t guarded(hiccl_comm *c, F &&body) noexcept {
   }
 }
 // the sweep of c's program over `hierarchy` (ring_lvl: level of the ring's
-// nodes), and the union of several (hiccl_sweep.cpp)
-void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl, Sweep &sw);
+// nodes; conflicts across fences ordered by the later primitive), and the
+// union of several (hiccl_sweep.cpp)
+void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl,
+                 const Ranges &ranges, const std::vector<Conflict> &conflicts, Sweep &sw);
 void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw);
 // factorize c's program again (hiccl_plan.cpp), keeping c's state
 hiccl_status_t replan(hiccl_comm *c, const std::vector<int> &hierarchy, int stripe, int pipeline);

@@ -195,46 +195,14 @@ uint32_t two_steps(const std::vector<int> &h, const std::vector<int> &leaves, bo
   return (uint32_t)upper.size();
 }
 
+constexpr uint32_t NONE = 0xffffffffu;
+
+// The operands of a member are ops[src .. src + nsrc) and ops[dst .. dst + ndst),
+// where up to `room` fit.
 struct Member {
-  std::vector<unsigned long long> src, dst;
   unsigned long long nbytes;
+  uint32_t src, nsrc, dst, ndst, room;
   uint32_t rop, tok, team, ttok;
-};
-
-// ---- ranges ------------------------------------------------------------------
-
-struct Touch {
-  unsigned long long lo, hi;
-  uint32_t member;
-  bool write;
-};
-
-// accesses sorted by lo with prefix maxima of hi
-struct TouchIndex {
-  std::vector<Touch> r;
-  std::vector<unsigned long long> pmax;
-  void build(const std::vector<Member> &ms, size_t n) {
-    r.clear();
-    for (size_t i = 0; i < n; ++i) {
-      for (unsigned long long a : ms[i].src) r.push_back(Touch{a, a + ms[i].nbytes, (uint32_t)i, false});
-      for (unsigned long long a : ms[i].dst) r.push_back(Touch{a, a + ms[i].nbytes, (uint32_t)i, true});
-    }
-    std::sort(r.begin(), r.end(), [](const Touch &a, const Touch &b) { return a.lo < b.lo; });
-    pmax.resize(r.size());
-    for (size_t k = 0; k < r.size(); ++k) pmax[k] = std::max(r[k].hi, k ? pmax[k - 1] : 0ull);
-  }
-  // f(touch) for every access overlapping [lo, hi) until it returns false
-  template <typename F>
-  bool each(unsigned long long lo, unsigned long long hi, F f) const {
-    size_t k = std::lower_bound(r.begin(), r.end(), hi, [](const Touch &x, unsigned long long v) { return x.lo < v; }) -
-               r.begin();
-    while (k > 0) {
-      --k;
-      if (pmax[k] <= lo) break;
-      if (r[k].hi > lo && !f(r[k])) return false;
-    }
-    return true;
-  }
 };
 
 // Width of the accesses that every operand of a member allows: 16 bytes when
@@ -242,10 +210,11 @@ struct TouchIndex {
 // elements at both ends), told as 32 when they lie equally far off a 32-byte
 // sector (the vectors then start with one), else the widest of 4 and 2 that
 // the addresses (and the length) share.
-uint32_t width_log2(const Member &m) {
+uint32_t width_log2(const Member &m, const std::vector<unsigned long long> &ops) {
+  const unsigned long long *src = &ops[m.src], *dst = &ops[m.dst], base = src[0];
   unsigned long long a = 0, off = 0;
-  for (unsigned long long v : m.src) a |= v, off |= v ^ m.src[0];
-  for (unsigned long long v : m.dst) a |= v, off |= v ^ m.src[0];
+  for (uint32_t k = 0; k < m.nsrc; ++k) a |= src[k], off |= src[k] ^ base;
+  for (uint32_t k = 0; k < m.ndst; ++k) a |= dst[k], off |= dst[k] ^ base;
   if (off % 16 == 0) return off % 32 == 0 ? 5 : 4;
   return a % 4 == 0 && m.nbytes % 4 == 0 ? 2 : 1;
 }
@@ -338,35 +307,106 @@ void plan_launches(Sweep &sw) {
   }
 }
 
+// Classes of equal shape, in order of first appearance.  (Neighbours are mostly
+// alike: the maps are searched where a member differs from the one before.)
+void make_classes(const hiccl_comm &c, const std::vector<Member> &ms, const std::vector<unsigned long long> &ops,
+                  Sweep &sw) {
+  // copies of one shape go together, as misaligned as the worst of them: in an
+  // All-to-all of odd chunks one pair of ranks in eight happens to agree, and a
+  // launch of its own costs its ramp (64 ranks x 1 MiB of BF16: 27.5 us with
+  // it, 25.1 us without)
+  std::map<std::pair<unsigned long long, uint32_t>, uint32_t> shapes;
+  std::vector<uint32_t> widths(ms.size());
+  auto alike = [](const Member &a, const Member &b) { return a.nbytes == b.nbytes && a.nsrc == b.nsrc && a.ndst == b.ndst; };
+  uint32_t *worst = nullptr;
+  auto shape_of = [&](size_t i) -> uint32_t & {
+    if (!i || !worst || !alike(ms[i], ms[i - 1])) worst = &shapes.emplace(std::make_pair(ms[i].nbytes, ms[i].ndst), 5u).first->second;
+    return *worst;
+  };
+  for (size_t i = 0; i < ms.size(); ++i) {
+    widths[i] = width_log2(ms[i], ops);
+    if (ms[i].nsrc > 1) continue;
+    uint32_t &w = shape_of(i);
+    w = std::min(w, widths[i]);
+  }
+  using Key = std::tuple<unsigned long long, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t>;
+  std::map<Key, uint32_t> at;
+  std::vector<uint32_t> first, class_of(ms.size());   // first member of a class, class of a member
+  size_t nptrs = 0;
+  for (size_t i = 0; i < ms.size(); ++i) {
+    const Member &m = ms[i];
+    if (m.nsrc == 1) widths[i] = shape_of(i);
+    if (i && alike(m, ms[i - 1]) && m.rop == ms[i - 1].rop && m.tok == ms[i - 1].tok && widths[i] == widths[i - 1]) {
+      class_of[i] = class_of[i - 1];
+    } else {
+      const Key k(m.nbytes, m.nsrc, m.ndst, m.rop, m.tok, widths[i]);
+      class_of[i] = at.emplace(k, (uint32_t)first.size()).first->second;
+      if (class_of[i] == first.size()) first.push_back((uint32_t)i);
+    }
+    nptrs += m.nsrc + m.ndst;
+  }
+  for (uint32_t i : first) {
+    const Member &m = ms[i];
+    SweepClass k{};
+    k.nbytes = m.nbytes;
+    k.nsrc = m.nsrc;
+    k.ndst = m.ndst;
+    k.tok = m.tok;
+    k.team = m.team;
+    k.ttok = m.ttok;
+    k.meta = sweep_meta((uint32_t)c.dtype, m.rop, widths[i], 1, 0);
+    sw.classes.push_back(k);
+  }
+  for (uint32_t k : class_of) ++sw.classes[k].nmem;
+  size_t ptr = 0;
+  std::vector<size_t> to;
+  for (SweepClass &k : sw.classes) {
+    k.ptr = ptr;
+    to.push_back(ptr);
+    ptr += (size_t)k.nmem * (k.nsrc + k.ndst);
+  }
+  sw.ptrs.resize(nptrs);
+  for (size_t i = 0; i < ms.size(); ++i) {
+    const Member &m = ms[i];
+    size_t &q = to[class_of[i]];
+    for (uint32_t k = 0; k < m.nsrc; ++k) sw.ptrs[q++] = ops[m.src + k];
+    for (uint32_t k = 0; k < m.ndst; ++k) sw.ptrs[q++] = ops[m.dst + k];
+  }
+  sw.valid = true;
+  plan_launches(sw);
+}
+
 }  // namespace
 
-void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl, Sweep &sw) {
+// (Every plan pays for its sweep, so this shares the ranges and conflicts that
+// the step table needs anyway and keeps all operands in one list.  Planning's
+// share for 64 ranks: All-reduce 33 us, with ranges sorted anew and two vectors
+// a member 330 us; All-to-all 150 against 490 us.)
+void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl,
+                 const Ranges &ranges, const std::vector<Conflict> &conflicts, Sweep &sw) {
   sw = Sweep();
-  if (c.epochs > 32) return;   // the range index is rebuilt per epoch
+  if (c.epochs > 32) return;   // (nothing measured beyond)
   std::vector<Member> ms;
+  std::vector<unsigned long long> ops, mine;
+  std::vector<uint32_t> member_of(c.prims.size(), NONE);
   std::vector<Program> progs;
-  TouchIndex idx;
-  int epoch = 0;
-  long long node_ranks = c.P / c.ring;
-  for (const Prim &p : c.prims) {
-    if (p.count == 0) continue;
-    Member m;
-    m.nbytes = (unsigned long long)p.count * c.esize;
-    m.rop = 0;
-    m.tok = m.team = m.ttok = 0;
-    if (p.epoch != epoch) {
-      epoch = p.epoch;
-      idx.build(ms, ms.size());
-    }
-    if (p.kind == 0) {
-      m.src.push_back(p.send[p.root]);
-      for (int j : p.leaves)
-        if (!(j == p.root && p.recv[j] == p.send[p.root])) m.dst.push_back(p.recv[j]);
-      if (m.dst.empty()) continue;
-    } else if (p.leaves.size() == 1) {   // the operator is omitted
-      if (p.leaves[0] == p.root && p.send[p.root] == p.recv[p.root]) continue;
-      m.src.push_back(p.send[p.leaves[0]]);
-      m.dst.push_back(p.recv[p.root]);
+  ms.reserve(c.prims.size());
+  ops.reserve(ranges.all.size());
+  const long long node_ranks = c.P / c.ring;
+  size_t next = 0;   // conflict
+  for (size_t i = 0; i < c.prims.size(); ++i) {
+    const Prim &p = c.prims[i];
+    while (next < conflicts.size() && conflicts[next].later < i) ++next;
+    const size_t r0 = ranges.of[i], r1 = ranges.of[i + 1], ops0 = ops.size();
+    if (r0 == r1) continue;
+    Member m{};
+    m.nbytes = ranges.all[r0].hi - ranges.all[r0].lo;
+    m.src = (uint32_t)ops0;
+    if (p.kind == 0 || p.leaves.size() == 1) {   // copies (one input: the operator is omitted)
+      if (ranges.all[r0].write || r1 - r0 < 2) continue;   // in place: nothing to do
+      m.nsrc = 1;
+      ops.resize(ops0 + (r1 - r0));
+      for (size_t r = r0; r < r1; ++r) ops[ops0 + (r - r0)] = ranges.all[r].lo;
     } else {
       const bool rounds = p.op == HICCL_SUM && (c.dtype == HICCL_BF16 || c.dtype == HICCL_FP8E4M3);
       const bool exact = p.op != HICCL_SUM || c.dtype == HICCL_I32;
@@ -388,89 +428,58 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
         progs.push_back(Program{p.leaves, node, rounds, exact, e.order, tok, team, ttok});
         pg = &progs.back();
       }
-      for (int r : pg->order) m.src.push_back(p.send[r]);
-      m.dst.push_back(p.recv[p.root]);
+      m.nsrc = (uint32_t)pg->order.size();
+      for (int r : pg->order) ops.push_back(p.send[r]);
+      ops.push_back(p.recv[p.root]);
       m.rop = (uint32_t)p.op;
       m.tok = pg->tok;
       m.team = pg->team;
       m.ttok = pg->ttok;
     }
+    m.dst = m.src + m.nsrc;
+    m.ndst = m.room = (uint32_t)(ops.size() - m.dst);
     // earlier epochs: no conflict, or a copy of exactly what one expression
     // stores (whose sources it may overwrite in place)
-    if (p.epoch > 0) {
-      const unsigned long long n = m.nbytes;
-      uint32_t with = 0xffffffffu;
-      bool good = true, again = false;   // again: a destination that was written before
-      auto conflict = [&](const Touch &t, unsigned long long lo) {
-        if (with != 0xffffffffu && with != t.member) return good = false;
-        with = t.member;
-        return good = t.lo == lo && t.hi == lo + n;   // same bytes at the same offsets
-      };
-      for (unsigned long long a : m.src)
-        good = good && idx.each(a, a + n, [&](const Touch &t) { return !t.write || conflict(t, a); });
-      for (unsigned long long a : m.dst)
-        good = good && idx.each(a, a + n, [&](const Touch &t) {
-          again |= t.write;
-          return conflict(t, a);
-        });
-      if (!good) return;
-      if (with != 0xffffffffu) {
-        Member &x = ms[with];
-        // the copy's source has to hold the expression's value
-        const bool holds = m.src.size() == 1 && (std::find(x.dst.begin(), x.dst.end(), m.src[0]) != x.dst.end() ||
-                                                 (x.src.size() == 1 && x.src[0] == m.src[0]));
-        if (!holds) return;
-        for (unsigned long long a : m.dst)
-          if (!again || std::find(x.dst.begin(), x.dst.end(), a) == x.dst.end()) x.dst.push_back(a);
-        continue;
-      }
+    uint32_t with = NONE;
+    bool again = false;   // a destination that was written before
+    for (; next < conflicts.size() && conflicts[next].later == i; ++next) {
+      const Conflict &x = conflicts[next];
+      const uint32_t k = member_of[x.earlier];
+      if (k == NONE) continue;                                  // it does nothing
+      if (!x.same || (with != NONE && with != k)) return;       // part of a value, or two of them
+      with = k;
+      again |= x.rewrites;
     }
-    ms.push_back(std::move(m));
-  }
-
-  // classes of equal shape, in order of first appearance
-  using Key = std::tuple<unsigned long long, size_t, size_t, uint32_t, uint32_t, uint32_t>;
-  std::map<Key, uint32_t> at;
-  std::vector<std::vector<uint32_t>> members;
-  std::vector<uint32_t> widths(ms.size());
-  // copies of one shape go together, as misaligned as the worst of them: in an
-  // All-to-all of odd chunks one pair of ranks in eight happens to agree, and a
-  // launch of its own costs its ramp (64 ranks x 1 MiB of BF16: 27.5 us with
-  // it, 25.1 us without)
-  std::map<std::pair<unsigned long long, size_t>, uint32_t> shape;
-  for (size_t i = 0; i < ms.size(); ++i) {
-    widths[i] = width_log2(ms[i]);
-    if (ms[i].src.size() > 1) continue;
-    uint32_t &w = shape.emplace(std::make_pair(ms[i].nbytes, ms[i].dst.size()), widths[i]).first->second;
-    w = std::min(w, widths[i]);
-  }
-  for (size_t i = 0; i < ms.size(); ++i) {
-    if (ms[i].src.size() == 1) widths[i] = shape[{ms[i].nbytes, ms[i].dst.size()}];
-    const Key k(ms[i].nbytes, ms[i].src.size(), ms[i].dst.size(), ms[i].rop, ms[i].tok, widths[i]);
-    auto it = at.emplace(k, (uint32_t)members.size()).first;
-    if (it->second == members.size()) members.emplace_back();
-    members[it->second].push_back((uint32_t)i);
-  }
-  for (const std::vector<uint32_t> &v : members) {
-    const Member &m0 = ms[v[0]];
-    SweepClass k{};
-    k.nbytes = m0.nbytes;
-    k.ptr = sw.ptrs.size();
-    k.nmem = (uint32_t)v.size();
-    k.nsrc = (uint32_t)m0.src.size();
-    k.ndst = (uint32_t)m0.dst.size();
-    k.tok = m0.tok;
-    k.team = m0.team;
-    k.ttok = m0.ttok;
-    k.meta = sweep_meta((uint32_t)c.dtype, m0.rop, widths[v[0]], 1, 0);
-    for (uint32_t i : v) {
-      sw.ptrs.insert(sw.ptrs.end(), ms[i].src.begin(), ms[i].src.end());
-      sw.ptrs.insert(sw.ptrs.end(), ms[i].dst.begin(), ms[i].dst.end());
+    if (with == NONE) {
+      member_of[i] = (uint32_t)ms.size();
+      ms.push_back(m);
+      continue;
     }
-    sw.classes.push_back(k);
+    // the copy's source has to hold the expression's value
+    Member &x = ms[with];
+    auto stored = [&](unsigned long long a) {
+      return std::find(ops.begin() + x.dst, ops.begin() + x.dst + x.ndst, a) != ops.begin() + x.dst + x.ndst;
+    };
+    const unsigned long long from = ops[m.src];
+    if (m.nsrc != 1 || !(stored(from) || (x.nsrc == 1 && ops[x.src] == from))) return;
+    member_of[i] = with;
+    // its destinations follow those that the expression has; a list without
+    // room moves to the end, with room for as many again
+    mine.clear();
+    for (uint32_t k = m.dst; k < m.dst + m.ndst; ++k)
+      if (!again || !stored(ops[k])) mine.push_back(ops[k]);
+    ops.resize(ops0);
+    const uint32_t all = x.ndst + (uint32_t)mine.size();
+    if (all > x.room) {
+      x.room = std::max(all, 2 * x.ndst);
+      ops.resize(ops0 + x.room);
+      std::copy_n(ops.begin() + x.dst, x.ndst, ops.begin() + ops0);
+      x.dst = (uint32_t)ops0;
+    }
+    std::copy(mine.begin(), mine.end(), ops.begin() + x.dst + x.ndst);
+    x.ndst = all;
   }
-  sw.valid = true;
-  plan_launches(sw);
+  make_classes(c, ms, ops, sw);
 }
 
 void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw) {

@@ -431,3 +431,30 @@ def test_pipeline_slots_match_the_oracle(name, P, h, s, m, ring):
     plan = factorize(prog, h, s, m, ring)
     assert comm.plan_info()["slots"] == plan.slots()
     assert comm.plan_info()["stages"] == plan.stages()
+
+
+@pytest.mark.parametrize("P", [8, 40, 64])
+def test_races_among_many_operands(P):
+    """The race check of a few and of thousands of operands (which it sorts in
+    two ways): neighbours that touch are no race, one byte range too long is,
+    and the two primitives are named."""
+    from paper_2408_05962_gb300 import hiccl as H
+    d = 16
+
+    def compose(grow):
+        comm = H.Comm(P, "f32")
+        for i in range(P):
+            for j in range(P):                               # an All-to-all, rows side by side
+                send, recv = [0] * P, [0] * P
+                send[i] = 0x7f0000000000 + 4 * d * (P * i + j)
+                recv[j] = 0x7f8000000000 + 4 * d * (P * j + i)
+                comm.add_multicast(send, recv, d + (grow and (i, j) == (P // 2, P - 1)), i, [j])
+        return comm
+
+    compose(False).plan([P], 1, 1)
+    comm = compose(True)
+    with pytest.raises(H.HicclError) as e:
+        comm.plan([P], 1, 1)
+    assert e.value.status == H.ERR_RACE
+    a, b = P // 2 * P + P - 1, (P // 2 + 1) * P + P - 1      # the next sender's chunk of the same row
+    assert f"primitives {a} and {b} overlap" in H.hiccl_last_error(comm.handle)
