@@ -357,7 +357,11 @@ hiccl_status_t hiccl_get_trace(hiccl_comm_t comm, unsigned long long *out, size_
  * user-buffer operand lies in its primitive's registered ranges and every
  * relay operand in the relay arena; the work-item entries of each step tile
  * its segments exactly once; no item mixes pipeline slots or exceeds 64
- * entries; the runs of an item cover its entries.  HICCL_ERR_INVALID with the
+ * entries; the runs of an item cover its entries.  And of the sweep, if there
+ * is one: every operand lies in the primitives' registered ranges (destinations
+ * in written ones) and is aligned as its kernel's accesses are; the units tile
+ * every class once; the expressions save and take back values in balance and
+ * fit the space for them; the hints name the classes.  HICCL_ERR_INVALID with the
  * first violation in hiccl_last_error; HICCL_ERR_STATE without a plan. */
 hiccl_status_t hiccl_validate(hiccl_comm_t comm);
 
@@ -405,8 +409,11 @@ hiccl_status_t hiccl_debug_sweep(hiccl_comm_t comm, void *out, size_t capacity, 
 /* Host-side fault injection for tests of hiccl_validate: corrupt the host
  * copy of a planned (hiccl_plan, not uploaded) table.  what = 0: make a step
  * depend on a later step (a cycle); 1: move a user-buffer operand out of its
- * primitive's buffers; 2: drop the last entry's segments.  Nothing of it
- * reaches the GPU: hiccl_init on the corrupted communicator is refused. */
+ * primitive's buffers; 2: drop the last entry's segments; of the sweep, 3:
+ * move an operand out of the buffers; 4: drop a unit; 5: unbalance an
+ * expression; 6: empty a section of a fold in two steps.  Nothing of it reaches
+ * the GPU: hiccl_init, hiccl_group and hiccl_run_static refuse the corrupted
+ * plan. */
 hiccl_status_t hiccl_debug_corrupt(hiccl_comm_t comm, int what);
 
 /* Fault injection for tests: add `extra` (0 restores) phantom dependencies to

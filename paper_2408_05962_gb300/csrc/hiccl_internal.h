@@ -337,6 +337,7 @@ struct Plan {
   unsigned long long stages = 0, slots = 0;
   Sweep sweep;
   bool valid = false;
+  bool corrupted = false;                  // by hiccl_debug_corrupt: never runs
 };
 
 // Host image of the executor's read-only arrays for a plan whose relay
@@ -405,6 +406,9 @@ hiccl_status_t guarded(hiccl_comm *c, F &&body) noexcept {
 void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int ring_lvl,
                  const Ranges &ranges, const std::vector<Conflict> &conflicts, Sweep &sw);
 void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw);
+// Consistency of a sweep before it reaches the GPU (ranges: of c's program,
+// empty for a group); false with the first violation in `why`.
+bool check_sweep(const hiccl_comm &c, const Ranges &ranges, const Sweep &sw, std::string &why);
 // factorize c's program again (hiccl_plan.cpp), keeping c's state
 hiccl_status_t replan(hiccl_comm *c, const std::vector<int> &hierarchy, int stripe, int pipeline);
 // runtime entry points (hiccl_runtime.cu)

@@ -148,6 +148,9 @@ struct Builder {
     }
   };
   std::vector<Scratch> scr;
+  // branch roots, piece boundaries and leaves of the primitive being emitted
+  std::vector<int> ks, others, branch;
+  std::vector<unsigned long long> bd;
   std::vector<int> grp;   // grp[l * P + r] = r / G[l + 1] (level-l subgroup of rank r)
 
   Builder(const hiccl_comm &comm, const std::vector<int> &hier, int stripe, int pipeline)
@@ -307,8 +310,9 @@ struct Builder {
   // the s branch roots of a primitive (Sec. 4.3): offsets o, o+1, ..., o+s-1
   // (mod G) of the root's smallest enclosing group of G >= s ranks; a primitive
   // whose leaves all lie in that group is not striped
-  std::vector<int> stripe_ranks(int root, const std::vector<int> &leaves) const {
-    if (s == 1) return {root};
+  void stripe_ranks(int root, const std::vector<int> &leaves, std::vector<int> &ks) const {
+    ks.assign(1, root);
+    if (s == 1) return;
     int l = L;
     while (G[l] < s) --l;   // smallest enclosing group with >= s ranks
     long long g = G[l];
@@ -316,10 +320,9 @@ struct Builder {
     bool all_inside = true;
     for (int r : leaves)
       if (r < base || r >= base + g) { all_inside = false; break; }
-    if (all_inside) return {root};
-    std::vector<int> ks(s);
+    if (all_inside) return;
+    ks.resize(s);
     for (int b = 0; b < s; ++b) ks[b] = (int)(base + (o + b) % g);
-    return ks;
   }
 
   // ---- multicast tree: deliver from `holder` to every rank of `leaves` ---------
@@ -495,30 +498,29 @@ struct Builder {
 
   // piece boundaries (Sec. 4.5): count cut into `parts` pieces at
   // min(count, roundup(ceil(count * k / parts), q)), q the 16-byte quantum
-  std::vector<unsigned long long> bounds(size_t count, int parts) const {
+  void bounds(size_t count, int parts, std::vector<unsigned long long> &b) const {
     unsigned long long q = quantum_of(c.dtype);
-    std::vector<unsigned long long> b(parts + 1);
-    for (int k = 0; k <= parts; ++k) {
+    b.assign(parts + 1, 0);
+    b[parts] = count;
+    for (int k = 1; k < parts; ++k) {
       unsigned __int128 num = (unsigned __int128)count * (unsigned)k;
       unsigned long long v = (unsigned long long)((num + parts - 1) / parts);
       v = (v + q - 1) / q * q;
       b[k] = std::min<unsigned long long>(v, count);
     }
-    return b;
   }
 
   // M(root, leaves, count) (Sec. 3.1) as s striped branches of m channels:
   // stage 0 copies piece b to stripe rank k_b, which multicasts it (Sec. 4.3)
   void multicast(const Prim &pr) {
-    std::vector<int> ks = stripe_ranks(pr.root, pr.leaves);
+    stripe_ranks(pr.root, pr.leaves, ks);
     int nb = (int)ks.size();
-    auto bd = bounds(pr.count, nb * m);
+    bounds(pr.count, nb * m, bd);
     bool leaf_root = std::binary_search(pr.leaves.begin(), pr.leaves.end(), pr.root);
     bool self_copy = leaf_root && pr.recv[pr.root] != pr.send[pr.root];
-    std::vector<int> others;
+    others.clear();
     for (int j : pr.leaves)
       if (j != pr.root) others.push_back(j);
-    std::vector<int> branch;
     for (int b = 0; b < nb; ++b) {
       const int k = ks[b];
       if (k != pr.root) {   // the leaves of branch b: all but k (the root too, unless in place)
@@ -551,9 +553,9 @@ struct Builder {
   // R(leaves, root, count) (Sec. 3.1), the mirror: piece b is reduced at
   // stripe rank k_b and copied to the root (Sec. 4.3)
   void reduction(const Prim &pr) {
-    std::vector<int> ks = stripe_ranks(pr.root, pr.leaves);
+    stripe_ranks(pr.root, pr.leaves, ks);
     int nb = (int)ks.size();
-    auto bd = bounds(pr.count, nb * m);
+    bounds(pr.count, nb * m, bd);
     for (int b = 0; b < nb; ++b) {
       for (int ch = 0; ch < m; ++ch) {
         unsigned long long lo = bd[b * m + ch], hi = bd[b * m + ch + 1];
@@ -935,8 +937,9 @@ void build_image(const Plan &p, unsigned long long relay_base, TableImage &im) {
 // every relay operand inside the relay arena; the entries of each step tile
 // its segments exactly once, in order; no item mixes slots (an item never
 // waits on itself) or exceeds its entry bound; the runs of each item cover
-// its entries' bytes.  Returns false with a message on the first violation.
-bool validate_plan(const hiccl_comm &c, const Plan &p, std::string &msg) {
+// its entries' bytes.  A sweep has to pass check_sweep.  Returns false with a
+// message on the first violation.
+bool validate_plan(const hiccl_comm &c, const Ranges &ranges, const Plan &p, std::string &msg) {
   const size_t N = p.steps.size();
   auto bad = [&](const std::string &m) {
     msg = m;
@@ -1014,7 +1017,7 @@ bool validate_plan(const hiccl_comm &c, const Plan &p, std::string &msg) {
     }
     if (rbytes != bytes) return bad("runs of item " + std::to_string(it) + " do not cover its entries");
   }
-  return true;
+  return !p.sweep.valid || check_sweep(c, ranges, p.sweep, msg);
 }
 
 static hiccl_status_t build_plan(hiccl_comm *c, const int *hierarchy, int nlevels, int stripe,
@@ -1329,7 +1332,7 @@ static hiccl_status_t build_plan(hiccl_comm *c, const int *hierarchy, int nlevel
   plan.valid = true;
   {
     std::string why;
-    if (!validate_plan(*c, plan, why)) return fail(c, HICCL_ERR_INVALID, "internal plan check: " + why);
+    if (!validate_plan(*c, ranges, plan, why)) return fail(c, HICCL_ERR_INVALID, "internal plan check: " + why);
   }
   c->plan = std::move(plan);
   return HICCL_OK;
@@ -1580,6 +1583,7 @@ hiccl_status_t hiccl_init(hiccl_comm_t c, const int *hierarchy, int nlevels, int
     const bool same = c->state == hiccl_comm::PLANNED && c->plan.valid && hierarchy && nlevels >= 1 &&
                       c->plan.hierarchy == std::vector<int>(hierarchy, hierarchy + nlevels) &&
                       c->plan.stripe == stripe && c->plan.pipeline == pipeline;
+    if (same && c->plan.corrupted) return fail(c, HICCL_ERR_INVALID, "plan check: the table was corrupted");
     hiccl_status_t st = same ? HICCL_OK : build_plan(c, hierarchy, nlevels, stripe, pipeline);
     if (st != HICCL_OK) return st;
     c->state = hiccl_comm::PLANNED;
@@ -1597,6 +1601,7 @@ static hiccl_status_t group_build(const hiccl_comm_t *comms, int n, hiccl_comm *
   unsigned long long segb = 0;
   for (int i = 0; i < n; ++i) {
     if (!comms[i] || !comms[i]->plan.valid) return HICCL_ERR_STATE;
+    if (comms[i]->plan.corrupted) return HICCL_ERR_INVALID;
     if (segb && comms[i]->plan.seg != segb) return HICCL_ERR_UNSUPPORTED;   // FP8 with other payloads
     segb = comms[i]->plan.seg;
   }
@@ -1688,7 +1693,7 @@ static hiccl_status_t group_build(const hiccl_comm_t *comms, int n, hiccl_comm *
   P.valid = true;
   {
     std::string why;
-    if (!validate_plan(*g, P, why)) return HICCL_ERR_INVALID;
+    if (!validate_plan(*g, Ranges(), P, why)) return HICCL_ERR_INVALID;
   }
   g->state = hiccl_comm::PLANNED;
   *out = owner.release();
@@ -1748,7 +1753,9 @@ hiccl_status_t hiccl_validate(hiccl_comm_t c) {
     if (!c) return HICCL_ERR_INVALID;
     if (!c->plan.valid) return fail(c, HICCL_ERR_STATE, "no plan");
     std::string why;
-    if (!validate_plan(*c, c->plan, why)) return fail(c, HICCL_ERR_INVALID, "plan check: " + why);
+    Ranges ranges;
+    collect_ranges(*c, ranges);
+    if (!validate_plan(*c, ranges, c->plan, why)) return fail(c, HICCL_ERR_INVALID, "plan check: " + why);
     return HICCL_OK;
   });
 }
@@ -1802,12 +1809,19 @@ hiccl_status_t hiccl_debug_corrupt(hiccl_comm_t c, int what) {
       return fail(c, HICCL_ERR_STATE, "needs a planned communicator that is not uploaded");
     Plan &p = c->plan;
     const size_t N = p.steps.size();
+    Sweep &sw = p.sweep;
+    if (what >= 3 && what <= 6 && (!sw.valid || sw.classes.empty())) return fail(c, HICCL_ERR_INVALID, "no sweep");
+    const auto fold = std::find_if(sw.classes.begin(), sw.classes.end(), [](const SweepClass &k) { return k.nsrc > 1; });
+    auto done = [&]() {
+      p.corrupted = true;
+      return HICCL_OK;
+    };
     switch (what) {
       case 0: {   // a dependency on a later step: a cycle in the dependency graph
         for (size_t i = 0; i + 1 < N; ++i)
           if (p.pred_off[i + 1] > p.pred_off[i]) {
             p.preds[p.pred_off[i]] = (uint32_t)(N - 1);
-            return HICCL_OK;
+            return done();
           }
         return fail(c, HICCL_ERR_INVALID, "no step with a predecessor");
       }
@@ -1816,15 +1830,29 @@ hiccl_status_t hiccl_debug_corrupt(hiccl_comm_t c, int what) {
           for (uint32_t k = 0; k < st.nsrc + st.ndst; ++k)
             if (!p.locs[st.loc0 + k].scratch) {
               p.locs[st.loc0 + k].addr += (unsigned long long)c->prims[st.prim].count * c->esize + 4096;
-              return HICCL_OK;
+              return done();
             }
         return fail(c, HICCL_ERR_INVALID, "no user operand");
       }
       case 2: {   // the last entry of a step dropped: segments left uncovered
         if (p.entries.empty()) return fail(c, HICCL_ERR_INVALID, "no entries");
         p.entries.back().seg_hi = p.entries.back().seg_lo;
-        return HICCL_OK;
+        return done();
       }
+      case 3:   // the sweep's last operand, a destination, moved out of the buffers
+        sw.ptrs.back() += 1ull << 40;
+        return done();
+      case 4:   // a unit of the sweep's last class dropped
+        --sw.classes.back().upm;
+        return done();
+      case 5:   // an expression that takes back a value it never saved
+        if (fold == sw.classes.end()) return fail(c, HICCL_ERR_INVALID, "no fold");
+        sw.toks[fold->tok] |= TOK_POP << TOK_OPS;
+        return done();
+      case 6:   // an empty section in a fold of two steps
+        if (fold == sw.classes.end() || fold->team < 2) return fail(c, HICCL_ERR_INVALID, "no fold in two steps");
+        sw.toks[fold->ttok + fold->nsrc + 1] = 0;
+        return done();
       default:
         return fail(c, HICCL_ERR_INVALID, "unknown corruption");
     }

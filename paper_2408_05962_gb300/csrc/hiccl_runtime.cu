@@ -1460,6 +1460,7 @@ extern "C" hiccl_status_t hiccl_run_static(hiccl_comm_t c, void *stream) {
   return guarded(c, [&]() -> hiccl_status_t {
     if (!c) return HICCL_ERR_INVALID;
     if (!c->plan.valid) return HICCL_ERR_STATE;
+    if (c->plan.corrupted) return fail(c, HICCL_ERR_INVALID, "plan check: the table was corrupted");
     const Plan &p = c->plan;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const unsigned long long N = p.steps.size();

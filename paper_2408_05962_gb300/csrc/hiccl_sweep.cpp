@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <map>
+#include <string>
 #include <tuple>
 
 #include "hiccl_internal.h"
@@ -376,6 +377,95 @@ void make_classes(const hiccl_comm &c, const std::vector<Member> &ms, const std:
   plan_launches(sw);
 }
 
+// ---- the check of a sweep ------------------------------------------------------
+
+// Byte ranges joined to disjoint spans.
+struct Bytes {
+  struct Span {
+    unsigned long long lo, hi;
+  };
+  std::vector<Span> v;
+  void join() {
+    std::sort(v.begin(), v.end(), [](const Span &a, const Span &b) { return a.lo < b.lo; });
+    size_t w = 0;
+    for (size_t k = 1; k < v.size(); ++k) {
+      if (v[k].lo <= v[w].hi) v[w].hi = std::max(v[w].hi, v[k].hi);
+      else v[++w] = v[k];
+    }
+    if (!v.empty()) v.resize(w + 1);
+  }
+  // the span that holds [lo, hi), if any
+  const Span *find(unsigned long long lo, unsigned long long hi) const {
+    auto it = std::upper_bound(v.begin(), v.end(), lo, [](unsigned long long a, const Span &s) { return a < s.lo; });
+    return it == v.begin() || hi > (--it)->hi ? nullptr : &*it;
+  }
+};
+// Ranges of nbytes, each mostly in the span of the one that had its hint before.
+struct Inside {
+  static constexpr uint32_t HINTS = 64;
+  struct Hint {
+    unsigned long long lo, room;   // [lo, lo + room) + nbytes
+  };
+  const Bytes &in;
+  const unsigned long long nbytes;
+  Hint hints[HINTS] = {};
+  Inside(const Bytes &b, unsigned long long n) : in(b), nbytes(n) {}
+  bool operator()(unsigned long long a, uint32_t hint) {
+    Hint &h = hints[hint % HINTS];
+    if (a - h.lo < h.room) return true;
+    const Bytes::Span *s = in.find(a, a + nbytes);
+    if (s) h = Hint{s->lo, s->hi - s->lo - nbytes + 1};
+    return s != nullptr;
+  }
+};
+// what a program reads or writes, and what it writes
+void join_ranges(const Ranges &ranges, Bytes &all, Bytes &written) {
+  struct Open {
+    unsigned long long lo = 0, hi = 0;
+  };
+  std::vector<Open> open;   // by rank and direction: its ranges mostly continue one another
+  all.v.reserve(64);
+  written.v.reserve(64);
+  auto close = [&](const Open &o, bool write) {
+    if (o.lo == o.hi) return;
+    all.v.push_back(Bytes::Span{o.lo, o.hi});
+    if (write) written.v.push_back(Bytes::Span{o.lo, o.hi});
+  };
+  for (const Range &r : ranges.all) {
+    const size_t k = 2 * (size_t)r.rank + r.write;
+    if (k >= open.size()) open.resize(k + 64);
+    Open &o = open[k];
+    if (r.lo <= o.hi && r.hi >= o.lo && o.lo != o.hi) {
+      o.lo = std::min(o.lo, r.lo);
+      o.hi = std::max(o.hi, r.hi);
+    } else {
+      close(o, r.write);
+      o.lo = r.lo;
+      o.hi = r.hi;
+    }
+  }
+  for (size_t k = 0; k < open.size(); ++k) close(open[k], k & 1);
+  all.join();
+  written.join();
+}
+
+// Do n tokens start with a value, save and take back in balance and never hold
+// more than `most` values?
+bool balanced(const uint32_t *tok, uint32_t n, uint32_t most) {
+  if (n == 0 || (tok[0] & 3u) != TOK_START) return false;
+  uint32_t sp = 0;
+  for (uint32_t k = 0; k < n; ++k) {
+    if (k && (tok[k] & 3u) == TOK_START) return false;   // would lose the accumulator
+    if ((tok[k] & 3u) == TOK_PUSH) return false;
+    if ((tok[k] & TOK_PUSH) && ++sp > most) return false;
+    for (uint32_t o = tok[k] >> TOK_OPS; o; o >>= 2) {
+      if ((o & 3u) == 0) return false;
+      if ((o & 3u) >= TOK_POP && sp-- == 0) return false;
+    }
+  }
+  return sp == 0;
+}
+
 }  // namespace
 
 // (Every plan pays for its sweep, so this shares the ranges and conflicts that
@@ -480,6 +570,93 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
     x.ndst = all;
   }
   make_classes(c, ms, ops, sw);
+}
+
+bool check_sweep(const hiccl_comm &c, const Ranges &ranges, const Sweep &sw, std::string &why) {
+  auto bad = [&](const std::string &m) {
+    why = "sweep: " + m;
+    return false;
+  };
+  Bytes all, written;   // (a group has no primitives; its members were checked)
+  join_ranges(ranges, all, written);
+  size_t next = 0;       // class
+  for (const SweepLaunch &L : sw.launches) {
+    if (L.class_lo != next || L.class_hi <= L.class_lo || L.class_hi > sw.classes.size() || L.kernel >= SWEEP_KERNELS)
+      return bad("launches do not divide the classes");
+    next = L.class_hi;
+    if (L.threads < 32 || L.threads % 32 || L.threads > SWEEP_THREADS[L.kernel] || L.stack_words > SWEEP_MAX_DEPTH * 16)
+      return bad("a launch has a bad shape");
+    const bool team = L.kernel == SWEEP_TEAM || L.kernel == SWEEP_FP8_TEAM;
+    unsigned long long units = 0;
+    for (size_t i = L.class_lo; i < L.class_hi; ++i) {
+      const SweepClass &k = sw.classes[i];
+      const std::string at = "class " + std::to_string(i);
+      const uint32_t dt = sweep_dtype(k.meta), lw = sweep_lw(k.meta), v = sweep_v(k.meta);
+      const bool fold = k.nsrc > 1, fp8 = dt == HICCL_FP8E4M3;
+      const uint32_t elem = fp8 ? 16 : dt == HICCL_BF16 ? 2 : 4;
+      // a kernel that handles the class
+      bool runs = sweep_kernel(k.meta) == L.kernel && k.nsrc && k.ndst && k.nmem && k.nbytes;
+      switch (L.kernel) {
+        case SWEEP_COPY: runs = runs && !fold && lw >= 4; break;
+        case SWEEP_FOLD: runs = runs && lw >= 4 && !(fold && fp8); break;
+        case SWEEP_FP8: case SWEEP_FP8_TEAM: runs = runs && fold && fp8 && lw >= 4; break;
+        case SWEEP_NARROW: runs = runs && fold && !fp8 && (lw == 2 || (lw == 1 && dt == HICCL_BF16)); break;
+        case SWEEP_SHIFT: runs = runs && !fold; break;
+        default: runs = runs && fold && !fp8 && lw >= 4; break;
+      }
+      if (!runs) return bad(at + " does not fit its kernel");
+      // units that tile the members
+      const unsigned long long unit = row_bytes(L.kernel, k) * v;
+      if (!v || k.unit0 != units || (k.upm - 1ull) * unit >= k.nbytes || k.upm * unit < k.nbytes || !k.group ||
+          (fold && k.group != k.ndst))
+        return bad("units of " + at + " do not tile it");
+      units += (unsigned long long)k.upm * k.nmem * ((k.ndst + k.group - 1) / k.group);
+      // operands inside the buffers, as far off a boundary as the kernel's accesses allow
+      const unsigned long long n = (unsigned long long)k.nsrc + k.ndst;
+      if (k.ptr > sw.ptrs.size() || k.nmem > (sw.ptrs.size() - k.ptr) / n) return bad("operands of " + at + " are missing");
+      Inside readable(all, k.nbytes), writable(written, k.nbytes);
+      const unsigned long long mask = (1ull << lw) - 1;
+      for (uint32_t m = 0; m < k.nmem; ++m) {
+        const unsigned long long *p = &sw.ptrs[k.ptr + m * n];
+        bool in = true;
+        unsigned long long off = 0, low = 0;
+        // (neighbouring members of a fold read the same rows, copies write every row in turn)
+        for (uint32_t q = 0; q < k.nsrc; ++q) in = in && (c.group || readable(p[q], q));
+        for (uint32_t q = k.nsrc; q < n; ++q) in = in && (c.group || writable(p[q], n == 2 ? m : q));
+        if (!in) return bad("an operand of " + at + " lies outside the primitives' buffers");
+        for (uint32_t q = 0; q < n; ++q) off |= p[q] ^ p[0], low |= p[q];
+        if (((low | k.nbytes) & (elem - 1)) || ((lw >= 4 ? off : fold ? low | k.nbytes : 0) & mask))
+          return bad("operands of " + at + " are not aligned");
+      }
+      if (!fold) continue;
+      // expressions that fit the saved values
+      const uint32_t acc = fp8 ? 16 : lw >= 4 ? (dt == HICCL_BF16 ? 8 : 4) : lw == 2 && dt == HICCL_BF16 ? 2 : 1;
+      const uint32_t most = L.stack_words / (acc * v);
+      if (k.tok > sw.toks.size() || k.nsrc > sw.toks.size() - k.tok || !balanced(&sw.toks[k.tok], k.nsrc, most))
+        return bad("tokens of " + at + " are not an expression");
+      if (!team) continue;
+      const size_t need = (size_t)k.nsrc + 2 * k.team + 1;
+      if (k.team < 2 || k.team > SWEEP_TEAM_MAX || k.ttok > sw.toks.size() || need > sw.toks.size() - k.ttok)
+        return bad("the two steps of " + at + " are missing");
+      const uint32_t *t = &sw.toks[k.ttok], *b = t + k.nsrc;
+      bool good = b[0] == 0 && b[k.team] == k.nsrc && balanced(b + k.team + 1, k.team, most);
+      for (uint32_t s = 0; s < k.team && good; ++s)
+        good = b[s] < b[s + 1] && b[s + 1] <= k.nsrc && balanced(t + b[s], b[s + 1] - b[s], most);
+      if (!good) return bad("the two steps of " + at + " are not an expression");
+    }
+    if (units != L.units) return bad("a launch has another number of units than its classes");
+    if (L.class_hi - L.class_lo > SWEEP_PREFIX) {   // every unit's class lies between two hints
+      const size_t nh = (size_t)((units - 1) >> SWEEP_HINT_SHIFT) + 2, nc = L.class_hi - L.class_lo;
+      if (L.hint > sw.hints.size() || nh > sw.hints.size() - L.hint) return bad("hints are missing");
+      const SweepClass *k = &sw.classes[L.class_lo];
+      for (size_t i = 0; i < nh; ++i) {
+        const size_t h = sw.hints[L.hint + i];
+        const unsigned long long u = (unsigned long long)i << SWEEP_HINT_SHIFT;
+        if (h >= nc || k[h].unit0 > u || (h + 1 < nc && k[h + 1].unit0 <= u)) return bad("a hint names a wrong class");
+      }
+    }
+  }
+  return next == sw.classes.size() || bad("launches do not divide the classes");
 }
 
 void group_sweep(const std::vector<const Sweep *> &members, Sweep &sw) {

@@ -315,3 +315,32 @@ def test_group_sweep_is_the_union():
     assert sum(k["nmem"] for k in cls) == total
     assert sorted(ptrs) == sorted(p for c in members for p in decode(c.sweep())[2])
     assert [x["kernel"] for x in lau] == [FOLD, TEAM]         # the flat sum is sequential
+
+
+@pytest.mark.parametrize("what,needle", [(3, "outside the primitives' buffers"), (4, "do not tile"),
+                                         (5, "not an expression"), (6, "two steps")])
+def test_corrupted_sweeps_are_caught_on_the_host(what, needle):
+    """What a start launches is checked as the step table is: an operand outside
+    the buffers, a missing unit, an unbalanced expression, an empty section."""
+    prog = PR.reducescatter(16, 37)
+    comm = register(prog, FakeAddresses(prog).addr)
+    comm.plan([4, 4], 2, 2)
+    comm.validate()
+    comm.corrupt(what)
+    with pytest.raises(H.HicclError) as e:
+        comm.validate()
+    assert e.value.status == H.ERR_INVALID
+    assert needle in H.hiccl_last_error(comm.handle)
+
+
+@pytest.mark.parametrize("what", range(7))
+def test_corrupted_plans_do_not_run(what):
+    """A corrupted plan is refused before any CUDA call, by itself and in a group."""
+    prog = PR.allreduce(16, 37)
+    comm = register(prog, FakeAddresses(prog).addr)
+    comm.plan([4, 4], 2, 2)
+    comm.corrupt(what)
+    for run in (lambda: comm.init([4, 4], 2, 2), comm.run_static, lambda: H.Comm.group_plan([comm])):
+        with pytest.raises(H.HicclError) as e:
+            run()
+        assert e.value.status == H.ERR_INVALID
