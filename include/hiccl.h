@@ -391,7 +391,7 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
  * sources, destinations, first token, meta, destinations per unit, sections,
  * first token of the two-step form, 0, 0); the
  * launches (32 bytes: u32 kernel, first and end class, units, threads, saved
- * words per thread, first hint, 0); the pointers (u64; per member its sources in evaluation order, then its
+ * words per thread, first hint, most sections of a class in two steps); the pointers (u64; per member its sources in evaluation order, then its
  * destinations); the tokens (u32, one per source: bit 0 the source starts the
  * accumulator, bit 1 after the old one was saved, else it is combined in;
  * then two-bit operations from bit 8 on: 1 round the accumulator to the

@@ -181,7 +181,9 @@ enum : uint32_t {
 constexpr uint32_t SWEEP_GROUP = 2, SWEEP_TILE = 8192;
 constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128, 512, 256};   // most threads of a CTA
 
-constexpr uint32_t SWEEP_TEAM_MAX = 32;    // sections of an expression
+// Sections of an expression: their values take 512 bytes (FP8 576) of shared
+// memory each.  (With at most 32, one warp folded all 512 sources of {64, 8}.)
+constexpr uint32_t SWEEP_TEAM_MAX = 128;
 // In a fold pass of few units every warp folds one source after the other,
 // about 300 cycles each, while most of an SM idles: below eight units an SM
 // the sections go to the warps of a CTA, as many as fill the SMs
@@ -189,6 +191,14 @@ constexpr uint32_t SWEEP_TEAM_MAX = 32;    // sections of an expression
 // x 64 KiB 12.7 / 9.4 us, Reduce of 64 ranks x 16 KiB 10.8 / 6.1 us; at 1024
 // units (16 ranks x 512 KiB) 7.3 / 5.2 us, at 2048 (1 MiB) 8.6 / 10.6 us.
 constexpr uint32_t SWEEP_TEAM_UNITS = 152 * 8, SWEEP_TEAM_WARPS = 152 * 32;
+// More than 32 sections: every warp evaluates the expression of all their values,
+// so the lines lie earlier.  Reduce, F32, by one warp / by 64 sections of {64, 8}
+// (us): 2 units 67 / 14, 128 units 67 / 16, 512 76 / 39; 128 of {128, 8}: 132 / 25,
+// 133 / 29, 146 / 73, 1024 units 148 / 164; 50 of {50, 2}, BF16: 512 units 26.8 / 29.3.
+// Where a level has fewer sections, by 2 or 64 of {2, 32, 4}: 1 unit 32 / 12, 128
+// 32 / 14; by 4 or 64 of {4, 16, 4}: 512 units 22 / 23.  FP8 values take as long to
+// fold as sources, so there fewer stay better: {4, 16, 4}, 128 units, 22.5 / 27.7.
+constexpr uint32_t SWEEP_TEAM_MANY = 152 * 3, SWEEP_TEAM_FEW = 152 * 2;
 
 // token of one source, in evaluation order: START the accumulator with it
 // (first saving the old one when PUSH is set), else combine it; then up to
@@ -243,7 +253,7 @@ struct SweepLaunch {
   uint32_t threads;
   uint32_t stack_words;        // 32-bit words of saved values per thread
   uint32_t hint;               // first hint
-  uint32_t pad;
+  uint32_t sections;           // of the class that has most (launches of teams)
 };
 
 // ---------------------------------------------------------------------------

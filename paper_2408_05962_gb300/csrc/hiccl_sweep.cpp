@@ -143,11 +143,10 @@ struct Program {   // an expression shared by members: evaluation order and toke
 };
 
 // The two-step form of a program's expression (see SweepClass::team): the
-// groups of the level that makes a section and the list of sections shortest
-// together, or equal parts where the operator is exact (the order of exact
+// groups of one level, or equal parts where the operator is exact (the order of exact
 // operations does not change the result).  Returns the number of sections (0: none) and
 // appends their tokens, bounds and the tokens of their values.
-uint32_t two_steps(const std::vector<int> &h, const std::vector<int> &leaves, bool rounds, bool exact, bool chained,
+uint32_t two_steps(const std::vector<int> &h, const std::vector<int> &leaves, bool rounds, bool exact, bool chained, bool few,
                    std::vector<uint32_t> &toks, uint32_t &depth) {
   const uint32_t n = (uint32_t)leaves.size();
   if (n < 8 || (chained && !exact)) return 0;
@@ -164,12 +163,19 @@ uint32_t two_steps(const std::vector<int> &h, const std::vector<int> &leaves, bo
     std::vector<int> reps;
     Expr top(h, reps, rounds);
     int level = -1;
+    // the level that makes a section and the list of sections shortest together;
+    // with more than 32 sections where there is no other, or in a pass of few
+    // units where that leaves fewer sources in series: those of the sections
+    // that a warp takes in turn, and the values, which come from shared memory
+    // and take two thirds of the time
+    auto series = [&](uint32_t T) { return 3 * ((T + 15) / 16 * ((n + T - 1) / T)) + 2 * T; };
     for (int l = 0; l < (int)h.size(); ++l) {
       std::vector<uint32_t> b;
       for (size_t a = 0; a < n; a = top.next_in(leaves, a, n, l)) b.push_back((uint32_t)a);
-      if (b.size() > SWEEP_TEAM_MAX || b.size() == n) break;
-      if (b.size() < 2) continue;
-      if (level >= 0 && n / b.size() + b.size() >= n / bounds.size() + bounds.size()) continue;
+      const uint32_t T = (uint32_t)b.size(), T0 = (uint32_t)bounds.size();
+      if (T > SWEEP_TEAM_MAX || T == n) break;
+      if (T < 2) continue;
+      if (level >= 0 && (T <= 32 ? n / T + T >= n / T0 + T0 : !few || series(T) >= series(T0))) continue;
       level = l;
       bounds = b;
     }
@@ -241,7 +247,9 @@ void plan_launches(Sweep &sw) {
   auto folded = [](const SweepClass &k) { return k.nsrc > 1 && sweep_lw(k.meta) >= 4; };
   for (const SweepClass &k : sw.classes)
     if (folded(k)) fold_units += (k.nbytes + row_bytes(fold_kernel(k), k) - 1) / row_bytes(fold_kernel(k), k) * k.nmem;
-  auto teamed = [&](const SweepClass &k) { return k.team > 1 && fold_units < SWEEP_TEAM_UNITS; };
+  auto teamed = [&](const SweepClass &k) {
+    return k.team > 1 && fold_units < (k.team > 32 ? SWEEP_TEAM_MANY : SWEEP_TEAM_UNITS);
+  };
   for (const SweepClass &k : sw.classes) folds |= folded(k) && !teamed(k) && fold_kernel(k) == SWEEP_FOLD;
   auto kernel_of = [&](const SweepClass &k) -> uint32_t {
     if (sweep_lw(k.meta) < 4) return k.nsrc > 1 ? SWEEP_NARROW : SWEEP_SHIFT;
@@ -299,7 +307,8 @@ void plan_launches(Sweep &sw) {
     while (!team && warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
     // a team's warps: no more than sections, and enough for SWEEP_TEAM_WARPS in all
     uint32_t sections = 1;
-    for (size_t i = a; i < z; ++i) sections = std::max(sections, sw.classes[i].team);
+    for (size_t i = a; team && i < z; ++i) sections = std::max(sections, sw.classes[i].team);
+    L.sections = team ? sections : 0;
     while (team && warps > sections) warps /= 2;
     while (team && warps > 1 && units * (warps / 2) >= SWEEP_TEAM_WARPS) warps /= 2;
     L.threads = warps * 32;
@@ -483,6 +492,11 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
   ms.reserve(c.prims.size());
   ops.reserve(ranges.all.size());
   const long long node_ranks = c.P / c.ring;
+  const unsigned long long row = c.dtype == HICCL_FP8E4M3 ? 4 * FP8_BLOCK_BYTES : 512;
+  unsigned long long units = 0;   // of the folds
+  for (const Prim &p : c.prims)
+    if (p.kind == 1 && p.leaves.size() > 1) units += ((unsigned long long)p.count * c.esize + row - 1) / row;
+  const bool few = c.dtype != HICCL_FP8E4M3 && units < SWEEP_TEAM_FEW;
   size_t next = 0;   // conflict
   for (size_t i = 0; i < c.prims.size(); ++i) {
     const Prim &p = c.prims[i];
@@ -513,7 +527,7 @@ void build_sweep(const hiccl_comm &c, const std::vector<int> &hierarchy, int rin
         const uint32_t tok = (uint32_t)sw.toks.size();
         sw.toks.insert(sw.toks.end(), e.toks.begin(), e.toks.end());
         const uint32_t ttok = (uint32_t)sw.toks.size();
-        const uint32_t team = two_steps(hierarchy, p.leaves, rounds, exact, c.ring > 1, sw.toks, depth);
+        const uint32_t team = two_steps(hierarchy, p.leaves, rounds, exact, c.ring > 1, few, sw.toks, depth);
         sw.depth = std::max(sw.depth, depth);
         progs.push_back(Program{p.leaves, node, rounds, exact, e.order, tok, team, ttok});
         pg = &progs.back();
@@ -636,7 +650,7 @@ bool check_sweep(const hiccl_comm &c, const Ranges &ranges, const Sweep &sw, std
         return bad("tokens of " + at + " are not an expression");
       if (!team) continue;
       const size_t need = (size_t)k.nsrc + 2 * k.team + 1;
-      if (k.team < 2 || k.team > SWEEP_TEAM_MAX || k.ttok > sw.toks.size() || need > sw.toks.size() - k.ttok)
+      if (k.team < 2 || k.team > L.sections || L.sections > SWEEP_TEAM_MAX || k.ttok > sw.toks.size() || need > sw.toks.size() - k.ttok)
         return bad("the two steps of " + at + " are missing");
       const uint32_t *t = &sw.toks[k.ttok], *b = t + k.nsrc;
       bool good = b[0] == 0 && b[k.team] == k.nsrc && balanced(b + k.team + 1, k.team, most);

@@ -565,6 +565,8 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FOLD], 16) sweep_fold_kern
   else fold_member<FOLD_GROUPS_SHORT>(A, u, lane);
 }
 
+constexpr uint32_t TEAM_STATIC = 32;   // sections whose values lie in static shared memory
+
 // A short fold pass: a CTA to a unit.  Its warps evaluate the expression's
 // sections (SweepClass::team), leave their values in shared memory, and after
 // a barrier every warp evaluates the expression of those and stores its share
@@ -608,14 +610,19 @@ __device__ __forceinline__ void team_any(const SweepArgs &A, const Unit &u, unsi
     else team_unit<ANY_32, W>(A, u, off, end, dt, rop, parts, stack);
   }
 }
+// (MANY: more than TEAM_STATIC sections, whose values then lie in dynamic shared
+// memory; with all of them there, small passes take 0.2 to 0.4 us longer, 4.5
+// instead of 4.1 us for a maximum over 8 ranks)
+template <bool MANY>
 __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_TEAM], 2)
     sweep_team_kernel(const __grid_constant__ SweepArgs A) {
-  __shared__ uint4 parts[SWEEP_TEAM_MAX * 32];
+  __shared__ uint4 few[MANY ? 1 : TEAM_STATIC * 32];
   extern __shared__ __align__(16) uint32_t saved[];
   launch_order();
   const int lane = threadIdx.x & 31;
   const Unit u = find_unit(A, blockIdx.x);
-  uint32_t *stack = saved + threadIdx.x;
+  uint4 *parts = MANY ? reinterpret_cast<uint4 *>(saved) : few;
+  uint32_t *stack = saved + (MANY ? A.sections * 128 : 0) + threadIdx.x;
   const Body b = body_of(u.k, u.P);
   team_any<16>(A, u, b.head + (unsigned long long)u.part * 512 + lane * 16, b.end, parts, stack);
   if (u.part + 1 == u.k.upm && b.end - b.head != u.k.nbytes) {
@@ -951,16 +958,19 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(
 }
 
 // a short pass: a CTA to a unit, as sweep_team_kernel
+template <bool MANY>
 __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8_TEAM], 2)
     sweep_fp8_team_kernel(const __grid_constant__ SweepArgs A) {
-  __shared__ __align__(16) char parts[SWEEP_TEAM_MAX * FP8_STEP];
+  __shared__ __align__(16) char few[MANY ? 16 : TEAM_STATIC * FP8_STEP];
   extern __shared__ __align__(16) uint32_t saved[];
   launch_order();
   const Unit u = find_unit(A, blockIdx.x);
   const SweepClass &k = u.k;
+  char *parts = MANY ? reinterpret_cast<char *>(saved) : few;
   const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5, grp = (threadIdx.x & 31) >> 3;
-  char *base = reinterpret_cast<char *>(saved) + warp * (FP8_SLOTS * FP8_STEP);
-  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + warps * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
+  char *rings = reinterpret_cast<char *>(saved) + (MANY ? A.sections * FP8_STEP : 0);
+  char *base = rings + warp * (FP8_SLOTS * FP8_STEP);
+  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(rings + warps * (FP8_SLOTS * FP8_STEP)) + threadIdx.x;
   const uint32_t *tok = A.toks + k.ttok, *bounds = tok + k.nsrc, *upper = bounds + k.team + 1;
   Fp8Ring ring;
   fp8_ring_at(ring, u, base);
@@ -983,18 +993,28 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8_TEAM], 2)
 
 typedef void (*Kernel)(const SweepArgs);
 const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel,
-                                         sweep_shift_kernel, sweep_team_kernel, sweep_fp8_team_kernel};
+                                         sweep_shift_kernel, sweep_team_kernel<false>, sweep_fp8_team_kernel<false>};
+Kernel kernel_of(const SweepLaunch &L) {
+  if (L.sections <= TEAM_STATIC) return KERNELS[L.kernel];
+  return L.kernel == SWEEP_FP8_TEAM ? sweep_fp8_team_kernel<true> : sweep_team_kernel<true>;
+}
 
 }  // namespace
 
 // dynamic shared memory: at most SWEEP_MAX_DEPTH saved values of 16 words for
-// each of 256 threads beside the rings of eight warps; more than half an SM's
-// keeps a second CTA off it
-constexpr size_t SWEEP_MAX_SMEM = SWEEP_MAX_DEPTH * 16 * 4 * 256 + 8 * FP8_SLOTS * FP8_STEP, SWEEP_HALF_SM = 120 * 1024;
+// each of 256 threads beside the rings of eight warps, and the values of many
+// sections; more than half an SM's keeps a second CTA off it
+constexpr size_t SWEEP_MAX_SMEM = SWEEP_MAX_DEPTH * 16 * 4 * 256 + 8 * FP8_SLOTS * FP8_STEP, SWEEP_HALF_SM = 120 * 1024,
+                 SWEEP_MANY_SMEM = SWEEP_MAX_SMEM + SWEEP_TEAM_MAX * FP8_STEP;
+static_assert(SWEEP_MANY_SMEM <= 227 * 1024, "a CTA's shared memory");
 
 cudaError_t sweep_prepare() {
   for (uint32_t i = 0; i < SWEEP_KERNELS; ++i) {
     const cudaError_t e = cudaFuncSetAttribute(KERNELS[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_MAX_SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  for (Kernel k : {Kernel(sweep_team_kernel<true>), Kernel(sweep_fp8_team_kernel<true>)}) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_MANY_SMEM);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1008,6 +1028,8 @@ cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_
   cfg.dynamicSmemBytes = (size_t)L.stack_words * 4 * L.threads;
   if (L.kernel == SWEEP_FP8 || L.kernel == SWEEP_FP8_TEAM) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;
   SweepArgs B = A;
+  B.sections = L.sections;
+  if (L.sections > TEAM_STATIC) cfg.dynamicSmemBytes += L.sections * (L.kernel == SWEEP_FP8_TEAM ? FP8_STEP : 512);
   if (L.kernel == SWEEP_FOLD) {
     B.groups = L.units < SHORT_UNITS ? FOLD_GROUPS_SHORT : FOLD_GROUPS;
     cfg.dynamicSmemBytes += warps * B.groups * RING_GROUP * 512;
@@ -1019,7 +1041,7 @@ cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, KERNELS[L.kernel], B);
+  return cudaLaunchKernelEx(&cfg, kernel_of(L), B);
 }
 
 }  // namespace hiccl

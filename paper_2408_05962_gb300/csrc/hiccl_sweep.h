@@ -15,6 +15,7 @@ struct SweepArgs {
   uint32_t nclass;
   uint32_t units;
   uint32_t groups = 0;                  // of a fold's ring
+  uint32_t sections = 0;                // whose values a team's CTA holds
   unsigned long long minus0 = 0x8000000080000000ull;   // two binary32 -0 (see mul2)
   uint32_t unit0[SWEEP_PREFIX];         // first units, for searching without a memory access
   SweepClass first[SWEEP_INLINE];       // the classes themselves, where there are few
