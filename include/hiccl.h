@@ -314,8 +314,8 @@ typedef enum {
 } hiccl_option_t;
 
 /* Set an option.  None changes a result bit but RING.  The options shape the
- * step executor; a sweep heeds CTAS_PER_SM = 1 (one CTA on an SM at a time)
- * and TRACE, which has the communicator run step by step.
+ * step executor; a sweep heeds CTAS_PER_SM = 1 (one CTA of at most 512
+ * threads on an SM at a time) and TRACE, which has the communicator run step by step.
  * TIMEOUT_NS, CTAS_PER_SM and THREADS apply to the next start
  * (a start whose grid differs from the previous start's begins from zeroed
  * dependency counters; a CUDA graph that recorded a start before such a

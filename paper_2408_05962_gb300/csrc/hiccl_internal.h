@@ -180,6 +180,7 @@ enum : uint32_t {
 // 16 MiB: 43.1 / 42.5 / 41.2 / 42.4 / 45.9 us.
 constexpr uint32_t SWEEP_GROUP = 2, SWEEP_TILE = 8192;
 constexpr uint32_t SWEEP_THREADS[SWEEP_KERNELS] = {128, 64, 128, 64, 128, 512, 256};   // most threads of a CTA
+constexpr uint32_t SWEEP_ONE_THREADS = 512;   // with one CTA an SM
 
 // Sections of an expression: their values take 512 bytes (FP8 576) of shared
 // memory each.  (With at most 32, one warp folded all 512 sources of {64, 8}.)

@@ -1229,7 +1229,7 @@ hiccl_status_t hiccl_start(hiccl_comm_t c, void *stream) {
     t.timeout_ns = c->timeout_ns;
     if (d->sweep) {
       for (size_t i = 0; i < d->sweeps.size(); ++i) {
-        const cudaError_t e = sweep_launch(c->plan.sweep.launches[i], d->sweeps[i], c->ctas_per_sm == 1, s);
+        const cudaError_t e = sweep_launch(c->plan.sweep.launches[i], d->sweeps[i], c->ctas_per_sm == 1 ? d->nsm : 0, s);
         if (e != cudaSuccess) {
           cudaGetLastError();
           return cuda_fail(c, e, "sweep launch");

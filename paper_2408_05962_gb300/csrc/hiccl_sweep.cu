@@ -26,6 +26,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "hiccl_device.cuh"
@@ -523,12 +524,27 @@ __device__ __forceinline__ void copy_member(const Unit &u, int lane) {
     copy_unit<2, 1>(u.P, u.d0, u.d1, edge_of<2>(k, b, lane), k.nbytes);
 }
 
-// V vectors a lane in flight, stored to a group of destinations
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_COPY], 8) sweep_copy_kernel(const __grid_constant__ SweepArgs A) {
-  launch_order();
+// The units of a warp: one, in a grid that has a warp for each; or (WALK) every
+// so many, in a grid of one CTA an SM.
+template <bool WALK, typename F>
+__device__ __forceinline__ void each_unit(const SweepArgs &A, F body) {
   const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (unit >= A.units) return;
-  copy_member(find_unit(A, unit), threadIdx.x & 31);
+  if constexpr (WALK) {
+    const uint32_t step = gridDim.x * (blockDim.x >> 5);
+#pragma unroll 1
+    for (unsigned long long i = unit; i < A.units; i += step) body((uint32_t)i);
+  } else {
+    if (unit < A.units) body(unit);
+  }
+}
+// ONE: the kernel for one CTA an SM
+#define SWEEP_BOUNDS(kern, ctas) __launch_bounds__(ONE ? SWEEP_ONE_THREADS : SWEEP_THREADS[kern], ONE ? 1 : ctas)
+
+// V vectors a lane in flight, stored to a group of destinations
+template <bool ONE>
+__global__ void SWEEP_BOUNDS(SWEEP_COPY, 8) sweep_copy_kernel(const __grid_constant__ SweepArgs A) {
+  launch_order();
+  each_unit<ONE>(A, [&](uint32_t unit) { copy_member(find_unit(A, unit), threadIdx.x & 31); });
 }
 
 template <int G>
@@ -554,15 +570,16 @@ __device__ __forceinline__ void fold_member(const SweepArgs &A, const Unit &u, i
     else fold_any<4, 1, 8>(A, k, u.P, edge_of<4>(k, b, lane), k.nbytes, words, 4 * threads);
   }
 }
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FOLD], 16) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
+template <bool ONE>
+__global__ void SWEEP_BOUNDS(SWEEP_FOLD, 16) sweep_fold_kernel(const __grid_constant__ SweepArgs A) {
   launch_order();
-  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (unit >= A.units) return;
-  const Unit u = find_unit(A, unit);
-  if (u.k.nsrc == 1) copy_member(u, lane);
-  else if (A.groups == FOLD_GROUPS) fold_member<FOLD_GROUPS>(A, u, lane);
-  else fold_member<FOLD_GROUPS_SHORT>(A, u, lane);
+  each_unit<false>(A, [&](uint32_t unit) {
+    const int lane = threadIdx.x & 31;
+    const Unit u = find_unit(A, unit);
+    if (u.k.nsrc == 1) copy_member(u, lane);
+    else if (A.groups == FOLD_GROUPS) fold_member<FOLD_GROUPS>(A, u, lane);
+    else fold_member<FOLD_GROUPS_SHORT>(A, u, lane);
+  });
 }
 
 constexpr uint32_t TEAM_STATIC = 32;   // sections whose values lie in static shared memory
@@ -644,18 +661,16 @@ __device__ __forceinline__ void narrow_unit(const SweepArgs &A, const SweepClass
   else if (v == 2) fold_any<W, 2, 8>(A, k, P, off, k.nbytes, stack, blockDim.x);
   else fold_any<W, 1, 16>(A, k, P, off, k.nbytes, stack, blockDim.x);
 }
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_NARROW], 10) sweep_narrow_kernel(const __grid_constant__ SweepArgs A) {
+template <bool ONE>
+__global__ void SWEEP_BOUNDS(SWEEP_NARROW, 10) sweep_narrow_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ uint32_t saved[];
   launch_order();
-  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (unit >= A.units) return;
-  const Unit u = find_unit(A, unit);
-  const SweepClass &k = u.k;
-  const unsigned long long *P = u.P;
-  const uint32_t part = u.part;
-  if (sweep_lw(k.meta) == 2) narrow_unit<4>(A, k, P, part, lane, saved + threadIdx.x);
-  else narrow_unit<2>(A, k, P, part, lane, saved + threadIdx.x);
+  each_unit<false>(A, [&](uint32_t unit) {
+    const int lane = threadIdx.x & 31;
+    const Unit u = find_unit(A, unit);
+    if (sweep_lw(u.k.meta) == 2) narrow_unit<4>(A, u.k, u.P, u.part, lane, saved + threadIdx.x);
+    else narrow_unit<2>(A, u.k, u.P, u.part, lane, saved + threadIdx.x);
+  });
 }
 
 // Copies between operands that lie differently off a 16-byte boundary.  The
@@ -730,13 +745,14 @@ __device__ __forceinline__ void shift_unit(const Unit &u, int lane) {
       *reinterpret_cast<unsigned short *>(dst + at) = ev;
   }
 }
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_SHIFT], 8) sweep_shift_kernel(const __grid_constant__ SweepArgs A) {
+template <bool ONE>
+__global__ void SWEEP_BOUNDS(SWEEP_SHIFT, 8) sweep_shift_kernel(const __grid_constant__ SweepArgs A) {
   launch_order();
-  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (unit >= A.units) return;
-  const Unit u = find_unit(A, unit);
-  if (sweep_v(u.k.meta) == 4) shift_unit<4>(u, threadIdx.x & 31);
-  else shift_unit<1>(u, threadIdx.x & 31);
+  each_unit<ONE>(A, [&](uint32_t unit) {
+    const Unit u = find_unit(A, unit);
+    if (sweep_v(u.k.meta) == 4) shift_unit<4>(u, threadIdx.x & 31);
+    else shift_unit<1>(u, threadIdx.x & 31);
+  });
 }
 
 // ---- FP8 blocks --------------------------------------------------------------------
@@ -938,23 +954,25 @@ __device__ __forceinline__ void fp8_ring_at(Fp8Ring &r, const Unit &u, char *bas
   r.on2 = lane < 4 && r.off + 512 < u.k.nbytes;
 }
 
-__global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8], 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
+template <bool ONE>
+__global__ void SWEEP_BOUNDS(SWEEP_FP8, 6) sweep_fp8_kernel(const __grid_constant__ SweepArgs A) {
   extern __shared__ __align__(16) uint32_t saved[];
   launch_order();
-  const uint32_t unit = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (unit >= A.units) return;
-  const Unit u = find_unit(A, unit);
-  char *base = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (FP8_SLOTS * FP8_STEP);
-  ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + (blockDim.x >> 5) * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
-  Fp8Ring ring;
-  fp8_ring_at(ring, u, base);
-  ring.start(u.P, u.k.nsrc);
-  unsigned long long acc[8];
-  fp8_fold([&](uint32_t q) { return ring.next(q); }, A.toks + u.k.tok, u.k.nsrc, A.minus0, stack, blockDim.x, acc);
-  const Fp8Raw r = fp8_encode(acc);
-  ring.drain();
-  fp8_write(const_cast<char *>(ring.mine), r);
-  fp8_store(u, ring, base, 0, 1);
+  each_unit<ONE>(A, [&](uint32_t unit) {
+    const Unit u = find_unit(A, unit);
+    char *base = reinterpret_cast<char *>(saved) + (threadIdx.x >> 5) * (FP8_SLOTS * FP8_STEP);
+    ulonglong2 *stack = reinterpret_cast<ulonglong2 *>(saved) + (blockDim.x >> 5) * (FP8_SLOTS * FP8_STEP / 16) + threadIdx.x;
+    Fp8Ring ring;
+    fp8_ring_at(ring, u, base);
+    ring.start(u.P, u.k.nsrc);
+    unsigned long long acc[8];
+    fp8_fold([&](uint32_t q) { return ring.next(q); }, A.toks + u.k.tok, u.k.nsrc, A.minus0, stack, blockDim.x, acc);
+    const Fp8Raw r = fp8_encode(acc);
+    ring.drain();
+    fp8_write(const_cast<char *>(ring.mine), r);
+    fp8_store(u, ring, base, 0, 1);
+    if constexpr (ONE) __syncwarp();   // slot 0 has been read
+  });
 }
 
 // a short pass: a CTA to a unit, as sweep_team_kernel
@@ -992,11 +1010,17 @@ __global__ void __launch_bounds__(SWEEP_THREADS[SWEEP_FP8_TEAM], 2)
 }
 
 typedef void (*Kernel)(const SweepArgs);
-const Kernel KERNELS[SWEEP_KERNELS] = {sweep_copy_kernel, sweep_fold_kernel, sweep_fp8_kernel, sweep_narrow_kernel,
-                                         sweep_shift_kernel, sweep_team_kernel<false>, sweep_fp8_team_kernel<false>};
-Kernel kernel_of(const SweepLaunch &L) {
-  if (L.sections <= TEAM_STATIC) return KERNELS[L.kernel];
-  return L.kernel == SWEEP_FP8_TEAM ? sweep_fp8_team_kernel<true> : sweep_team_kernel<true>;
+template <bool ONE>
+Kernel kernel_of(uint32_t kernel, bool many) {
+  switch (kernel) {
+    case SWEEP_COPY: return sweep_copy_kernel<ONE>;
+    case SWEEP_FOLD: return sweep_fold_kernel<ONE>;
+    case SWEEP_FP8: return sweep_fp8_kernel<ONE>;
+    case SWEEP_NARROW: return sweep_narrow_kernel<ONE>;
+    case SWEEP_SHIFT: return sweep_shift_kernel<ONE>;
+    case SWEEP_TEAM: return many ? sweep_team_kernel<true> : sweep_team_kernel<false>;
+    default: return many ? sweep_fp8_team_kernel<true> : sweep_fp8_team_kernel<false>;
+  }
 }
 
 }  // namespace
@@ -1009,31 +1033,41 @@ constexpr size_t SWEEP_MAX_SMEM = SWEEP_MAX_DEPTH * 16 * 4 * 256 + 8 * FP8_SLOTS
 static_assert(SWEEP_MANY_SMEM <= 227 * 1024, "a CTA's shared memory");
 
 cudaError_t sweep_prepare() {
-  for (uint32_t i = 0; i < SWEEP_KERNELS; ++i) {
-    const cudaError_t e = cudaFuncSetAttribute(KERNELS[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_MAX_SMEM);
-    if (e != cudaSuccess) return e;
-  }
-  for (Kernel k : {Kernel(sweep_team_kernel<true>), Kernel(sweep_fp8_team_kernel<true>)}) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_MANY_SMEM);
-    if (e != cudaSuccess) return e;
-  }
+  for (uint32_t i = 0; i < SWEEP_KERNELS; ++i)
+    for (bool many : {false, true})
+      for (Kernel k : {kernel_of<false>(i, many), kernel_of<true>(i, many)}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   many && (i == SWEEP_TEAM || i == SWEEP_FP8_TEAM) ? SWEEP_MANY_SMEM : SWEEP_MAX_SMEM);
+        if (e != cudaSuccess) return e;
+      }
   return cudaSuccess;
 }
 
-cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_sm, cudaStream_t s) {
-  const unsigned warps = L.threads / 32;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(L.kernel == SWEEP_TEAM || L.kernel == SWEEP_FP8_TEAM ? L.units : (L.units + warps - 1) / warps);
-  cfg.blockDim = dim3(L.threads);
-  cfg.dynamicSmemBytes = (size_t)L.stack_words * 4 * L.threads;
-  if (L.kernel == SWEEP_FP8 || L.kernel == SWEEP_FP8_TEAM) cfg.dynamicSmemBytes += warps * FP8_SLOTS * FP8_STEP;
+cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, unsigned one_per_sm, cudaStream_t s) {
+  const bool team = L.kernel == SWEEP_TEAM || L.kernel == SWEEP_FP8_TEAM, fp8 = L.kernel == SWEEP_FP8 || L.kernel == SWEEP_FP8_TEAM;
+  // One CTA an SM: CTAs of up to 16 warps (the usual ones, one at a time: All-to-all
+  // of 64 ranks x 4 MiB 314 us, Reduce-scatter 254 us, 110 and 73 us step by step),
+  // copies and FP8 folds walking over their units in a single wave (91 us), the
+  // other folds in waves, as their registers do not suffice for the walk (53 us)
+  const bool one = one_per_sm && !team;
   SweepArgs B = A;
   B.sections = L.sections;
-  if (L.sections > TEAM_STATIC) cfg.dynamicSmemBytes += L.sections * (L.kernel == SWEEP_FP8_TEAM ? FP8_STEP : 512);
-  if (L.kernel == SWEEP_FOLD) {
-    B.groups = L.units < SHORT_UNITS ? FOLD_GROUPS_SHORT : FOLD_GROUPS;
-    cfg.dynamicSmemBytes += warps * B.groups * RING_GROUP * 512;
+  if (L.kernel == SWEEP_FOLD) B.groups = !one && L.units < SHORT_UNITS ? FOLD_GROUPS_SHORT : FOLD_GROUPS;
+  size_t per_warp = (size_t)L.stack_words * 4 * 32;
+  if (L.kernel == SWEEP_FOLD) per_warp += B.groups * RING_GROUP * 512;
+  if (fp8) per_warp += FP8_SLOTS * FP8_STEP;
+  unsigned warps = L.threads / 32;
+  if (one) {
+    warps = std::min(SWEEP_ONE_THREADS / 32, std::max(1u, (L.units + one_per_sm - 1) / one_per_sm));
+    while (warps > 1 && warps * per_warp > SWEEP_MAX_SMEM) --warps;
   }
+  unsigned grid = team ? L.units : (L.units + warps - 1) / warps;
+  if (one && L.kernel != SWEEP_FOLD && L.kernel != SWEEP_NARROW) grid = std::min(grid, one_per_sm);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(warps * 32);
+  cfg.dynamicSmemBytes = warps * per_warp;
+  if (L.sections > TEAM_STATIC) cfg.dynamicSmemBytes += L.sections * (fp8 ? FP8_STEP : 512);
   if (one_per_sm && cfg.dynamicSmemBytes < SWEEP_HALF_SM) cfg.dynamicSmemBytes = SWEEP_HALF_SM;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -1041,7 +1075,8 @@ cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel_of(L), B);
+  const bool many = L.sections > TEAM_STATIC;
+  return cudaLaunchKernelEx(&cfg, one ? kernel_of<true>(L.kernel, many) : kernel_of<false>(L.kernel, many), B);
 }
 
 }  // namespace hiccl

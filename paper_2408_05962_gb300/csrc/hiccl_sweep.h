@@ -22,7 +22,7 @@ struct SweepArgs {
 };
 
 cudaError_t sweep_prepare();            // once per device, with it current
-// one_per_sm: at most one CTA on an SM (CTAS_PER_SM = 1)
-cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, bool one_per_sm, cudaStream_t s);
+// one_per_sm: at most one CTA on an SM (CTAS_PER_SM = 1) of so many; 0: no limit
+cudaError_t sweep_launch(const SweepLaunch &L, const SweepArgs &A, unsigned one_per_sm, cudaStream_t s);
 
 }  // namespace hiccl
