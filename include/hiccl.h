@@ -186,7 +186,7 @@ typedef struct {
   int threads;                    /* HICCL_OPT_THREADS value                     */
   unsigned long long item_bytes;  /* HICCL_OPT_ITEM_BYTES value                  */
   float us;                       /* median time of one start, microseconds      */
-  int trials;                     /* configurations timed                        */
+  int trials;                     /* configurations covered                      */
 } hiccl_tune_t;
 
 /* Pick the fastest configuration of an initialized communicator by timing it
@@ -197,6 +197,8 @@ typedef struct {
  * paper's optimization parameters (Sec. 4.1), with the executor defaults;
  * with a ring (HICCL_OPT_RING > 1) only stripes up to the node size.  None of
  * these changes a result bit; the ring, which does, is not tuned.
+ * Starts that run a sweep do not depend on any of them: one timing then covers
+ * all candidates and the communicator keeps its configuration.
  * The communicator ends up initialized with the best configuration, which
  * *best receives (may be NULL).  The trials execute the collective: receive
  * buffers are overwritten.  Blocking. */

@@ -1302,17 +1302,11 @@ hiccl_status_t hiccl_autotune(hiccl_comm_t c, void *stream, int flags, hiccl_tun
     hiccl_tune_t top = cur;
     top.us = 3.4e38f;
     int trials = 0;
-    // time one configuration; the communicator is left initialized with it
-    auto trial = [&](const hiccl_tune_t &k, float &us) -> hiccl_status_t {
-      c->order = k.order;
-      c->item_bytes = k.item_bytes;
-      c->threads = k.threads;
-      hiccl_status_t st = replan(c, h, k.stripe, k.pipeline);
-      if (st != HICCL_OK) return st;
-      if ((st = dev_upload(c)) != HICCL_OK) return st;
-      c->state = hiccl_comm::READY;
+    // median of three starts after a warm-up
+    auto measure = [&](float &us) -> hiccl_status_t {
       float ts[4];
       for (int r = 0; r < 4; ++r) {
+        hiccl_status_t st;
         cudaEventRecord(e0, s);
         if ((st = hiccl_start(c, s)) != HICCL_OK) return st;
         cudaEventRecord(e1, s);
@@ -1322,10 +1316,31 @@ hiccl_status_t hiccl_autotune(hiccl_comm_t c, void *stream, int flags, hiccl_tun
       }
       std::sort(ts + 1, ts + 4);   // run 0 is the warm-up
       us = ts[2] * 1000.f;
-      ++trials;
       return HICCL_OK;
     };
+    // A sweep is the same launches with every candidate: one timing serves them
+    // all, and the communicator stays as it is.  (Timed one by one, some twenty
+    // plans and uploads, the noise chose the stripe, and with it the schedule's
+    // byte counts.)
+    const bool swept = c->plan.sweep.valid && !c->trace;
+    // time one configuration; the communicator is left initialized with it
+    auto trial = [&](const hiccl_tune_t &k, float &us) -> hiccl_status_t {
+      c->order = k.order;
+      c->item_bytes = k.item_bytes;
+      c->threads = k.threads;
+      hiccl_status_t st = replan(c, h, k.stripe, k.pipeline);
+      if (st != HICCL_OK) return st;
+      if ((st = dev_upload(c)) != HICCL_OK) return st;
+      c->state = hiccl_comm::READY;
+      st = measure(us);
+      if (st == HICCL_OK) ++trials;
+      return st;
+    };
     auto consider = [&](hiccl_tune_t k) -> hiccl_status_t {
+      if (swept) {
+        ++trials;
+        return HICCL_OK;
+      }
       float us = 0.f;
       hiccl_status_t st = trial(k, us);
       if (st != HICCL_OK) return st;
@@ -1334,6 +1349,14 @@ hiccl_status_t hiccl_autotune(hiccl_comm_t c, void *stream, int flags, hiccl_tun
       return HICCL_OK;
     };
     hiccl_status_t st = HICCL_OK;
+    if (swept) {
+      if (!c->dev->sweep) {   // (hiccl_debug_withhold had it run step by step)
+        st = dev_upload(c);
+        if (st == HICCL_OK) c->state = hiccl_comm::READY;
+      }
+      top = cur;
+      if (st == HICCL_OK) st = measure(top.us);
+    }
     if (flags & 1) {   // the paper's stripe and pipeline parameters first
       std::vector<int> ss{cur.stripe, 1};
       if (!h.empty() && h.back() > 1 && h.back() <= c->P) ss.push_back(h.back());
@@ -1359,7 +1382,7 @@ hiccl_status_t hiccl_autotune(hiccl_comm_t c, void *stream, int flags, hiccl_tun
         k.item_bytes = ib;
         if (st == HICCL_OK && !(order == base.order && ib == base.item_bytes)) st = consider(k);
       }
-    if (st == HICCL_OK) {
+    if (st == HICCL_OK && !swept) {
       float us = 0.f;
       st = trial(top, us);   // leave the communicator on the best configuration
     }
