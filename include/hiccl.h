@@ -273,6 +273,12 @@ typedef struct {
  * buffers and only its operand table. */
 hiccl_status_t hiccl_plan_info(hiccl_comm_t comm, hiccl_plan_info_t *out);
 
+/* Device memory that hiccl_init (of a group: hiccl_group) allocates for the
+ * plan with the present TRACE option, in blocks of 512 bytes: a sweep's operand
+ * table, or the step table, counters, relay buffers and trace.  Valid after
+ * hiccl_init or hiccl_plan; HICCL_ERR_STATE without a plan. */
+hiccl_status_t hiccl_device_bytes(hiccl_comm_t comm, unsigned long long *bytes);
+
 /* One step of the plan, for inspection and host-side checking.
  *   kind: 0 copy, 1 reduce.  level: hierarchy level crossed, -1 local.
  *   op: the reduce's hiccl_op_t (0 for copies).

@@ -2,6 +2,7 @@
 // the device runtime (hiccl_runtime.cu).  Not part of the public ABI.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <new>
 #include <string>
@@ -271,6 +272,12 @@ struct Sweep {
   std::vector<SweepLaunch> launches;
   uint32_t depth = 0;                         // saved values of the deepest expression
 };
+
+// bytes of its tables on the device
+inline size_t sweep_bytes(const Sweep &w) {
+  return std::max<size_t>(w.classes.size() * sizeof(SweepClass) + w.ptrs.size() * 8 + (w.toks.size() + w.hints.size()) * 4, 16);
+}
+constexpr size_t TRACE_BYTES = 6 * sizeof(unsigned long long);   // of a work item
 
 struct Loc {
   unsigned long long addr;   // device address, or relay-arena offset when scratch

@@ -1878,6 +1878,28 @@ hiccl_status_t hiccl_plan_info(hiccl_comm_t c, hiccl_plan_info_t *out) {
   });
 }
 
+hiccl_status_t hiccl_device_bytes(hiccl_comm_t c, unsigned long long *out) {
+  return guarded(c, [&]() -> hiccl_status_t {
+    if (!c || !out) return HICCL_ERR_INVALID;
+    *out = 0;
+    if (!c->plan.valid) return fail(c, HICCL_ERR_STATE, "no plan");
+    const Plan &p = c->plan;
+    auto blocks = [](unsigned long long n) { return (n + 511) & ~511ull; };   // as the allocator gives them out
+    if (p.sweep.valid && !c->trace) {
+      *out = blocks(sweep_bytes(p.sweep));
+      return HICCL_OK;
+    }
+    const size_t N = p.steps.size(), NI = p.item_off.size() - 1;
+    unsigned long long table = 0;   // its arrays start at multiples of 256 bytes
+    for (unsigned long long n : {record_bytes(p), (unsigned long long)(NI * sizeof(DevItem)), N * 4ull, (N + 1) * 4ull,
+                                 p.succ.size() * 4ull, p.locs.size() * 8ull})
+      table += (n + 255) & ~255ull;
+    *out = blocks(table) + blocks(N * 16 + sizeof(DevCtl)) + blocks(p.scratch_bytes);
+    if (c->trace) *out += blocks(NI * TRACE_BYTES);
+    return HICCL_OK;
+  });
+}
+
 hiccl_status_t hiccl_get_step(hiccl_comm_t c, unsigned long long index, hiccl_step_desc_t *d,
                               unsigned long long *src_addr, int *src_scratch, int *src_rank,
                               unsigned long long *dst_addr, int *dst_scratch, int *dst_rank,

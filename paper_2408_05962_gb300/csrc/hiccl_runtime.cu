@@ -1072,7 +1072,7 @@ static hiccl_status_t upload_sweep(hiccl_comm *c) {
   DevState *d = c->dev;
   const size_t cb = w.classes.size() * sizeof(SweepClass), pb = w.ptrs.size() * 8, tb = w.toks.size() * 4,
                hb = w.hints.size() * 4;
-  std::vector<char> img(std::max<size_t>(cb + pb + tb + hb, 16));
+  std::vector<char> img(sweep_bytes(w));
   if (cb) std::memcpy(img.data(), w.classes.data(), cb);
   if (pb) std::memcpy(img.data() + cb, w.ptrs.data(), pb);
   if (tb) std::memcpy(img.data() + cb + pb, w.toks.data(), tb);
@@ -1196,7 +1196,7 @@ static hiccl_status_t upload_steps(hiccl_comm *c) {
   t.seg = p.seg;
   t.trace = nullptr;
   if (c->trace && t.nitems) {
-    hiccl_status_t st = dalloc((void **)&d->trace, t.nitems * 6 * sizeof(unsigned long long), "trace buffer");
+    hiccl_status_t st = dalloc((void **)&d->trace, t.nitems * TRACE_BYTES, "trace buffer");
     if (st != HICCL_OK) return st;
     t.trace = d->trace;
   }

@@ -109,6 +109,7 @@ _SIGS = {
     "hiccl_debug_sweep": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t,
                                          ctypes.POINTER(ctypes.c_size_t)]),
     "hiccl_plan_info": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(PlanInfo)]),
+    "hiccl_device_bytes": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_ulonglong)]),
     "hiccl_get_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_ulonglong, ctypes.POINTER(StepDesc),
                                       ctypes.POINTER(ctypes.c_ulonglong), ctypes.POINTER(ctypes.c_int),
                                       ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_ulonglong),
@@ -270,6 +271,12 @@ def hiccl_plan_info(comm) -> dict:
     info = PlanInfo()
     _check(comm, lib().hiccl_plan_info(comm, ctypes.byref(info)))
     return info.as_dict()
+
+
+def hiccl_device_bytes(comm) -> int:
+    n = ctypes.c_ulonglong(0)
+    _check(comm, lib().hiccl_device_bytes(comm, ctypes.byref(n)))
+    return n.value
 
 
 def hiccl_debug_image(comm):
@@ -443,6 +450,9 @@ class Comm:
 
     def plan_info(self):
         return hiccl_plan_info(self.handle)
+
+    def device_bytes(self):
+        return hiccl_device_bytes(self.handle)
 
     def image(self):
         return hiccl_debug_image(self.handle)

@@ -13,7 +13,7 @@ payload) arrive at any time.  The server
   short requests to drain, and a large request is never starved by later
   small ones;
 * memoizes plans (Sec. 5.2: a schedule is optimized once and reused): a
-  finished request leaves its communicator -- step table, counters, relay
+  finished request leaves its communicator -- its tables, counters, relay
   buffers -- and its arena buffers resident, keyed by the request's shape; a
   later request of the same shape takes them over with no factorization, no
   upload and no allocation.  Idle entries are evicted, least recently used
@@ -21,9 +21,9 @@ payload) arrive at any time.  The server
   makes room: a request that waits for memory held by running requests
   leaves the idle plans in place;
 * plans the other admitted requests on a pool of host threads (the native
-  factorizer), counts each plan's device footprint (table, counters, relay
-  buffers) against the budget together with the buffers, then uploads it on
-  the pool;
+  factorizer), counts each plan's device footprint (a sweep's operand table,
+  or table, counters and relay buffers) against the budget together with the
+  buffers, then uploads it on the pool;
 * launches planned requests on whichever of its ``slots`` CUDA streams is
   free -- each request alone (``group_max`` 1), or up to ``group_max``
   waiting requests together as one grouped persistent launch
@@ -374,8 +374,7 @@ class Server:
         comm.plan(req.hierarchy, 1, 1)
         rd, wr = comm.hbm_bytes()
         req.hbm_bytes = rd + wr
-        info = comm.plan_info()
-        req.dev_bytes = info["table_bytes"] + info["scratch_bytes"]
+        req.dev_bytes = comm.device_bytes()
 
     @staticmethod
     def _upload(req: Request):
@@ -436,8 +435,7 @@ class Server:
     def _build_group(batch):
         """Combined table of a batch (pool thread): plan union and upload."""
         grp = H.Comm.group([r.comm for r in batch])
-        info = grp.plan_info()
-        return grp, info["table_bytes"] + info["scratch_bytes"]
+        return grp, grp.device_bytes()
 
     def _start_on(self, sl, grp, batch, gb):
         """Launch ``grp`` on slot ``sl``; ``gb``: device bytes of a combined

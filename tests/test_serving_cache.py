@@ -138,3 +138,30 @@ def test_planned_request_waits_for_memory_held_by_others():
     srv._finish(srv.ready.popleft(), time.perf_counter())   # b done; its plan is kept idle
     srv._reserve_uploads()                               # evicting b's idle plan makes room for a
     assert [r for _, r in srv.uploading] == [a] and not a.error
+
+
+def test_footprints_are_what_init_allocates():
+    """A swept plan counts its operand table and no step table or relays, so a
+    request whose relays would not fit is served; a traced one, which runs step
+    by step, counts them and its trace."""
+    shape = dict(kind="allreduce", P=16, hierarchy=[4, 4], bytes_per_rank=16 * 4096 * 4, dtype="f32")
+    seen = {}
+    for trace in (0, 1):
+        srv = Server(64 << 20, slots=1, device="cpu", comm_options={H.OPT_TRACE: trace})
+        srv.pool = _Pool()
+        r = Request(**shape)
+        srv.submit(r)
+        with srv.lock:
+            srv._admit()
+        srv.planning = srv._collect(srv.planning, srv.to_upload.append)
+        info = r.comm.plan_info()
+        steps = info["table_bytes"] + info["scratch_bytes"] + 48 * info["items"]
+        blob = r.comm.sweep()
+        sweep = len(blob) - 40 - 32 * int.from_bytes(blob[8:16], "little")   # without the counts and the launches
+        seen[trace] = r.dev_bytes
+        # allocations take whole blocks of 512 bytes (the step table is four, its arrays start at 256)
+        assert 0 <= r.dev_bytes - (steps if trace else sweep) < (4 * 512 + 6 * 256 if trace else 512) and r.dev_bytes % 512 == 0
+        srv.budget = srv.arena.used + seen[0]                # room for the operand table only
+        srv._reserve_uploads()
+        assert bool(r.error) == bool(trace) and [q for _, q in srv.uploading] == ([] if trace else [r])
+    assert seen[1] > 50 * seen[0]
