@@ -290,8 +290,8 @@ def measured_peak():
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("hiccl_sweep.cu", "hiccl_sweep.cpp", "hiccl_sweep.h", "hiccl_device.cuh", "hiccl_runtime.cu",
-              "hiccl_internal.h"):
+    for f in ("hiccl_sweep.cu", "hiccl_sweep_kernels.cuh", "hiccl_sweep_rare.cu", "hiccl_sweep.cpp", "hiccl_sweep.h",
+              "hiccl_device.cuh", "hiccl_runtime.cu", "hiccl_internal.h"):
         with open(os.path.join(ROOT, "paper_2408_05962_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -1,6 +1,6 @@
-// Device arithmetic shared by the step executor (hiccl_runtime.cu) and the
-// sweep kernels (hiccl_sweep.cu): the payloads' combine operators and the
-// BF16 / FP8 conversions.
+// Device arithmetic: the BF16 / FP8 conversions of the step executor
+// (hiccl_runtime.cu) and the sweep kernels (hiccl_sweep_kernels.cuh), and the executor's
+// combine operators (the sweeps combine many sources at a time with their own).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -157,6 +157,7 @@ enum : uint32_t { ERR_TIMEOUT = 1, ERR_BADSTEP = 2, ERR_STALL = 3 };
 // the schedule's steps would round them) and no relay is written or read, so
 // a pass moves each input and each output once.  Members of equal shape form
 // a class; a class is cut into warp-sized units.
+constexpr uint32_t SWEEP_SMS = 152;        // of a GB300 (plans are made without a device too)
 constexpr uint32_t SWEEP_MAX_DEPTH = 6;    // partial values held while an inner group is folded
 constexpr uint32_t SWEEP_PREFIX = 96;      // classes of a launch searched in the parameter bank
 constexpr uint32_t SWEEP_INLINE = 4;       // classes of a launch passed as arguments
@@ -186,13 +187,14 @@ constexpr uint32_t SWEEP_ONE_THREADS = 512;   // with one CTA an SM
 // Sections of an expression: their values take 512 bytes (FP8 576) of shared
 // memory each.  (With at most 32, one warp folded all 512 sources of {64, 8}.)
 constexpr uint32_t SWEEP_TEAM_MAX = 128;
+constexpr uint32_t SWEEP_TEAM_STATIC = 32;   // whose values lie in static shared memory
 // In a fold pass of few units every warp folds one source after the other,
 // about 300 cycles each, while most of an SM idles: below eight units an SM
 // the sections go to the warps of a CTA, as many as fill the SMs
 // (SWEEP_TEAM_WARPS in all).  Measured without / with, All-reduce of 64 ranks
 // x 64 KiB 12.7 / 9.4 us, Reduce of 64 ranks x 16 KiB 10.8 / 6.1 us; at 1024
 // units (16 ranks x 512 KiB) 7.3 / 5.2 us, at 2048 (1 MiB) 8.6 / 10.6 us.
-constexpr uint32_t SWEEP_TEAM_UNITS = 152 * 8, SWEEP_TEAM_WARPS = 152 * 32;
+constexpr uint32_t SWEEP_TEAM_UNITS = SWEEP_SMS * 8, SWEEP_TEAM_WARPS = SWEEP_SMS * 32;
 // More than 32 sections: every warp evaluates the expression of all their values,
 // so the lines lie earlier.  Reduce, F32, by one warp / by 64 sections of {64, 8}
 // (us): 2 units 67 / 14, 128 units 67 / 16, 512 76 / 39; 128 of {128, 8}: 132 / 25,
@@ -200,7 +202,7 @@ constexpr uint32_t SWEEP_TEAM_UNITS = 152 * 8, SWEEP_TEAM_WARPS = 152 * 32;
 // Where a level has fewer sections, by 2 or 64 of {2, 32, 4}: 1 unit 32 / 12, 128
 // 32 / 14; by 4 or 64 of {4, 16, 4}: 512 units 22 / 23.  FP8 values take as long to
 // fold as sources, so there fewer stay better: {4, 16, 4}, 128 units, 22.5 / 27.7.
-constexpr uint32_t SWEEP_TEAM_MANY = 152 * 3, SWEEP_TEAM_FEW = 152 * 2;
+constexpr uint32_t SWEEP_TEAM_MANY = SWEEP_SMS * 3, SWEEP_TEAM_FEW = SWEEP_SMS * 2;
 
 // token of one source, in evaluation order: START the accumulator with it
 // (first saving the old one when PUSH is set), else combine it; then up to
@@ -432,6 +434,8 @@ hiccl_status_t replan(hiccl_comm *c, const std::vector<int> &hierarchy, int stri
 // runtime entry points (hiccl_runtime.cu)
 hiccl_status_t dev_upload(hiccl_comm *c);
 void dev_release(hiccl_comm *c);
+// after a change of CTAS_PER_SM
+hiccl_status_t dev_options(hiccl_comm *c);
 // CTAs of an executor launch of c on the calling thread's current device
 // (SMs x resident CTAs per SM for c's THREADS and CTAS_PER_SM); 0 when no
 // device can be queried

@@ -1951,7 +1951,7 @@ hiccl_status_t hiccl_set_option(hiccl_comm_t c, hiccl_option_t opt, long long va
       case HICCL_OPT_CTAS_PER_SM:
         if (value < 1 || value > 32) return fail(c, HICCL_ERR_INVALID, "ctas per SM must be in [1, 32]");
         c->ctas_per_sm = (int)value;
-        return HICCL_OK;
+        return dev_options(c);
       case HICCL_OPT_THREADS:
         if (value != 128 && value != 256 && value != 512)
           return fail(c, HICCL_ERR_INVALID, "threads per CTA must be 128, 256 or 512");

@@ -977,6 +977,10 @@ struct DeviceRes {
   cudaStream_t upload = nullptr;
   int nsm = 0;
   int occ[4] = {0, 0, 0, 0};
+  struct Kernel {   // of a sweep's launch
+    std::once_flag once;
+    cudaError_t status = cudaSuccess;
+  } sweeps[SWEEP_KERNEL_FORMS];
 };
 static DeviceRes g_dev[MAXDEV];
 
@@ -987,7 +991,6 @@ static cudaError_t device_res(int dev, DeviceRes **out) {
     cudaError_t e = cudaStreamCreateWithFlags(&r.upload, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r.nsm, cudaDevAttrMultiProcessorCount, dev);
     for (int i = 1; i < 4 && e == cudaSuccess; ++i) e = exec_occupancy(64 << i, &r.occ[i]);
-    if (e == cudaSuccess) e = sweep_prepare();
     r.status = e;
   });
   *out = &r;
@@ -1058,6 +1061,27 @@ void dev_release(hiccl_comm *c) {
   c->dev = nullptr;
 }
 
+// the sweep kernels that c's starts may launch
+static hiccl_status_t sweep_kernels(hiccl_comm *c) {
+  const int dev = c->dev->device;
+  for (const SweepLaunch &L : c->plan.sweep.launches)
+    for (bool one : {false, true}) {
+      if (one && c->ctas_per_sm != 1) continue;
+      DeviceRes::Kernel &k = g_dev[dev].sweeps[sweep_kernel_index(L, one)];
+      std::call_once(k.once, [&]() {
+        int cur = dev;
+        k.status = cudaGetDevice(&cur);
+        if (k.status == cudaSuccess && cur != dev) k.status = cudaSetDevice(dev);
+        if (k.status == cudaSuccess) k.status = sweep_prepare(L, one);
+        if (cur != dev) cudaSetDevice(cur);
+      });
+      if (k.status != cudaSuccess) return cuda_fail(c, k.status, "sweep kernel");
+    }
+  return HICCL_OK;
+}
+
+hiccl_status_t dev_options(hiccl_comm *c) { return c->dev && c->dev->sweep ? sweep_kernels(c) : HICCL_OK; }
+
 static hiccl_status_t dev_alloc(hiccl_comm *c, void **ptr, size_t bytes, const char *what) {
   const cudaError_t e = cudaMallocAsync(ptr, bytes, c->dev->upload);
   if (e == cudaSuccess) return HICCL_OK;
@@ -1077,7 +1101,8 @@ static hiccl_status_t upload_sweep(hiccl_comm *c) {
   if (pb) std::memcpy(img.data() + cb, w.ptrs.data(), pb);
   if (tb) std::memcpy(img.data() + cb + pb, w.toks.data(), tb);
   if (hb) std::memcpy(img.data() + cb + pb + tb, w.hints.data(), hb);
-  const hiccl_status_t st = dev_alloc(c, &d->sweep_table, img.size(), "sweep table");
+  hiccl_status_t st = sweep_kernels(c);
+  if (st == HICCL_OK) st = dev_alloc(c, &d->sweep_table, img.size(), "sweep table");
   if (st != HICCL_OK) return st;
   cudaError_t e = cudaMemcpyAsync(d->sweep_table, img.data(), img.size(), cudaMemcpyHostToDevice, d->upload);
   if (e != cudaSuccess) return cuda_fail(c, e, "upload sweep table");

@@ -276,8 +276,9 @@ void plan_launches(Sweep &sw) {
       SweepClass &k = sw.classes[i];
       const uint32_t dt = sweep_dtype(k.meta), lw = sweep_lw(k.meta);
       uint32_t v = 1;
-      if (kern == SWEEP_SHIFT) v = rows >= 4 * 2432 ? 4 : 1;
-      else if (kern == SWEEP_NARROW) v = rows >= 8 * 2432 ? 8 : rows >= 2 * 2432 ? 2 : 1;
+      constexpr uint32_t WARPS = SWEEP_SMS * 16;   // that keep every SM busy
+      if (kern == SWEEP_SHIFT) v = rows >= 4 * WARPS ? 4 : 1;
+      else if (kern == SWEEP_NARROW) v = rows >= 8 * WARPS ? 8 : rows >= 2 * WARPS ? 2 : 1;
       else if (k.nsrc == 1) v = rows >= 4096 ? 4 : rows >= 2048 ? 2 : 1;
       const unsigned long long unit = row_bytes(kern, k) * v;
       const unsigned long long upm = (k.nbytes + unit - 1) / unit;
@@ -304,7 +305,7 @@ void plan_launches(Sweep &sw) {
     // a short pass uses small CTAs, so that its units reach every SM
     uint32_t warps = most / 32;
     const bool team = kern == SWEEP_TEAM || kern == SWEEP_FP8_TEAM;
-    while (!team && warps > 1 && units < (unsigned long long)warps * 304) warps /= 2;
+    while (!team && warps > 1 && units < (unsigned long long)warps * (2 * SWEEP_SMS)) warps /= 2;
     // a team's warps: no more than sections, and enough for SWEEP_TEAM_WARPS in all
     uint32_t sections = 1;
     for (size_t i = a; team && i < z; ++i) sections = std::max(sections, sw.classes[i].team);

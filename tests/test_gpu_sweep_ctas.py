@@ -38,4 +38,17 @@ def test_one_cta_an_sm(kind, P, h, d, dtype, pad):
             c.wait()
         got.append(b.recv.clone())
     c.destroy()
+    c = H.Comm(P, dtype)                                   # limited from the start, and under capture
+    c.set_option(H.OPT_CTAS_PER_SM, 1)
+    c.add_collective(kind, d, b.send_ptrs(), b.recv_ptrs(), P - 1)
+    c.init(h, 1, 1)
+    b.recv.view(torch.uint8).fill_(0xa5)
+    s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=s):
+        c.start(s)
+    graph.replay()
+    torch.cuda.synchronize()
+    c.destroy()
+    assert torch.equal(got[0].view(torch.uint8), b.recv.view(torch.uint8))
     assert torch.equal(got[0].view(torch.uint8), got[1].view(torch.uint8))
