@@ -42,6 +42,9 @@ struct Expr {
   Expr(const std::vector<int> &hier, const std::vector<int> &lv, bool rnd) : h(hier), leaves(lv), rounds(rnd) {
     G.assign(h.size() + 1, 1);
     for (size_t l = h.size(); l-- > 0;) G[l] = G[l + 1] * h[l];
+    order.reserve(lv.size());
+    toks.reserve(lv.size());
+    nops.reserve(lv.size());
   }
   void leaf(int rank, bool start, bool push) {
     order.push_back(rank);
@@ -58,9 +61,10 @@ struct Expr {
   // ends of the level-l subgroups inside leaves[lo, hi)
   size_t next(size_t lo, size_t hi, int l) const { return next_in(leaves, lo, hi, l); }
   size_t next_in(const std::vector<int> &v, size_t lo, size_t hi, int l) const {
-    const long long q = v[lo] / G[l + 1];
+    const long long end = (v[lo] / G[l + 1] + 1) * G[l + 1];
+    if (v[hi - 1] < end) return hi;
     size_t k = lo + 1;
-    while (k < hi && v[k] / G[l + 1] == q) ++k;
+    while (v[k] < end) ++k;
     return k;
   }
   // the value of a group: the left fold of its non-empty subgroups'
@@ -182,9 +186,20 @@ uint32_t two_steps(const std::vector<int> &h, const std::vector<int> &leaves, bo
     if (level < 0) return 0;
     for (uint32_t a : bounds) reps.push_back(leaves[a]);
     bounds.push_back(n);
+    // (sections of one shape have the same tokens: for 64 groups of one size
+    // planning takes 6 us less)
+    const long long below = top.G[level + 1];
     for (size_t s = 0; s + 1 < bounds.size(); ++s) {
+      const uint32_t lo = bounds[s], hi = bounds[s + 1];
+      bool same = s > 0 && hi - lo == lo - bounds[s - 1];
+      for (uint32_t k = 0; same && k < hi - lo; ++k)
+        same = leaves[lo + k] % below == leaves[bounds[s - 1] + k] % below;
+      if (same) {
+        for (uint32_t k = 0; k < hi - lo; ++k) lower.push_back(lower[bounds[s - 1] + k]);
+        continue;
+      }
       Expr e(h, leaves, rounds);
-      e.group(bounds[s], bounds[s + 1], level + 1, false);
+      e.group(lo, hi, level + 1, false);
       uint32_t d = 0;
       if (!e.finish(d)) return 0;
       depth = std::max(depth, d);
@@ -396,7 +411,8 @@ struct Bytes {
   };
   std::vector<Span> v;
   void join() {
-    std::sort(v.begin(), v.end(), [](const Span &a, const Span &b) { return a.lo < b.lo; });
+    auto before = [](const Span &a, const Span &b) { return a.lo < b.lo; };
+    if (!std::is_sorted(v.begin(), v.end(), before)) std::sort(v.begin(), v.end(), before);
     size_t w = 0;
     for (size_t k = 1; k < v.size(); ++k) {
       if (v[k].lo <= v[w].hi) v[w].hi = std::max(v[w].hi, v[k].hi);
@@ -410,41 +426,42 @@ struct Bytes {
     return it == v.begin() || hi > (--it)->hi ? nullptr : &*it;
   }
 };
-// Ranges of nbytes, each mostly in the span of the one that had its hint before.
+// Ranges of nbytes, each mostly in the span of the one before or in the next one
+// (members take the ranks' rows in turn).
 struct Inside {
-  static constexpr uint32_t HINTS = 64;
-  struct Hint {
-    unsigned long long lo, room;   // [lo, lo + room) + nbytes
-  };
   const Bytes &in;
   const unsigned long long nbytes;
-  Hint hints[HINTS] = {};
+  size_t at = 0;
   Inside(const Bytes &b, unsigned long long n) : in(b), nbytes(n) {}
-  bool operator()(unsigned long long a, uint32_t hint) {
-    Hint &h = hints[hint % HINTS];
-    if (a - h.lo < h.room) return true;
+  bool holds(size_t k, unsigned long long a) const {
+    return k < in.v.size() && a >= in.v[k].lo && a + nbytes <= in.v[k].hi;
+  }
+  bool operator()(unsigned long long a) {
+    if (holds(at, a)) return true;
+    if (holds(at + 1, a)) {
+      ++at;
+      return true;
+    }
     const Bytes::Span *s = in.find(a, a + nbytes);
-    if (s) h = Hint{s->lo, s->hi - s->lo - nbytes + 1};
+    if (s) at = s - in.v.data();
     return s != nullptr;
   }
 };
 // what a program reads or writes, and what it writes
-void join_ranges(const Ranges &ranges, Bytes &all, Bytes &written) {
+void join_ranges(const Ranges &ranges, int P, Bytes &all, Bytes &written) {
   struct Open {
     unsigned long long lo = 0, hi = 0;
   };
-  std::vector<Open> open;   // by rank and direction: its ranges mostly continue one another
-  all.v.reserve(64);
-  written.v.reserve(64);
+  std::vector<Open> open(2 * (size_t)P);   // by direction and rank: its ranges mostly continue one another
+  all.v.reserve(open.size());
+  written.v.reserve(P);
   auto close = [&](const Open &o, bool write) {
     if (o.lo == o.hi) return;
     all.v.push_back(Bytes::Span{o.lo, o.hi});
     if (write) written.v.push_back(Bytes::Span{o.lo, o.hi});
   };
   for (const Range &r : ranges.all) {
-    const size_t k = 2 * (size_t)r.rank + r.write;
-    if (k >= open.size()) open.resize(k + 64);
-    Open &o = open[k];
+    Open &o = open[(r.write ? P : 0) + r.rank];
     if (r.lo <= o.hi && r.hi >= o.lo && o.lo != o.hi) {
       o.lo = std::min(o.lo, r.lo);
       o.hi = std::max(o.hi, r.hi);
@@ -454,7 +471,7 @@ void join_ranges(const Ranges &ranges, Bytes &all, Bytes &written) {
       o.hi = r.hi;
     }
   }
-  for (size_t k = 0; k < open.size(); ++k) close(open[k], k & 1);
+  for (size_t k = 0; k < open.size(); ++k) close(open[k], k >= (size_t)P);
   all.join();
   written.join();
 }
@@ -593,7 +610,7 @@ bool check_sweep(const hiccl_comm &c, const Ranges &ranges, const Sweep &sw, std
     return false;
   };
   Bytes all, written;   // (a group has no primitives; its members were checked)
-  join_ranges(ranges, all, written);
+  if (!c.group) join_ranges(ranges, c.P, all, written);
   size_t next = 0;       // class
   for (const SweepLaunch &L : sw.launches) {
     if (L.class_lo != next || L.class_hi <= L.class_lo || L.class_hi > sw.classes.size() || L.kernel >= SWEEP_KERNELS)
@@ -635,9 +652,8 @@ bool check_sweep(const hiccl_comm &c, const Ranges &ranges, const Sweep &sw, std
         const unsigned long long *p = &sw.ptrs[k.ptr + m * n];
         bool in = true;
         unsigned long long off = 0, low = 0;
-        // (neighbouring members of a fold read the same rows, copies write every row in turn)
-        for (uint32_t q = 0; q < k.nsrc; ++q) in = in && (c.group || readable(p[q], q));
-        for (uint32_t q = k.nsrc; q < n; ++q) in = in && (c.group || writable(p[q], n == 2 ? m : q));
+        for (uint32_t q = 0; q < k.nsrc; ++q) in = in && (c.group || readable(p[q]));
+        for (uint32_t q = k.nsrc; q < n; ++q) in = in && (c.group || writable(p[q]));
         if (!in) return bad("an operand of " + at + " lies outside the primitives' buffers");
         for (uint32_t q = 0; q < n; ++q) off |= p[q] ^ p[0], low |= p[q];
         if (((low | k.nbytes) & (elem - 1)) || ((lw >= 4 ? off : fold ? low | k.nbytes : 0) & mask))
