@@ -391,8 +391,11 @@ hiccl_status_t hiccl_debug_image(hiccl_comm_t comm, void *recs, size_t recs_capa
 
 /* Inspection: the sweep of a planned communicator -- the one pass that
  * hiccl_start runs when the program reduces to independent expressions, each
- * a copy or a nested fold over equal byte ranges (every collective of Table 2
- * does; TRACE and hiccl_debug_withhold select the step-by-step executor).
+ * a copy or a nested fold over equal byte ranges (the collectives of
+ * hiccl_collective_t do, over up to seven levels; of Table 2's compositions, All-gather as Gather and
+ * Broadcast and Reduce-scatter as Reduce and Scatter do not, as their second half
+ * reads or writes other ranges than the first; TRACE and hiccl_debug_withhold
+ * select the step-by-step executor).
  * `out` receives, without padding: the counts of classes, launches, operand
  * pointers, tokens and hints (u64 each); the classes (64 bytes: bytes per operand
  * u64, first pointer u64, then u32 first unit, units per member, members,

@@ -1,7 +1,8 @@
 """Build the in-tree C-ABI library ``_lib/libhiccl.so`` for sm_103a.
 
-Two translation units compiled in parallel -- the host factorizer (g++) and
-the device runtime (nvcc) -- then linked with nvcc (static CUDA runtime).
+Its translation units (host factorizer and sweeps, device runtime, sweep
+kernels in two modules) are compiled in parallel, then linked with nvcc (static
+CUDA runtime).
 Run ``python -m paper_2408_05962_gb300.build`` or call ``build()``.
 """
 from __future__ import annotations
